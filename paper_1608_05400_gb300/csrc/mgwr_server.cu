@@ -169,6 +169,28 @@ struct Ticket {
 
 bool pow2(long long x) { return x > 0 && (x & (x - 1)) == 0; }
 
+// dst[0 .. count) = src: one thread per 8 MB, at most eight.  One core of the host
+// copies 14 GB/s (37 ms for a 2-D 255 x 255, M = 1024 field); a request's data
+// should not take longer to hand over than the GPU takes to solve a smaller one.
+void copy_values(double* dst, const double* src, size_t count) {
+  const size_t each = size_t(1) << 20;
+  size_t parts = (count + each - 1) / each;
+  const size_t cores = std::max(1u, std::thread::hardware_concurrency());
+  parts = std::min(parts, std::min<size_t>(8, cores));
+  std::vector<std::thread> helpers;
+  size_t done = 0;  // parts handed to helpers
+  try {
+    for (; done + 1 < parts; ++done) {
+      const size_t a = count * done / parts, b = count * (done + 1) / parts;
+      helpers.emplace_back([=] { std::memcpy(dst + a, src + a, (b - a) * sizeof(double)); });
+    }
+  } catch (...) {  // no more threads: the rest here
+  }
+  const size_t a = parts > 0 ? count * done / parts : 0;
+  std::memcpy(dst + a, src + a, (count - a) * sizeof(double));
+  for (auto& h : helpers) h.join();
+}
+
 }  // namespace
 
 // Idle handles kept for later requests of the same shape and precision.
@@ -505,7 +527,7 @@ int submit_ticket(mgwr_server* s, const mgwr_request* rq, double* lent, uint64_t
     if (lent == nullptr) {
       if (!t->f.alloc(&s->pool, count)) return MGWR_E_NOMEM;
       const auto t0 = Clock::now();
-      std::memcpy(t->f.data(), rq->f, count * sizeof(double));
+      copy_values(t->f.data(), rq->f, count);
       std::lock_guard<std::mutex> lk(s->mu);
       s->submit_copy_s += std::chrono::duration<double>(Clock::now() - t0).count();
     }
@@ -661,10 +683,15 @@ int mgwr_poll(mgwr_server_t s, uint64_t ticket, int timeout_us, double* u_out, m
     const bool done = s->cv_done.wait_for(lk, std::chrono::microseconds(timeout_us),
                                           [&] { return t->state == 2; });
     if (!done) return MGWR_E_TIMEOUT;
+    it = s->tickets.find(ticket);  // others may have been added or taken meanwhile
+    if (it == s->tickets.end()) return MGWR_E_INVAL;
   }
   if (res != nullptr) *res = t->res;
-  if (u_out != nullptr && !t->u.empty()) std::memcpy(u_out, t->u.data(), t->u.size() * sizeof(double));
+  // the ticket is this call's now: its solution is copied without holding up the server
+  const std::unique_ptr<Ticket> own = std::move(it->second);
   s->tickets.erase(it);
+  lk.unlock();
+  if (u_out != nullptr && !t->u.empty()) copy_values(u_out, t->u.data(), t->u.size());
   return MGWR_OK;
 }
 
