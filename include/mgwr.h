@@ -59,12 +59,17 @@ extern "C" {
 #define MGWR_E_STATE (-9)   /* call not valid in the handle's current state   */
 
 /* arithmetic of a solve (mgwr_set_precision) */
-#define MGWR_FP64 0  /* every kernel in IEEE double                          */
+#define MGWR_FP64 0  /* fields in IEEE double, arithmetic at least as exact   */
 #define MGWR_MIXED 1 /* FP32 V-cycles on the defect, FP64 defect + update     */
 #define MGWR_MIXED_DD 2 /* FP32 V-cycles; defect + update in double-float    */
 #define MGWR_DD 3       /* refinement with double-float inner cycles         */
 #define MGWR_AUTO 4     /* MGWR_MIXED_DD or MGWR_DD by the grid (below)      */
-/* MGWR_MIXED keeps the finest iterate, the update and the stencil part of
+/* MGWR_FP64 computes in IEEE double, but for the half-sweeps of lines of 64 ..
+ * 1024 steps: the line products run as exact integer products of eight-bit
+ * slices on the tensor cores, rounded to double once (error about 1e-16 of a
+ * line's scale, below that of an FP64 transform); a line whose right-hand side
+ * holds an infinity or NaN becomes NaN.
+ * MGWR_MIXED keeps the finest iterate, the update and the stencil part of
  * every outer defect in IEEE double.  Its full outer defects take the time
  * convolution T_M u in double-float (FP32 instructions, error about 2^-44
  * |T_M u|, against about 1e-15 |T_M u| in FP64) when the tolerance is at least
@@ -203,7 +208,8 @@ int mgwr_set_outer_switch(mgwr_t h, double rel);
  * L/(8E) threads transforms one line pair of length L = 2M (8192 for
  * M > 4096, where E is 1 or 2), synchronising with warp barriers when the
  * group fits in one warp.  A request a length cannot take falls back to the
- * nearest smaller E; mgwr_get_engine_split reports the E launches use.
+ * nearest smaller E; mgwr_get_engine_split reports the E launches use.  The
+ * FP64 half-sweeps of 64 .. 1024 steps have one form, whatever E is set.
  * For MGWR_K_SWEEP32 (not the one-point solve) with 64 <= M <= 4096, `split`
  * may also be E | MGWR_SPLIT_STAGED: a persistent kernel whose thread groups
  * receive the f and neighbour lines of their next line pair in shared memory

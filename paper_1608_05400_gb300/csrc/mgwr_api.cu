@@ -95,6 +95,10 @@ struct mgwr_handle {
   double* dk = nullptr;         // batch * (M+1): d_0..d_M
   double* kcol = nullptr;       // batch * nlev * M inverse columns
   unsigned char* tc_band = nullptr;  // their Toeplitz bands in bf16 pieces (tensor-core sweeps)
+  // sliced bands of the inverse columns (FP64 half-sweeps on the tensor cores,
+  // lines of 64 .. 1024 steps) and the scratch of their digits
+  unsigned char* toep_band = nullptr;
+  unsigned char* toep_scratch = nullptr;
   double* c_dev = nullptr;      // batch
   Hier<double> h64;
   Hier<float> h32;
@@ -242,6 +246,10 @@ constexpr int defect_class() {
 // a valid line always lands) turns into an error of the call that ran it.
 int check_staging(mgwr_t h) {
   bool hit = false;
+  if (h->toep_band != nullptr) {
+    MGWR_CK(h, mgwr::take_toep_timeout(&hit));
+    if (hit) return fail(h, MGWR_E_CUDA, "sliced sweep: wait for its copies or MMAs gave up");
+  }
   MGWR_CK(h, mgwr::take_stage_timeout(&hit));
   if (hit) return fail(h, MGWR_E_CUDA, "staged sweep: wait for bulk copies gave up");
   MGWR_CK(h, mgwr::take_tc_timeout(&hit));
@@ -350,6 +358,20 @@ int ensure_h32(mgwr_t h) {
   return MGWR_OK;
 }
 
+// The sliced bands of the FP64 half-sweeps on the tensor cores and their
+// scratch (before any capture that runs them).
+int ensure_toep(mgwr_t h) {
+  if (h->toep_band != nullptr || !mgwr::toep_length(h->M)) return MGWR_OK;
+  const size_t lines = (size_t)h->B * h->nlev;
+  if (h->toep_scratch == nullptr)
+    MGWR_TRY(dev_alloc(h, &h->toep_scratch, mgwr::toep_scratch_bytes(shape(h, h->nlev - 1))));
+  unsigned char* band = nullptr;
+  MGWR_TRY(dev_alloc(h, &band, mgwr::toep_band_bytes(h->M) * lines));
+  MGWR_CK(h, mgwr::launch_toep_band(h->kcol, band, h->M, lines, h->stream));
+  h->toep_band = band;
+  return MGWR_OK;
+}
+
 // The double-float Toeplitz spectra and twiddles, split from FP64.
 int ensure_dd_spectra(mgwr_t h) {
   if (h->tspec_dd != nullptr) return MGWR_OK;
@@ -427,25 +449,21 @@ void prof_collect(mgwr_t h) {
 
 // ---- Algorithm 1 components ------------------------------------------------------
 
-template <class R>
-int coarsest(mgwr_t h, Hier<R>& H) {
-  const int pm = prof_begin(h, MGWR_K_COARSEST, (double)h->B);
-  MGWR_CK(h, mgwr::launch_sweep<R>(H.f[0], H.u[0], (R*)nullptr, H.spec, (size_t)h->nlev * h->L,
-                                    H.tw, H.zero, scratch_for<R>(h), shape(h, 0), 0, true, R(0),
-                                    split_of(h, sweep_class<R>(), 0) &
-                                        ~(mgwr::kTensor | mgwr::kRadix),
-                                    h->stream));
-  prof_end(h, pm);
-  H.rs[0] = R_STALE;
-  return MGWR_OK;
-}
-
 // One colour half-sweep of level l >= 1 (parity par) of the fields f -> u with
 // launch shape E: the tensor-core form for FP32 lines of 64 .. 256 steps when E
 // carries kTensor, else the FFT engine.
 template <class R>
 cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
                         const LevelShape& ls, int par, int E) {
+  if constexpr (std::is_same<R, double>::value) {
+    if (h->toep_band != nullptr) {
+      const size_t bb = mgwr::toep_band_bytes(h->M);
+      return mgwr::launch_sweep_toep(f, u, delta, h->kcol + (size_t)l * h->M,
+                                     (size_t)h->nlev * h->M, h->toep_band + (size_t)l * bb,
+                                     (size_t)h->nlev * bb, h->toep_scratch, ls, par, h->hinv2[l],
+                                     h->stream);
+    }
+  }
   if constexpr (std::is_same<R, float>::value) {
     const int eff = mgwr::effective_split(h->M, 4, E);
     if ((eff & mgwr::kTensor) && h->tc_band != nullptr) {
@@ -461,6 +479,27 @@ cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
   return mgwr::launch_sweep<R>(f, u, delta, H.spec + (size_t)l * h->L, (size_t)h->nlev * h->L,
                                H.tw, H.zero, scratch_for<R>(h), ls, par, false, R(h->hinv2[l]),
                                E & ~(mgwr::kTensor | mgwr::kRadix), h->stream);
+}
+
+template <class R>
+int coarsest(mgwr_t h, Hier<R>& H) {
+  const int pm = prof_begin(h, MGWR_K_COARSEST, (double)h->B);
+  if constexpr (std::is_same<R, double>::value) {
+    if (h->toep_band != nullptr) {
+      MGWR_CK(h, level_sweep(h, H, 0, H.f[0], H.u[0], (R*)nullptr, shape(h, 0), 0, 1));
+      prof_end(h, pm);
+      H.rs[0] = R_STALE;
+      return MGWR_OK;
+    }
+  }
+  MGWR_CK(h, mgwr::launch_sweep<R>(H.f[0], H.u[0], (R*)nullptr, H.spec, (size_t)h->nlev * h->L,
+                                    H.tw, H.zero, scratch_for<R>(h), shape(h, 0), 0, true, R(0),
+                                    split_of(h, sweep_class<R>(), 0) &
+                                        ~(mgwr::kTensor | mgwr::kRadix),
+                                    h->stream));
+  prof_end(h, pm);
+  H.rs[0] = R_STALE;
+  return MGWR_OK;
 }
 
 // One colour half-sweep at level l >= 1; delta != null also records the change of
@@ -929,7 +968,10 @@ int check_level(mgwr_t h, int hierarchy, int level) {
     return fail(h, MGWR_E_STATE, "the FP32 hierarchy exists only after mgwr_set_precision(MGWR_MIXED)");
   if (hierarchy == MGWR_HDD && !h->hdd.ready)
     return fail(h, MGWR_E_STATE, "the double-float hierarchy exists only after mgwr_set_precision(MGWR_DD)");
-  if (hierarchy == MGWR_H64) MGWR_TRY(ensure_full(h, h->h64));
+  if (hierarchy == MGWR_H64) {
+    MGWR_TRY(ensure_full(h, h->h64));
+    MGWR_TRY(ensure_toep(h));
+  }
   return MGWR_OK;
 }
 
@@ -1039,7 +1081,9 @@ int tune_hierarchy(mgwr_t h, Hier<R>& H, int cls_sweep, int cls_defect) {
     const LevelShape ls = tune_sample(h, l);
     st = ensure_field(h, &H.u[l], level_count(h, l));
     if (st == MGWR_OK) st = ensure_field(h, &H.f[l], level_count(h, l));
-    if (st == MGWR_OK)
+    // FP64 sweeps on the tensor cores have one launch shape
+    const bool fixed = std::is_same<R, double>::value && h->toep_band != nullptr;
+    if (st == MGWR_OK && !fixed)
       st = tune_class(h, cls_sweep, l, sizeof(R) == 4 ? 4 : 8, [&](int E) {
         // one smoothing step as the cycle runs it: red, then black recording its changes
         const Cx<R>* spec = H.spec + (size_t)l * h->L;
@@ -1185,6 +1229,9 @@ int refresh_derived(mgwr_t h) {
       MGWR_CK(h, mgwr::launch_band_bf16x3(h->kcol, h->tc_band, h->M, (size_t)h->B * h->nlev,
                                           h->stream));
   }
+  if (h->toep_band != nullptr)
+    MGWR_CK(h, mgwr::launch_toep_band(h->kcol, h->toep_band, h->M, (size_t)h->B * h->nlev,
+                                      h->stream));
   if (h->tspec_dd != nullptr)
     MGWR_CK(h, mgwr::launch_split_cx(h->tspec_dd, h->h64.tspec, (size_t)h->B * h->L, h->stream));
   if (h->hdd.ready)
@@ -1502,6 +1549,7 @@ int mgwr_autotune(mgwr_t h) {
   if (h == nullptr) return MGWR_E_INVAL;
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
   if (h->precision == MGWR_FP64) {
+    MGWR_TRY(ensure_toep(h));
     MGWR_TRY(tune_hierarchy(h, h->h64, MGWR_K_SWEEP64, MGWR_K_DEFECT64));
   } else if (h->precision == MGWR_DD) {
     MGWR_TRY(tune_hierarchy(h, h->hdd, MGWR_K_SWEEP_DD, MGWR_K_DEFECT_DD));
@@ -1635,7 +1683,10 @@ int solve_begin(mgwr_t h, SolveState& S, int cyc, int nu1, int nu2, double tol, 
   S.mixed = h->precision != MGWR_FP64;
   S.ddef = h->precision == MGWR_MIXED_DD || h->precision == MGWR_DD;
   S.ddc = h->precision == MGWR_DD;  // double-float inner cycles
-  if (h->precision == MGWR_FP64) MGWR_TRY(ensure_full(h, h->h64));
+  if (h->precision == MGWR_FP64) {
+    MGWR_TRY(ensure_full(h, h->h64));
+    MGWR_TRY(ensure_toep(h));
+  }
   const int L = h->nlev - 1;
   const size_t cntL = level_count(h, L);
   MGWR_CK(h, cudaEventRecord(h->ev0, h->stream));
@@ -2560,6 +2611,9 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
   if (M > mgwr::kShortMaxM)  // partitioned-convolution scratch: all block spectra of the finest level
     total += r512(16 * B * ((pts[0] + 1) / 2) * L);
   if (precision == MGWR_FP64) {
+    if (mgwr::toep_length(M))  // sliced bands and digits of the tensor-core sweeps
+      total += r512(mgwr::toep_band_bytes(M) * B * nlev) +
+               r512(mgwr::toep_scratch_bytes(LevelShape{d, n, M, batch}));
     for (size_t l = 0; l < nlev; ++l) total += (l + 1 < nlev ? 4 : 3) * r512(8 * B * pts[l] * M);
   } else if (precision == MGWR_DD) {
     total += 2 * r512(8 * B * pts[0] * M);  // FP64 finest iterate and right-hand side

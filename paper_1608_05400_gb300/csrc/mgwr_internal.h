@@ -136,6 +136,29 @@ cudaError_t launch_band_bf16x3(const double* kcol, unsigned char* band, int M, s
                                cudaStream_t s);
 cudaError_t take_tc_timeout(bool* hit);
 
+// One colour half-sweep of FP64 lines of M = 64 .. 1024 steps as sliced integer
+// products on the tensor cores, or where the lines are few as FP64 sums
+// (mgwr_toep.cu): as launch_sweep without all_points (the one point of the
+// coarsest grid is colour 0 of n = 1), the inverse column of instance b given
+// in FP64 (cols + b * cstride) and as its sliced band (band + b * bstride,
+// toep_band_bytes(M) bytes, written by launch_toep_band).  scratch holds
+// toep_scratch_bytes.  A wait that gives up (half a second) sets a flag read by
+// take_toep_timeout.  A line with an infinity or NaN in its gathered values
+// becomes NaN.
+inline bool toep_length(int M) { return M >= 64 && M <= 1024; }
+cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
+                              size_t cstride, const unsigned char* band, size_t bstride,
+                              unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
+                              cudaStream_t s);
+size_t toep_band_bytes(int M);
+// Bytes of scratch the launches on a level of this shape need (bounded: larger
+// fields go through it in slabs).
+size_t toep_scratch_bytes(const LevelShape& ls);
+// blob + line * toep_band_bytes(M): the sliced band of column cols[line].
+cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, size_t lines,
+                             cudaStream_t s);
+cudaError_t take_toep_timeout(bool* hit);
+
 // One colour half-sweep of FP32 lines of 64 .. 4096 steps on the register-pass
 // FFT engine (mgwr_fft_rp.cuh): as launch_sweep without all_points, with the
 // inverse-column spectra in that engine's spectral order (launch_spectra_rp).

@@ -1,0 +1,871 @@
+// FP64 Toeplitz products of whole time lines (64 .. 1024 steps): the FP64
+// smoother's half-sweep (Sec. 3 Eq. red-black, Sec. 6 Eq. red-black_2d) and
+// one-point solve, u_p = k * b_p with b_p = f_p + h^-2 sum of neighbour lines.
+//
+// GB300 issues two FP64 operations per clock and SM, so the FFT form of the
+// product (about 78 FP64 instructions per value at M = 1024) keeps that pipe
+// busy and cannot run faster.  Here both factors are cut into eight slices of
+// eight bits and multiplied as integers on tcgen05.mma (kind::f16), the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59,
+// 2012) on fp16 tensor cores as in Mukunoki, Ozaki, Ogita and Imamura (ISC 2020):
+//   b = 2^(E-6) sum_j B_j 2^(-8j),  k = 2^(F-6) sum_i K_i 2^(-8i),  i, j = 0..7,
+// with balanced digits of at most 128 (64 for the leading one), exact in fp16,
+// E and F the exponents of the largest |b| of the line and |k| of the column.
+// s_p, the sum of the products with i + j = p for p = 0..7, is an FP32
+// accumulator of integers; a segment of the sum is as long as keeps it within
+// 2^24, so every s_p is exact.  Segments are added in two 64-bit integers per
+// value and the total is rounded to FP64 once.  What is dropped, the products
+// with i + j > 7, is about 2^-59 (largest |k|) (largest |b|); the half-sweep's
+// error against 64-bit sums is that of the final rounding (about 1e-16 of the
+// line's scale; the FFT form's is 2e-16 to 4e-16).
+//
+// Two kernels per half-sweep:
+//  k_toep_gather  forms b (FP64), the line's exponent and the eight digits,
+//                 written as fp16 in the layout the MMA reads (16 bytes a value);
+//  k_toep_mma     one CTA per SM.  An item is NL lines x 128 output steps: the
+//                 MMA's 128 rows are output steps, its columns the lines, once
+//                 per slice j, so one instruction multiplies slice i of the
+//                 column with slices 0 .. 7-i of the lines (N = NL (8 - i)) and
+//                 the accumulator columns of order i + j are adjacent.
+// Because the time index of a chunk of 32 steps is stored reversed, element
+// (row, kk) of the Toeplitz operand depends on row + kk only, so its 8 x 8 core
+// matrices depend on one index and all blocks of all lags are windows into one
+// array of M/8 + 15 cores per slice (leading and stride byte offsets both 128
+// bytes): the whole operand (143 KB at M = 1024) stays in shared memory.
+// Far from the diagonal k is small and its leading digits vanish; the first
+// slice that is not zero from a lag on is recorded per 64 lags at set-up, and
+// the slices before it are neither loaded nor multiplied (on a fine level about
+// half the products remain).
+// Lines are processed in slabs whose digits stay in L2 between the kernels.
+//
+// Warp roles in k_toep_mma: warps 0-15 fold and store (tcgen05.ld), warp 16 loads
+// chunks of digits by bulk copies into a ring, warps 17 and 18 issue the MMAs; the
+// accumulator is double-buffered (2 x 8 NL columns).  Every wait is bounded.
+//
+// Measured (2-D, finest half-sweep, alpha = 0.5; slabs of 64 MB): 255 x 255, M =
+// 1024: FFT form 4.8 ms; 8 slabs of k_toep_gather 43 us (28 us of it FP64 sums at
+// the pipe's rate) and k_toep_mma 88 us: 1.05 ms.  Without its MMAs k_toep_mma takes
+// 69 us (folding: seven conversions a value and segment at a quarter of the rate,
+// tcgen05.ld latency, and the hand-overs of about 18 chunks an item).
+//
+// Where there are too few lines to fill the chip the product is a sum of FP64
+// products (k_toep_direct): one launch, 6 us for one line of 512 steps (FFT form
+// 26 us, the tensor-core pair 22 us).
+#include <cuda_fp16.h>
+
+#include <climits>
+
+#include "mgwr_common.cuh"
+#include "mgwr_tma.cuh"
+
+namespace mgwr {
+
+// Set when a CTA gave up waiting (read by take_toep_timeout).
+__device__ unsigned g_toep_timeout;
+
+namespace {
+
+constexpr int kSlices = 8;
+constexpr int kTile = 128;     // output steps of an item: the MMA's M
+constexpr int kChunk = 32;     // time steps per shared-memory chunk (two K = 16 steps)
+constexpr int kMaxStages = 8;  // chunks in flight, as many as shared memory holds
+constexpr int kFoldThreads = 512;
+constexpr int kLoader = 512, kIssuer = 544;  // first threads of warps 16 and 17
+constexpr int kIssuers = kChunk / 16;         // one warp per K step of a chunk
+constexpr int kThreads = kIssuer + 32 * kIssuers;
+
+__host__ __device__ constexpr int cores(int M) { return (M < kTile ? kTile : M) / 8 + 15; }
+__host__ __device__ constexpr size_t slice_bytes(int M) { return (size_t)cores(M) * 128; }
+// band blob: the slices, then { first slices by lag (4 bits per 64 lags), F, fold shift }
+__host__ __device__ constexpr size_t blob_bytes(int M) { return kSlices * slice_bytes(M) + 16; }
+
+struct BandHead {
+  unsigned long long first;
+  int F;
+  short shift;   // low bits dropped when the two sums are joined: |y| < 2^(62 + shift) units
+  short chunks;  // chunks from the diagonal down that have a nonzero slice
+};
+
+__device__ __forceinline__ const BandHead* band_head(const unsigned char* blob, int M) {
+  return reinterpret_cast<const BandHead*>(blob + kSlices * slice_bytes(M));
+}
+
+// Chunk c of tile tau holds the 32 steps from s0 = 128 tau + 96 - 32 c (M >= 128;
+// M - 32 - 32 c below): c counts from the diagonal down.
+__device__ __forceinline__ int tile_chunks(int M, int tau) {
+  return M < kTile ? M / kChunk : 4 * tau + 4;
+}
+__host__ __device__ __forceinline__ int chunk_lag0(int M, int c) {  // t0 - s0
+  return kChunk * c - (M < kTile ? M - kChunk : kTile - kChunk);
+}
+// smallest lag that chunks 2 x and 2 x + 1 multiply
+__device__ __forceinline__ int pair_lag(int M, int x) {
+  const int lag = chunk_lag0(M, 2 * x) - (kChunk - 1);
+  return lag > 0 ? lag : 0;
+}
+// first core of chunk c's window
+__device__ __forceinline__ int chunk_core(int M, int c) { return (chunk_lag0(M, c) + 96) / 8; }
+// first nonzero slice of chunk c
+__device__ __forceinline__ int first_slice(unsigned long long first, int c) {
+  return (int)(first >> (4 * (c >> 1))) & 15;
+}
+// Chunks of a segment starting with slice i0: an order sums at most 8 - i0
+// products a step, each at most 2^14, so 1024 / (8 - i0) steps stay within 2^24.
+__device__ __forceinline__ int segment_chunks(int i0) { return 32 / (kSlices - i0); }
+
+// exponent field of |x| (1 for zero and subnormals, 2047 for inf and NaN)
+__device__ __forceinline__ int exp_field(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7FF;
+  return e > 0 ? e : 1;
+}
+
+// The digits of x against the largest exponent field ef of its line: the
+// integer q = x 2^(62 - (ef - 1022)), |q| < 2^62 (bits below it rounded), plus 128
+// in every byte: byte j (from the low end) minus 128 is digit 7 - j.
+__device__ __forceinline__ unsigned long long biased_digits(double x, int ef) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e0 = (int)((b >> 52) & 0x7FF);
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  if (e0 > 0) m |= 1ull << 52;
+  int r = ef - (e0 > 0 ? e0 : 1);  // right shift of m 2^9
+  r = r > 63 ? 63 : r;
+  const unsigned long long q = ((m << 9) + ((1ull << r) >> 1)) >> r;
+  const unsigned long long s = (b >> 63) ? 0ull - q : q;
+  return s + 0x8080808080808080ull;
+}
+
+// Two values' digits of one byte position as fp16 pairs (x low, y high).
+__device__ __forceinline__ unsigned digit_pair(unsigned x, unsigned y, unsigned sel) {
+  const unsigned t = (__byte_perm(x, y, sel) & 0x00FF00FFu) | 0x64006400u;  // 1024 + byte
+  const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(1152.f));
+  return *reinterpret_cast<const unsigned*>(&v);
+}
+
+// ---- set-up ---------------------------------------------------------------------
+
+// The band of one column (blockIdx.x): core g holds k[8g - 127 + r + c] at row
+// r, column c, per slice; the first nonzero slice by lag; the exponent F.
+__global__ void __launch_bounds__(256)
+    k_toep_band(const double* __restrict__ cols, unsigned char* __restrict__ blob, int M) {
+  __shared__ short dig[kSlices][1024];
+  __shared__ int s_ef, s_last[kSlices];
+  __shared__ double s_sum[8];
+  const double* k = cols + (size_t)blockIdx.x * M;
+  unsigned char* out = blob + (size_t)blockIdx.x * blob_bytes(M);
+  if (threadIdx.x == 0) s_ef = 1;
+  if (threadIdx.x < kSlices) s_last[threadIdx.x] = -1;
+  __syncthreads();
+  int ef = 1;
+  for (int m = threadIdx.x; m < M; m += 256) ef = max(ef, exp_field(k[m]));
+  atomicMax(&s_ef, ef);
+  __syncthreads();
+  ef = s_ef;
+  double sum = 0.0;
+  for (int m = threadIdx.x; m < M; m += 256) {
+    const unsigned long long q = biased_digits(k[m], ef);
+    sum += fabs(k[m]);
+#pragma unroll
+    for (int i = 0; i < kSlices; ++i) {
+      const int v = (int)((q >> (8 * (7 - i))) & 0xFF) - 128;
+      dig[i][m] = (short)v;
+      if (v != 0) atomicMax(&s_last[i], m);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  for (int x = threadIdx.x; x < kSlices * cores(M) * 64; x += 256) {
+    const int i = x / (cores(M) * 64), rest = x - i * cores(M) * 64;
+    const int g = rest >> 6, r = (rest >> 3) & 7, c = rest & 7;
+    const int lag = 8 * g - 127 + r + c;
+    const int v = lag >= 0 && lag < M ? dig[i][lag] : 0;
+    *reinterpret_cast<__half*>(out + i * slice_bytes(M) + g * 128 + r * 16 + c * 2) =
+        __int2half_rn(v);
+  }
+  if (threadIdx.x == 0) {
+    unsigned long long first = 0;
+    const int pairs = M < kTile ? 1 : M / kChunk / 2;
+    for (int x = 0; x < pairs; ++x) {
+      int i = 0;
+      while (i < kSlices && s_last[i] < pair_lag(M, x)) ++i;
+      if (pair_lag(M, x) == 0) i = 0;  // the diagonal always runs (a zero column gives zeros)
+      first |= (unsigned long long)i << (4 * x);
+    }
+    // |y| <= |k|_1 2^E = 2^(E + F) 2^g, in units of 2^(E + F - 68): 2^(68 + g)
+    double total = 0.0;
+    for (int w = 0; w < 8; ++w) total += s_sum[w];
+    const int g = exp_field(total) - ef + 2;
+    BandHead* h = reinterpret_cast<BandHead*>(out + kSlices * slice_bytes(M));
+    h->first = first;
+    h->F = ef - 1022;
+    h->shift = (short)(6 + (g < 1 ? 1 : g > 20 ? 20 : g));
+    int live = 0;
+    while (live < pairs && first_slice(first, 2 * live) < kSlices) ++live;
+    h->chunks = (short)(2 * live);
+  }
+}
+
+// ---- gather ---------------------------------------------------------------------
+
+struct Geometry {
+  int d, n, M, par, npts;  // npts: lines of the colour per instance
+  int per_inst;            // groups of NL lines per instance
+  int group0, groups;      // the slab: groups group0 .. group0 + groups - 1 of all instances
+  size_t fstride;          // values of one instance's field
+  size_t bstride;          // bytes from one instance's band to the next
+};
+
+// b of steps m .. m + W - 1 of point p (line start `base`, neighbours by flag).
+template <int W>
+__device__ __forceinline__ void gather_steps(const double* __restrict__ f,
+                                             const double* __restrict__ u, size_t at, size_t M,
+                                             size_t nM, bool w, bool e, bool s, bool t,
+                                             double hinv2, double (&b)[W]) {
+  double a[W];
+#pragma unroll
+  for (int q = 0; q < W; q += 2) {
+    const double2 x =
+        w ? __ldg(reinterpret_cast<const double2*>(u + at - M + q)) : make_double2(0.0, 0.0);
+    a[q] = x.x;
+    a[q + 1] = x.y;
+  }
+  auto add = [&](const double* src) {
+#pragma unroll
+    for (int q = 0; q < W; q += 2) {
+      const double2 x = __ldg(reinterpret_cast<const double2*>(src + q));
+      a[q] += x.x;
+      a[q + 1] += x.y;
+    }
+  };
+  if (e) add(u + at + M);
+  if (s) add(u + at - nM);
+  if (t) add(u + at + nM);
+#pragma unroll
+  for (int q = 0; q < W; q += 2) {
+    const double2 x = __ldg(reinterpret_cast<const double2*>(f + at + q));
+    b[q] = fma(hinv2, a[q], x.x);
+    b[q + 1] = fma(hinv2, a[q + 1], x.y);
+  }
+}
+
+// One block per LPB lines: thread t holds line t % LPB, the octet t / LPB of its
+// steps.  LPB = 4 or 8 writes whole 32-byte sectors; small grids take fewer lines
+// per block, so that the FP64 sums of a line (four operations a value, two a clock
+// and SM: what bounds this kernel) spread over the SMs.
+template <int NL, int LPB>
+__global__ void __launch_bounds__(512, 3)
+    k_toep_gather(const double* __restrict__ f, const double* __restrict__ u,
+                  const unsigned char* __restrict__ band, unsigned char* __restrict__ dig,
+                  int* __restrict__ lexp, Geometry G, double hinv2) {
+  __shared__ int red[16][LPB];
+  const int T = blockDim.x;
+  const int g = blockIdx.x / (NL / LPB);
+  const int inst = (G.group0 + g) / G.per_inst;
+  const int x = threadIdx.x % LPB;
+  const int line = (blockIdx.x - g * (NL / LPB)) * LPB + x;  // of the group
+  const int k = (G.group0 + g - inst * G.per_inst) * NL + line;
+  const int M = G.M;
+  double b[8];
+  int ef = 1;
+  if (k < G.npts) {
+    int i = 0, j = 0;
+    const int p = colour_point(k, G.d, G.n, G.par, i, j);
+    const size_t base = inst * G.fstride + (size_t)p * M;
+    gather_steps<8>(f, u, base + 8 * (threadIdx.x / LPB), M, (size_t)G.n * M, i > 0,
+                    i < G.n - 1, G.d == 2 && j > 0, G.d == 2 && j < G.n - 1, hinv2, b);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) ef = max(ef, exp_field(b[q]));
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) b[q] = 0.0;
+  }
+  // the line's largest exponent: lanes of equal line, then the block's warps
+#pragma unroll
+  for (int o = LPB; o < 32; o <<= 1) ef = max(ef, __shfl_xor_sync(0xffffffffu, ef, o));
+  if ((threadIdx.x & 31) < LPB) red[threadIdx.x >> 5][x] = ef;
+  __syncthreads();
+  for (int w = 0; w < (T >> 5); ++w) ef = max(ef, red[w][x]);
+  if (threadIdx.x < LPB) {
+    const BandHead* h = band_head(band + inst * G.bstride, M);
+    // exponent of one unit of the joined sums (INT_MIN: infinities or NaN in the line)
+    lexp[g * NL + line] = ef == 2047 ? INT_MIN : ef - 1022 + h->F - 68 + h->shift;
+  }
+  unsigned lo[8], hi[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const unsigned long long z = biased_digits(b[q], ef);
+    lo[q] = (unsigned)z;
+    hi[q] = (unsigned)(z >> 32);
+  }
+  // chunk oct / 4; steps reversed within it: core 3 - oct % 4, column 7 - q
+  const int oct = threadIdx.x / LPB;
+  unsigned char* out = dig + ((size_t)g * (M / kChunk) + (oct >> 2)) * kSlices * NL * 64 +
+                       (line >> 3) * 512 + (3 - (oct & 3)) * 128 + (line & 7) * 16;
+#pragma unroll
+  for (int j = 0; j < kSlices; ++j) {
+    const unsigned sel =
+        (j & 3) == 0 ? 0x0703u : (j & 3) == 1 ? 0x0602u : (j & 3) == 2 ? 0x0501u : 0x0400u;
+    unsigned v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)  // columns 2c and 2c + 1
+      v[c] = j < 4 ? digit_pair(hi[7 - 2 * c], hi[6 - 2 * c], sel)
+                   : digit_pair(lo[7 - 2 * c], lo[6 - 2 * c], sel);
+    *reinterpret_cast<uint4*>(out + j * NL * 64) = make_uint4(v[0], v[1], v[2], v[3]);
+  }
+}
+
+// Few lines: the product as FP64 sums.  A block holds OB output steps of one
+// line, 256 / OB threads per step; b up to the last of them in shared memory.
+template <int OB>
+__global__ void __launch_bounds__(256)
+    k_toep_direct(const double* __restrict__ f, double* __restrict__ u, double* __restrict__ delta,
+                  const double* __restrict__ cols, size_t cstride, Geometry G, double hinv2) {
+  constexpr int LPO = 256 / OB;
+  __shared__ double sb[1024], sk[1024];
+  const int inst = blockIdx.y / G.npts;
+  const int k = blockIdx.y - inst * G.npts;
+  const int M = G.M;
+  const int t0 = (gridDim.x - 1 - blockIdx.x) * OB;  // longest sums first
+  int i = 0, j = 0;
+  const int p = colour_point(k, G.d, G.n, G.par, i, j);
+  const size_t base = inst * G.fstride + (size_t)p * M;
+  cols += inst * cstride;
+  for (int m = 2 * threadIdx.x; m < t0 + OB; m += 512) {
+    double b[2];
+    gather_steps<2>(f, u, base + m, M, (size_t)G.n * M, i > 0, i < G.n - 1, G.d == 2 && j > 0,
+                    G.d == 2 && j < G.n - 1, hinv2, b);
+    sb[m] = b[0];
+    sb[m + 1] = b[1];
+    const double2 c = __ldg(reinterpret_cast<const double2*>(cols + m));
+    sk[m] = c.x;
+    sk[m + 1] = c.y;
+  }
+  __syncthreads();
+  const int t = t0 + threadIdx.x / LPO;
+  const int lane = threadIdx.x % LPO;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int s = lane; s < t; s += 4 * LPO) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (s + q * LPO < t) a[q] = fma(sk[t - s - q * LPO], sb[s + q * LPO], a[q]);
+  }
+  double y = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+  for (int o = LPO / 2; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+  y = fma(sk[0], sb[t], y);  // the largest product last
+  if (lane == 0) {
+    if (delta != nullptr) delta[base + t] = y - u[base + t];
+    u[base + t] = y;
+  }
+}
+
+// ---- products ---------------------------------------------------------------------
+
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes; `lead`
+// bytes to the next core along K, `stride` bytes to the next eight rows.
+__device__ __forceinline__ uint64_t operand(unsigned addr, unsigned lead, unsigned stride) {
+  return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)(lead >> 4) << 16 |
+         (uint64_t)(stride >> 4) << 32 | (uint64_t)1 << 46;
+}
+
+// FP32 accumulator, fp16 A and B, both K-major, 128 rows, `n` columns.
+__device__ __forceinline__ uint32_t mma_shape(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_f16(unsigned tmem, uint64_t da, uint64_t db, uint32_t shape,
+                                        unsigned accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+      "l"(da), "l"(db), "r"(shape), "r"(accumulate)
+      : "memory");
+}
+
+__device__ __forceinline__ void mma_commit(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+          smem_u32(bar))
+      : "memory");
+}
+
+__device__ __forceinline__ void tc_fence_before() {
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+__device__ __forceinline__ void tc_fence_after() {
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_load4(unsigned addr, unsigned (&v)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr));
+}
+
+__device__ __forceinline__ void tmem_clear4(unsigned addr) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%1,%1,%1};" ::"r"(addr), "r"(0)
+               : "memory");
+}
+
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
+// A wait of the whole warp, its outcome uniform across the lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, unsigned parity) {
+  return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity) ? 1 : 0) != 0;
+}
+
+// The value of lane 0, uniform across the warp (the MMA's operands then live in
+// uniform registers).
+__device__ __forceinline__ unsigned uniform(unsigned x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
+// hi 2^32 + 256 lo, less its last `shift` bits (|result| < 2^62), times 2^e, rounded
+// once to FP64 (half away from zero) with integer operations only.
+__device__ __forceinline__ double join(long long hi, long long lo, int shift, int e) {
+  const long long v =
+      (hi << (32 - shift)) + (shift > 8 ? ((lo >> (shift - 9)) + 1) >> 1 : lo << (8 - shift));
+  if (v == 0) return 0.0;
+  if (e <= -1000 || e >= 900)
+    return e == INT_MIN ? __longlong_as_double(0x7FF8000000000000ll) : scalbn((double)v, e);
+  const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ull;
+  const unsigned long long mag = (unsigned long long)(v < 0 ? -v : v);
+  const int z = __clzll((long long)mag);
+  const unsigned long long m = mag << z;  // leading bit at 63
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1);  // 53 bits, carrying into 2^53
+  return __longlong_as_double(
+      (long long)(sign | (((unsigned long long)(e + 63 - z + 1022) << 52) + r)));
+}
+
+// Work order of a CTA.  Many groups: a contiguous run of them, every tile of
+// each (the band is reloaded only where the instance changes).  Few: items
+// dealt one by one, the longest tiles first.
+struct Items {
+  int groups, tiles, dealt;
+  __device__ __forceinline__ bool get(int it, int& g, int& tau) const {
+    if (dealt) {
+      const int x = blockIdx.x + it * gridDim.x;
+      if (x >= groups * tiles) return false;
+      const int q = x / groups;
+      tau = tiles - 1 - q;
+      g = x - q * groups;
+      return true;
+    }
+    const int a = (int)((long long)groups * blockIdx.x / gridDim.x);
+    const int b = (int)((long long)groups * (blockIdx.x + 1) / gridDim.x);
+    g = a + it / tiles;
+    tau = tiles - 1 - it % tiles;
+    return g < b;
+  }
+};
+
+template <int NL>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_toep_mma(double* __restrict__ u, double* __restrict__ delta,
+               const unsigned char* __restrict__ band, const unsigned char* __restrict__ dig,
+               const int* __restrict__ lexp, Geometry G, Items items, int stages) {
+  constexpr int kCols = kSlices * NL;               // columns of one accumulator
+  constexpr unsigned kTmem = 2 * kCols;             // 512 or 256
+  constexpr int kStage = kCols * kChunk * 2;        // bytes of a chunk's digits
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  // band: full / empty; chunk ring: full / empty; accumulators: full / empty
+  __shared__ __align__(8) uint64_t bars[2 + 2 * kMaxStages + 4];
+  uint64_t* const band_full = bars;
+  uint64_t* const band_empty = bars + 1;
+  uint64_t* const full = bars + 2;
+  uint64_t* const empty = full + kMaxStages;
+  uint64_t* const acc_full = empty + kMaxStages;
+  uint64_t* const acc_empty = acc_full + 2;
+  __shared__ unsigned tmem_slot;
+  const int M = G.M;
+  unsigned char* const sBand = smem_raw;
+  unsigned char* const sRing = smem_raw + kSlices * slice_bytes(M);
+
+  const int warp = threadIdx.x >> 5;
+  if (threadIdx.x == kLoader) {
+    mbar_init(band_full, 1);
+    mbar_init(band_empty, kIssuers);
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kIssuers);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&acc_full[a], kIssuers);
+      mbar_init(&acc_empty[a], kFoldThreads / 32);
+    }
+    mbar_fence_init();
+  }
+  if (warp == kIssuer / 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_slot)),
+                 "r"(kTmem)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = tmem_slot;
+  if (warp < kFoldThreads / 32) {
+    const unsigned at = tmem + ((unsigned)(32 * (warp & 3)) << 16);
+    for (int c = (warp >> 2) * 4; c < 2 * kCols; c += 16) tmem_clear4(at + (unsigned)c);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    tc_fence_before();
+  }
+  __syncthreads();
+  tc_fence_after();
+  bool ok = true;
+  int g = 0, tau = 0;
+
+  if (warp == kLoader / 32) {
+    if (threadIdx.x == kLoader) {
+      int cur = -1, bands = 0, chunks = 0, slot = 0, round = 0;
+      for (int it = 0; ok && items.get(it, g, tau); ++it) {
+        const int inst = (G.group0 + g) / G.per_inst;
+        const unsigned char* blob = band + inst * G.bstride;
+        if (inst != cur) {
+          if (bands > 0) ok = mbar_wait_bounded(band_empty, (unsigned)((bands - 1) & 1));
+          if (!ok) break;
+          mbar_arrive_expect_tx(band_full, (unsigned)(kSlices * slice_bytes(M)));
+          bulk_copy_g2s(sBand, blob, (unsigned)(kSlices * slice_bytes(M)), band_full);
+          ++bands;
+          cur = inst;
+        }
+        const unsigned long long first = band_head(blob, M)->first;
+        const int tc = tile_chunks(M, tau);
+        const int nc = min(tc, (int)band_head(blob, M)->chunks);
+        // digits of the tile's last chunk (c = 0), then backwards in time
+        const unsigned char* src = dig + ((size_t)g * (M / kChunk) + tc - 1) * kStage;
+        for (int c = 0; c < nc; ++c, src -= kStage) {
+          const int i0 = first_slice(first, c);
+          if (round > 0) ok = mbar_wait_bounded(&empty[slot], (unsigned)((round - 1) & 1));
+          if (!ok) break;
+          const unsigned bytes = (unsigned)((kSlices - i0) * NL * kChunk * 2);
+          mbar_arrive_expect_tx(&full[slot], bytes);
+          bulk_copy_g2s(sRing + slot * kStage, src, bytes, &full[slot]);
+          ++chunks;
+          if (++slot == stages) slot = 0, ++round;
+        }
+      }
+      if (!ok) {
+        // copies in flight land before the CTA can end
+        if (bands > 0) (void)mbar_wait_bounded(band_full, (unsigned)((bands - 1) & 1));
+        for (int x = chunks > stages ? chunks - stages : 0; x < chunks; ++x)
+          (void)mbar_wait_bounded(&full[x % stages], (unsigned)((x / stages) & 1));
+      }
+    }
+    __syncwarp();
+  } else if (warp >= kIssuer / 32) {
+    // Each issuer takes one K step of every chunk: waits and bookkeeping take a warp
+    // longer than the small MMAs of a step.  Accumulators start at zero (cleared by
+    // the warps that read them), so the order of the MMAs is free.  A whole warp
+    // walks the items (uniform control flow), one lane issues.
+    const bool lead = elect_one();
+    const unsigned tmem_u = uniform(tmem);
+    int cur = -1, bands = 0, seg = 0, slot = 0, round = 0, last = -1, last_round = 0;
+    const unsigned sb = (unsigned)slice_bytes(M) >> 4;
+    const unsigned kx = (unsigned)(warp - kIssuer / 32) * 16;  // operand offset of the K step
+    const uint64_t opA = operand(0, 128, 128) + ((smem_u32(sBand) >> 4) + kx);
+    const uint64_t opB = operand(0, 128, 512) + ((smem_u32(sRing) >> 4) + kx);
+    for (int it = 0; ok && items.get(it, g, tau); ++it) {
+      const int inst = (G.group0 + g) / G.per_inst;
+      if (inst != cur) {
+        if (cur >= 0 && lead) mma_commit(band_empty);  // when all products with the old band are done
+        ok = warp_wait(band_full, (unsigned)(bands & 1));
+        if (!ok) break;
+        ++bands;
+        cur = inst;
+      }
+      const BandHead* head = band_head(band + inst * G.bstride, M);
+      const unsigned long long f64 = head->first;
+      const unsigned long long first =
+          (unsigned long long)uniform((unsigned)(f64 >> 32)) << 32 | uniform((unsigned)f64);
+      const int nc = min(tile_chunks(M, tau), (int)uniform((unsigned)head->chunks));
+      for (int c = 0; ok && c < nc; ++seg) {
+        const int end = min(nc, c + segment_chunks(first_slice(first, c)));
+        const int a = seg & 1;
+        const unsigned dst = tmem_u + (unsigned)(a * kCols);
+        if (seg >= 2) ok = warp_wait(&acc_empty[a], (unsigned)((seg / 2 - 1) & 1));
+        for (; ok && c < end; ++c) {
+          ok = warp_wait(&full[slot], (unsigned)(round & 1));
+          if (!ok) break;
+          tc_fence_after();
+          if (lead) {
+            const int i0 = first_slice(first, c);
+            const uint64_t da = opA + (unsigned)chunk_core(M, c) * 8;
+            const uint64_t db = opB + (unsigned)slot * (kStage / 16);
+#pragma unroll
+            for (int i = 0; i < kSlices; ++i)
+              if (i >= i0)
+                mma_f16(dst + i * NL, da + (uint64_t)(i * sb), db, mma_shape(NL * (kSlices - i)), 1u);
+            mma_commit(&empty[slot]);
+            if (c + 1 == end) mma_commit(&acc_full[a]);
+          }
+          __syncwarp();
+          last = slot;
+          last_round = round;
+          if (++slot == stages) slot = 0, ++round;
+        }
+      }
+    }
+    // after a failure, what was issued finishes before the accumulators are released
+    if (!ok && last >= 0) (void)mbar_wait_bounded(&empty[last], (unsigned)(last_round & 1));
+  } else {
+    // warp w: steps 32 (w % 4) .. +31 of the tile, lines of quarter w / 4
+    constexpr int kMine = NL / 4;
+    const int lane = threadIdx.x & 31;
+    const int mine = (warp >> 2) * kMine;
+    const unsigned lane_row = (unsigned)(32 * (warp & 3)) << 16;
+    int seg = 0;
+    for (int it = 0; ok && items.get(it, g, tau); ++it) {
+      const int inst = (G.group0 + g) / G.per_inst;
+      const BandHead* head = band_head(band + inst * G.bstride, M);
+      const unsigned long long first = head->first;
+      const int shift = head->shift;
+      const int nc = min(tile_chunks(M, tau), (int)head->chunks);
+      // lane x holds the point and exponent of line x of this quarter
+      const int k = (G.group0 + g - inst * G.per_inst) * NL + mine + (lane & (kMine - 1));
+      int p = -1, e = 0;
+      if (k < G.npts) {
+        int i = 0, j = 0;
+        p = colour_point(k, G.d, G.n, G.par, i, j);
+        e = lexp[g * NL + mine + (lane & (kMine - 1))];
+      }
+      long long hi[kMine], lo[kMine];
+#pragma unroll
+      for (int x = 0; x < kMine; ++x) hi[x] = lo[x] = 0;
+      for (int c = 0; c < nc;) {
+        const int i0 = first_slice(first, c);
+        const int a = seg & 1;
+        ok = warp_wait(&acc_full[a], (unsigned)((seg / 2) & 1));
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int x0 = 0; x0 < kMine; x0 += 4) {
+          unsigned v[kSlices][4];
+#pragma unroll
+          for (int p = 0; p < kSlices; ++p) {
+            if (p >= i0) {
+              tmem_load4(tmem + lane_row + (unsigned)(a * kCols + p * NL + mine + x0), v[p]);
+            } else {
+#pragma unroll
+              for (int x = 0; x < 4; ++x) v[p][x] = 0u;
+            }
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int p = 0; p < kSlices; ++p)
+            if (p >= i0) tmem_clear4(tmem + lane_row + (unsigned)(a * kCols + p * NL + mine + x0));
+          // s_0 .. s_3 into hi (|256 s_0 + s_1|, |256 s_2 + s_3| < 2^31), the rest into lo
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            auto s = [&](int p) { return __float2int_rn(__uint_as_float(v[p][x])); };
+            long long& h = hi[x0 + x];
+            long long& l = lo[x0 + x];
+            if (i0 < 4) {
+              h = mad_wide(s(0) * 256 + s(1), 65536, h);
+              h = mad_wide(s(2) * 256 + s(3), 1, h);
+            }
+            // s_6 + s_7 / 256 to the nearest integer: 2^-61 of (largest |k|) (largest |b|)
+            const int s67 = __float2int_rn(
+                fmaf(__uint_as_float(v[7][x]), 0.00390625f, __uint_as_float(v[6][x])));
+            l = mad_wide(s(4), 65536, l);
+            l = mad_wide(s(5), 256, l);
+            l = mad_wide(s67, 1, l);
+          }
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[a]);
+        ++seg;
+        c += segment_chunks(i0);
+      }
+      if (!ok) break;
+      const int t = kTile * tau + 32 * (warp & 3) + lane;
+#pragma unroll
+      for (int x = 0; x < kMine; ++x) {
+        const int px = __shfl_sync(0xffffffffu, p, x);
+        const int ex = __shfl_sync(0xffffffffu, e, x);
+        if (px < 0 || t >= M) continue;
+        const double y = join(hi[x], lo[x], shift, ex);
+        const size_t at = inst * G.fstride + (size_t)px * M + t;
+        if (delta != nullptr) delta[at] = y - u[at];
+        u[at] = y;
+      }
+    }
+  }
+  if (!ok) atomicOr(&g_toep_timeout, 1u);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kIssuer / 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem)
+                 : "memory");
+}
+
+// Bytes of a slab's digits: what stays in L2 (129 MB) from one kernel to the next.
+constexpr size_t kSlabBytes = size_t(64) << 20;
+constexpr size_t kLineValue = 2 * kSlices;  // bytes of digits per value
+
+// Lines per group: 32, or 16 while that leaves SMs without an item.
+int lines_per_group(int M, int npts, int batch) {
+  const long long items = (long long)((npts + 31) / 32) * batch * ((M + kTile - 1) / kTile);
+  return items >= sm_count() ? 32 : 16;
+}
+
+int slab_groups(int M, int NL, int groups) {
+  const size_t per = (size_t)NL * M * kLineValue;
+  long long most = (long long)(kSlabBytes / per);
+  if (most < 1) most = 1;
+  const long long slabs = (groups + most - 1) / most;
+  return (int)((groups + slabs - 1) / slabs);
+}
+
+template <int NL>
+cudaError_t gather_launch(const double* f, const double* u, const unsigned char* band,
+                          unsigned char* dig, int* lexp, const Geometry& G, double hinv2,
+                          cudaStream_t s) {
+  const int M = G.M;
+#define MGWR_GATHER(LPB)                                                                  \
+  k_toep_gather<NL, LPB><<<(unsigned)(G.groups * (NL / LPB)), LPB * M / 8, 0, s>>>(f, u, band, dig, \
+                                                                                lexp, G, hinv2)
+  if (M >= 256 && G.groups * (NL / 4) < 2 * sm_count()) {
+    MGWR_GATHER(1);
+  } else if (M == 128 && G.groups * (NL / 8) < 2 * sm_count()) {
+    MGWR_GATHER(2);
+  } else if (M >= 512 || (M == 64 && G.groups * (NL / 8) < 2 * sm_count())) {
+    MGWR_GATHER(4);
+  } else {
+    MGWR_GATHER(8);
+  }
+#undef MGWR_GATHER
+  return counted(cudaGetLastError());
+}
+
+template <int NL>
+cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigned char* band,
+                        unsigned char* scratch, const Geometry& G, double hinv2, cudaStream_t s) {
+  const int M = G.M;
+  unsigned char* dig = scratch;
+  int* lexp = reinterpret_cast<int*>(scratch + (size_t)G.groups * NL * M * kLineValue);
+  cudaError_t e = gather_launch<NL>(f, u, band, dig, lexp, G, hinv2, s);
+  if (e != cudaSuccess) return e;
+  Items items;
+  items.groups = G.groups;
+  items.tiles = (M + kTile - 1) / kTile;
+  items.dealt = G.groups < 4 * sm_count();
+  const long long count = items.dealt ? (long long)G.groups * items.tiles : G.groups;
+  const unsigned grid = (unsigned)(count < sm_count() ? count : sm_count());
+  constexpr size_t kStage = (size_t)kSlices * NL * kChunk * 2;
+  const size_t band_bytes = kSlices * slice_bytes(M);
+  int stages = (int)((226 * 1024 - band_bytes) / kStage);
+  if (stages > kMaxStages) stages = kMaxStages;
+  // at least half the SM's shared memory and one byte: one CTA per SM, whose
+  // accumulators take its tensor memory (NL = 32)
+  size_t smem = band_bytes + stages * kStage;
+  if (smem < 116 * 1024) smem = 116 * 1024;
+  e = prepare_smem(k_toep_mma<NL>, smem);
+  if (e != cudaSuccess) return e;
+  k_toep_mma<NL><<<grid, kThreads, smem, s>>>(u, delta, band, dig, lexp, G, items, stages);
+  return counted(cudaGetLastError());
+}
+
+// Multiply-adds up to which the FP64 sums run (the chip does 304 a clock, 14000
+// clocks in all).  Measured at M = 512: 25 lines (3.3 M) 17 us by sums, 21 us by
+// the tensor-core pair, which takes as long for any grid up to one item per SM;
+// 31 lines (4.1 M) 23 against 21 us.
+constexpr long long kDirectWork = 1ll << 22;
+
+}  // namespace
+
+size_t toep_band_bytes(int M) { return blob_bytes(M); }
+
+cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, size_t lines,
+                             cudaStream_t s) {
+  k_toep_band<<<(unsigned)lines, 256, 0, s>>>(cols, blob, M);
+  return counted(cudaGetLastError());
+}
+
+size_t toep_scratch_bytes(const LevelShape& ls) {
+  // no slab of any colour or group size holds more lines than this
+  const size_t pts = (size_t)colour_count(ls.d, ls.n, 0);
+  size_t lines = ((pts + 31) / 32 * 32) * ls.batch;
+  const size_t per = (size_t)ls.M * kLineValue;
+  const size_t most = kSlabBytes / per + 32;
+  if (lines > most) lines = most;
+  return lines * (per + sizeof(int));
+}
+
+cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
+                              size_t cstride, const unsigned char* band, size_t bstride,
+                              unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
+                              cudaStream_t s) {
+  if (!toep_length(ls.M)) return cudaErrorInvalidValue;
+  const int npts = colour_count(ls.d, ls.n, par);
+  if (npts == 0 || ls.batch == 0) return cudaSuccess;
+  Geometry G;
+  G.d = ls.d;
+  G.n = ls.n;
+  G.M = ls.M;
+  G.par = par;
+  G.npts = npts;
+  G.fstride = ls.field_stride();
+  G.bstride = bstride;
+  const long long lines = (long long)npts * ls.batch;
+  if (lines * ls.M * ls.M / 2 <= kDirectWork && lines <= 65535) {
+    G.per_inst = G.group0 = G.groups = 0;
+    // fewest steps a block (shortest sums per block, but every block gathers its
+    // line up to its last step) with at most two blocks per SM; by the instance's
+    // lines, so that a batch sums as one instance does
+    const long long values = (long long)npts * ls.M, blocks = 2 * sm_count();
+#define MGWR_DIRECT(OB)                                                                     \
+  k_toep_direct<OB><<<dim3(ls.M / OB, (unsigned)lines), 256, 0, s>>>(f, u, delta, cols, cstride, \
+                                                                     G, hinv2)
+    if (values / 8 <= blocks)
+      MGWR_DIRECT(8);
+    else if (values / 16 <= blocks)
+      MGWR_DIRECT(16);
+    else
+      MGWR_DIRECT(32);
+#undef MGWR_DIRECT
+    return counted(cudaGetLastError());
+  }
+  const int NL = lines_per_group(ls.M, npts, ls.batch);
+  G.per_inst = (npts + NL - 1) / NL;
+  const int total = G.per_inst * ls.batch;
+  const int step = slab_groups(ls.M, NL, total);
+  for (int g0 = 0; g0 < total; g0 += step) {
+    G.group0 = g0;
+    G.groups = total - g0 < step ? total - g0 : step;
+    const cudaError_t e = NL == 32 ? slab_launch<32>(f, u, delta, band, scratch, G, hinv2, s)
+                                   : slab_launch<16>(f, u, delta, band, scratch, G, hinv2, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t take_toep_timeout(bool* hit) {
+  unsigned v = 0;
+  cudaError_t e = cudaMemcpyFromSymbol(&v, g_toep_timeout, sizeof(v));
+  if (e != cudaSuccess) return e;
+  *hit = v != 0;
+  if (v != 0) {
+    const unsigned z = 0;
+    e = cudaMemcpyToSymbol(g_toep_timeout, &z, sizeof(z));
+  }
+  return e;
+}
+
+}  // namespace mgwr

@@ -1,0 +1,130 @@
+"""FP64 half-sweeps of lines of 64 .. 1024 steps (sliced integer products on the tensor cores,
+FP64 sums where the lines are few) against sums in extended precision.
+
+Bounds, against S = sum |k| |b| of a value (b the gathered line, k the inverse column):
+  * sliced: b keeps 59 bits below its largest operand, the dropped products are below
+    2^-59 (largest |k|) (largest |b|), the total is rounded once: 4e-16 of the largest S and b.
+  * FP64 sums: b rounded five times, at most 32 products a thread in four chains, five shuffles:
+    about twenty roundings, 20 * 2^-53 = 2.3e-15.
+"""
+import numpy as np
+import pytest
+
+from paper_1608_05400_gb300 import inputs
+from paper_1608_05400_gb300 import mgwr as G
+
+pytestmark = pytest.mark.gpu
+Q = np.longdouble
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    G.load()
+
+
+def _points(d, n, colour):
+    if d == 1:
+        return [i for i in range(n) if i % 2 == (1 if colour == G.MGWR_RED else 0)]
+    return [i + n * j for j in range(n) for i in range(n) if (i + j) % 2 == colour]
+
+
+def _gathered(u, f, p, d, n):
+    i, j = (p, 0) if d == 1 else (p % n, p // n)
+    s = np.zeros(u.shape[1], dtype=Q)
+    for ok, q in ((i > 0, p - 1), (i < n - 1, p + 1), (d == 2 and j > 0, p - n),
+                  (d == 2 and j < n - 1, p + n)):
+        if ok:
+            s = s + u[q].astype(Q)
+    return f[p].astype(Q) + Q(float((n + 1) ** 2)) * s
+
+
+def _check(s, d, n, M, colour, u, f, batch, sample, bound):
+    l = s.num_levels() - 1
+    shape = (batch, n ** d, M) if batch > 1 else (n ** d, M)
+    s.field_set(G.MGWR_H64, l, G.MGWR_U, u.reshape(shape))
+    s.field_set(G.MGWR_H64, l, G.MGWR_F, f.reshape(shape))
+    s.smooth(G.MGWR_H64, l, colour)
+    got = s.field_get(G.MGWR_H64, l, G.MGWR_U).reshape(batch, n ** d, M)
+    k = s.inverse_column(l).reshape(batch, M)
+    pts = _points(d, n, colour)
+    others = np.setdiff1d(np.arange(n ** d), pts)
+    np.testing.assert_array_equal(got[:, others], u[:, others])
+    for b in range(batch):
+        kq = k[b].astype(Q)
+        for p in sorted({pts[int(x * (len(pts) - 1))] for x in sample}):
+            line = _gathered(u[b], f[b], p, d, n)
+            want = np.array([np.dot(kq[:m + 1][::-1], line[:m + 1]) for m in range(M)])
+            scale = np.array([np.dot(abs(kq[:m + 1][::-1]), abs(line[:m + 1])) for m in range(M)])
+            err = np.abs(got[b, p].astype(Q) - want)
+            assert float(err.max()) <= bound * float(scale.max()), (b, p, float(err.max() / scale.max()))
+
+
+# (d, n, M, batch): the two forms on both sides of their boundary (2^22 products), groups of 16
+# and of 32 lines, partly filled groups, several slabs, the shortest and the longest lines, and
+# instances with columns of their own
+@pytest.mark.parametrize("d,n,M,batch", [
+    (1, 1, 64, 1), (1, 63, 64, 1), (2, 15, 128, 1), (1, 31, 1024, 1),       # sums
+    (2, 63, 64, 3), (1, 1023, 128, 1), (2, 15, 256, 3), (1, 127, 512, 1), (2, 7, 1024, 2),
+    (2, 127, 256, 1), (2, 127, 1024, 1)])                                    # sliced
+@pytest.mark.parametrize("data", ["random", "smooth", "wide"])
+def test_half_sweep_against_extended_sums(d, n, M, batch, data):
+    if data != "random" and n == 127 and d == 2:
+        pytest.skip("one kind of data at the large sizes")
+    rng = np.random.default_rng(d + n + M)
+    N = n ** d
+    t = np.arange(1, M + 1) / M
+    if data == "random":
+        u, f = rng.uniform(-1, 1, (batch, N, M)), rng.uniform(-1, 1, (batch, N, M)) * (n + 1) ** 2
+    elif data == "smooth":
+        x = np.sin(np.pi * np.arange(1, N + 1) / (N + 1))[None, :, None]
+        u, f = x * t ** 0.3 * np.ones((batch, 1, 1)), x * (1 + 20 * t) * np.ones((batch, 1, 1))
+    else:  # twelve orders of magnitude within a line
+        u, f = (rng.uniform(-1, 1, (batch, N, M)) * 10.0 ** rng.uniform(-12, 0, (batch, N, M))
+                for _ in range(2))
+    lines = len(_points(d, n, G.MGWR_BLACK if n == 1 and d == 1 else G.MGWR_RED)) * batch
+    bound = 2.3e-15 if lines * M * M // 2 <= 1 << 22 else 4e-16
+    alphas = 0.45 if batch == 1 else list(np.linspace(0.15, 0.95, batch))
+    with G.Solver(d, n, M, 1.0, alphas) as s:
+        colour = G.MGWR_RED
+        if n == 1:  # the one point is colour 0 whatever the call names
+            s.field_set(G.MGWR_H64, 0, G.MGWR_F, f[0])
+            s.coarsest(G.MGWR_H64)
+            got, k = s.field_get(G.MGWR_H64, 0, G.MGWR_U)[0], s.inverse_column(0).astype(Q)
+            want = np.array([np.dot(k[:m + 1][::-1], f[0, 0, :m + 1].astype(Q)) for m in range(M)])
+            assert float(np.abs(got - want).max()) <= bound * float(np.abs(k).sum() * np.abs(f).max())
+            return
+        _check(s, d, n, M, colour, u, f, batch, (0.0, 0.37, 0.5, 1.0), bound)
+
+
+@pytest.mark.parametrize("scale", [1e-290, 1e290])
+def test_half_sweep_scales_exactly(scale):
+    # a power of two in f and u scales the half-sweep exactly, to the ends of FP64's range
+    d, n, M = 1, 255, 256
+    two = 2.0 ** round(np.log2(scale))
+    u, f = inputs.random_field(n, M, 1), inputs.random_field(n, M, 2, scale=(n + 1.0) ** 2)
+    out = []
+    for c in (1.0, two):
+        with G.Solver(d, n, M, 1.0, 0.5) as s:
+            l = s.num_levels() - 1
+            s.field_set(G.MGWR_H64, l, G.MGWR_U, c * u)
+            s.field_set(G.MGWR_H64, l, G.MGWR_F, c * f)
+            s.smooth(G.MGWR_H64, l, G.MGWR_RED)
+            out.append(s.field_get(G.MGWR_H64, l, G.MGWR_U))
+    np.testing.assert_array_equal(out[1], two * out[0])
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_infinities_and_nan_reach_the_solver(bad):
+    for d, n, M in ((1, 255, 256), (1, 31, 64)):  # sliced and sums
+        f = inputs.random_field(n, M, 3)
+        f[n // 2, M // 3] = bad
+        with G.Solver(d, n, M, 1.0, 0.5) as s:
+            s.set_rhs(f)
+            with pytest.raises(G.MGWRError) as e:
+                s.solve(1, 1, 1, tol=1e-10, max_cycles=5)
+            assert e.value.status == G.MGWR_E_NUMERIC
+            l = s.num_levels() - 1
+            s.field_set(G.MGWR_H64, l, G.MGWR_F, f)
+            s.field_set(G.MGWR_H64, l, G.MGWR_U, np.zeros_like(f))
+            s.smooth(G.MGWR_H64, l, G.MGWR_RED)
+            assert not np.isfinite(s.field_get(G.MGWR_H64, l, G.MGWR_U)[n // 2]).all()
