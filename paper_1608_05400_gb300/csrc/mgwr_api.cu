@@ -58,6 +58,10 @@ struct Hier {
   std::vector<R*> u, f, r;        // per level: batch * N_l * M values each
   std::vector<R*> dl;             // per level: black-point changes of the last step
   std::vector<int> rs;            // per level: RState of r
+  // Within a cycle, per level: u is zero but its memory was not cleared (the
+  // visit's first sweep or interpolation writes it without reading it); and the
+  // last step started there, so the black points' changes are their values.
+  std::vector<char> uz, from_zero;
   Cx<R>* spec = nullptr;          // batch * nlev * L: spectra of the inverse columns
   Cx<R>* spec_rp = nullptr;       // the same in the register-pass engine's order (FP32)
   Cx<R>* tspec_rp = nullptr;      // the Toeplitz spectra in that order (FP32)
@@ -326,6 +330,8 @@ void init_hier(mgwr_t h, Hier<R>& H) {
   H.r.assign(h->nlev, nullptr);
   H.dl.assign(h->nlev, nullptr);
   H.rs.assign(h->nlev, R_STALE);
+  H.uz.assign(h->nlev, 0);
+  H.from_zero.assign(h->nlev, 0);
 }
 
 int ensure_h32(mgwr_t h) {
@@ -454,14 +460,14 @@ void prof_collect(mgwr_t h) {
 // carries kTensor, else the FFT engine.
 template <class R>
 cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
-                        const LevelShape& ls, int par, int E) {
+                        const LevelShape& ls, int par, int E, bool zero_u = false) {
   if constexpr (std::is_same<R, double>::value) {
     if (h->toep_band != nullptr) {
       const size_t bb = mgwr::toep_band_bytes(h->M);
       return mgwr::launch_sweep_toep(f, u, delta, h->kcol + (size_t)l * h->M,
                                      (size_t)h->nlev * h->M, h->toep_band + (size_t)l * bb,
                                      (size_t)h->nlev * bb, h->toep_scratch, ls, par, h->hinv2[l],
-                                     h->stream);
+                                     h->stream, zero_u);
     }
   }
   if constexpr (std::is_same<R, float>::value) {
@@ -469,16 +475,16 @@ cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
     if ((eff & mgwr::kTensor) && h->tc_band != nullptr) {
       const size_t bb = mgwr::tc_band_bytes(h->M);
       return mgwr::launch_sweep_tc(f, u, delta, h->tc_band + (size_t)l * bb, (size_t)h->nlev * bb,
-                                   ls, par, (float)h->hinv2[l], h->stream);
+                                   ls, par, (float)h->hinv2[l], h->stream, zero_u);
     }
     if ((eff & mgwr::kRadix) && H.spec_rp != nullptr)
       return mgwr::launch_sweep_rp(f, u, delta, H.spec_rp + (size_t)l * h->L,
                                    (size_t)h->nlev * h->L, H.tw, H.zero, ls, par,
-                                   (float)h->hinv2[l], eff & ~mgwr::kRadix, h->stream);
+                                   (float)h->hinv2[l], eff & ~mgwr::kRadix, h->stream, zero_u);
   }
   return mgwr::launch_sweep<R>(f, u, delta, H.spec + (size_t)l * h->L, (size_t)h->nlev * h->L,
                                H.tw, H.zero, scratch_for<R>(h), ls, par, false, R(h->hinv2[l]),
-                               E & ~(mgwr::kTensor | mgwr::kRadix), h->stream);
+                               E & ~(mgwr::kTensor | mgwr::kRadix), h->stream, zero_u);
 }
 
 template <class R>
@@ -489,29 +495,30 @@ int coarsest(mgwr_t h, Hier<R>& H) {
       MGWR_CK(h, level_sweep(h, H, 0, H.f[0], H.u[0], (R*)nullptr, shape(h, 0), 0, 1));
       prof_end(h, pm);
       H.rs[0] = R_STALE;
+      H.uz[0] = 0;
       return MGWR_OK;
     }
   }
+  int E = split_of(h, sweep_class<R>(), 0);
   MGWR_CK(h, mgwr::launch_sweep<R>(H.f[0], H.u[0], (R*)nullptr, H.spec, (size_t)h->nlev * h->L,
                                     H.tw, H.zero, scratch_for<R>(h), shape(h, 0), 0, true, R(0),
-                                    split_of(h, sweep_class<R>(), 0) &
-                                        ~(mgwr::kTensor | mgwr::kRadix),
-                                    h->stream));
+                                    E & ~(mgwr::kTensor | mgwr::kRadix), h->stream));
   prof_end(h, pm);
   H.rs[0] = R_STALE;
+  H.uz[0] = 0;
   return MGWR_OK;
 }
 
 // One colour half-sweep at level l >= 1; delta != null also records the change of
 // every swept line (used by the black half-sweep ending a smoothing step).
 template <class R>
-int sweep_colour(mgwr_t h, Hier<R>& H, int l, int colour, R* delta) {
+int sweep_colour(mgwr_t h, Hier<R>& H, int l, int colour, R* delta, bool zero_u = false) {
   const int par = parity(h, colour);
   const size_t N = points(h, l);
   const double lines = (double)h->B * (double)(par == 0 ? (N + 1) / 2 : N / 2);
   const int pm = prof_begin(h, sweep_class<R>(), lines);
   MGWR_CK(h, level_sweep(h, H, l, H.f[l], H.u[l], delta, shape(h, l), par,
-                         split_of(h, sweep_class<R>(), l)));
+                         split_of(h, sweep_class<R>(), l), zero_u));
   prof_end(h, pm);
   return MGWR_OK;
 }
@@ -526,16 +533,27 @@ int smooth_colour(mgwr_t h, Hier<R>& H, int l, int colour) {
 
 // `steps` red-black smoothing steps; with `record`, the last black half-sweep
 // records its changes so that a defect that follows needs no convolution
-// (without, the level's defect state is stale).
+// (without, the level's defect state is stale).  A step from u = 0 reads no
+// iterate: the red points have no neighbour sums, and the black points' changes
+// are their new values, which need no record.
 template <class R>
 int smooth(mgwr_t h, Hier<R>& H, int l, int steps, bool record = true) {
   for (int s = 0; s < steps; ++s) {
-    MGWR_TRY(sweep_colour(h, H, l, MGWR_RED, (R*)nullptr));
-    MGWR_TRY(sweep_colour(h, H, l, MGWR_BLACK,
-                          record && s == steps - 1 ? H.dl[l] : (R*)nullptr));
+    const bool zero = H.uz[l] != 0;
+    const bool rec = record && s == steps - 1;
+    MGWR_TRY(sweep_colour(h, H, l, MGWR_RED, (R*)nullptr, zero));
+    MGWR_TRY(sweep_colour(h, H, l, MGWR_BLACK, rec && !zero ? H.dl[l] : (R*)nullptr));
+    H.uz[l] = 0;
+    H.from_zero[l] = rec && zero;
   }
   if (steps > 0) H.rs[l] = record ? R_DELTA : R_STALE;
   return MGWR_OK;
+}
+
+// The black points' changes of the last recording step (state R_DELTA).
+template <class R>
+const R* changes(const Hier<R>& H, int l) {
+  return H.from_zero[l] ? H.u[l] : H.dl[l];
 }
 
 // Full defect r = f - (T_M (x) I + A_h) u with one FFT convolution per line.
@@ -552,15 +570,17 @@ int defect(mgwr_t h, Hier<R>& H, int l, unsigned long long* norm_bits) {
   return MGWR_OK;
 }
 
-// Defect of level l from the last smoothing step's changes (no convolution).
+// Defect of level l from the last smoothing step's changes (no convolution);
+// without `keep` only its norm.
 template <class R>
-int defect_from_delta(mgwr_t h, Hier<R>& H, int l, unsigned long long* norm_bits) {
+int defect_from_delta(mgwr_t h, Hier<R>& H, int l, unsigned long long* norm_bits,
+                      bool keep = true) {
   const int pm = prof_begin(h, MGWR_K_DEFECT_DELTA, (double)(points(h, l) * h->B));
-  MGWR_CK(h, mgwr::launch_defect_from_delta<R>(H.dl[l], H.r[l], H.zero, shape(h, l),
-                                                parity(h, MGWR_RED), R(h->hinv2[l]), norm_bits,
-                                                h->stream));
+  MGWR_CK(h, mgwr::launch_defect_from_delta<R>(changes(H, l), keep ? H.r[l] : (R*)nullptr, H.zero,
+                                                shape(h, l), parity(h, MGWR_RED), R(h->hinv2[l]),
+                                                norm_bits, h->stream));
   prof_end(h, pm);
-  H.rs[l] = R_CURRENT;
+  if (keep) H.rs[l] = R_CURRENT;
   return MGWR_OK;
 }
 
@@ -585,47 +605,62 @@ int current_defect(mgwr_t h, Hier<R>& H, int l, const R** out) {
   return MGWR_OK;
 }
 
+// `clear`: the coarse iterate's memory is zeroed; else it is marked zero for the
+// cycle that follows.
 template <class R>
-int restrict_into(mgwr_t h, Hier<R>& H, int l, const R* r) {
+int restrict_into(mgwr_t h, Hier<R>& H, int l, const R* r, bool clear) {
   const int pm = prof_begin(h, MGWR_K_RESTRICT, (double)(points(h, l - 1) * h->B));
-  MGWR_CK(h, mgwr::launch_restrict<R>(r, H.f[l - 1], H.u[l - 1], shape(h, l), h->stream));
+  MGWR_CK(h, mgwr::launch_restrict<R>(r, H.f[l - 1], clear ? H.u[l - 1] : (R*)nullptr, shape(h, l),
+                                       h->stream));
   prof_end(h, pm);
   H.rs[l - 1] = R_ZERO_U;
+  H.uz[l - 1] = !clear;
   return MGWR_OK;
 }
 
+// `half`: a smoothing step follows, which reads only the black points and
+// rewrites the red ones from them, so only the black points are corrected.
 template <class R>
-int prolong_into(mgwr_t h, Hier<R>& H, int l) {
+int prolong_into(mgwr_t h, Hier<R>& H, int l, bool half = false) {
   const int pm = prof_begin(h, MGWR_K_PROLONG, (double)(points(h, l) * h->B));
-  MGWR_CK(h, mgwr::launch_prolong<R>(H.u[l], H.u[l - 1], shape(h, l), h->stream));
+  const bool fresh = H.uz[l] != 0;
+  MGWR_CK(h, mgwr::launch_prolong<R>(H.u[l], H.u[l - 1], shape(h, l),
+                                      half ? parity(h, MGWR_BLACK) : -1, fresh, h->stream));
   prof_end(h, pm);
+  H.uz[l] = 0;
   H.rs[l] = R_STALE;
   return MGWR_OK;
 }
 
 // Restriction of the defect a smoothing step left (state R_DELTA) straight from
-// the black half-sweep's changes: the fine defect is never stored.
+// the black half-sweep's changes: the fine defect is never stored.  The 8-byte
+// types take the form with regrouped sums (launch_restrict_changes).
 template <class R>
-int restrict_delta_into(mgwr_t h, Hier<R>& H, int l) {
+int restrict_delta_into(mgwr_t h, Hier<R>& H, int l, bool clear = false) {
   const int pm = prof_begin(h, MGWR_K_RESTRICT, (double)(points(h, l - 1) * h->B));
-  MGWR_CK(h, mgwr::launch_restrict_delta<R>(H.dl[l], H.f[l - 1], H.u[l - 1], H.zero, shape(h, l),
-                                             parity(h, MGWR_RED), R(h->hinv2[l]), h->stream));
+  if constexpr (sizeof(R) == 4)
+    MGWR_CK(h, mgwr::launch_restrict_delta<R>(changes(H, l), H.f[l - 1],
+                                               clear ? H.u[l - 1] : (R*)nullptr, H.zero,
+                                               shape(h, l), parity(h, MGWR_RED), R(h->hinv2[l]),
+                                               h->stream));
+  else
+    MGWR_CK(h, mgwr::launch_restrict_changes<R>(changes(H, l), H.f[l - 1], H.zero, shape(h, l),
+                                                 parity(h, MGWR_RED), R(h->hinv2[l]), h->stream));
+  if (sizeof(R) == 8 && clear)
+    MGWR_CK(h, cudaMemsetAsync(H.u[l - 1], 0, level_count(h, l - 1) * sizeof(R), h->stream));
   prof_end(h, pm);
   H.rs[l - 1] = R_ZERO_U;
+  H.uz[l - 1] = !clear;
   return MGWR_OK;
 }
 
-// Algorithm 1's "compute the defect and restrict it" for level l.  The fused
-// form pays for FP32 fields (2-D 511 x 511, M = 4096: 41 -> 25 ms per solve for
-// both steps); for the 8-byte types it measured slower than the two line
-// kernels (2-D 255 x 255, M = 1024, FP64: 13.8 -> 20 ms: twice the iterations
-// per byte, and 2 blocks per SM at its register count).
+// Algorithm 1's "compute the defect and restrict it" for level l, within a cycle.
 template <class R>
 int defect_restrict(mgwr_t h, Hier<R>& H, int l) {
-  if (sizeof(R) == 4 && H.rs[l] == R_DELTA) return restrict_delta_into(h, H, l);
+  if (H.rs[l] == R_DELTA) return restrict_delta_into(h, H, l);
   const R* r = nullptr;
   MGWR_TRY(current_defect(h, H, l, &r));
-  return restrict_into(h, H, l, r);
+  return restrict_into(h, H, l, r, false);
 }
 
 // One cycle from level l.  `keep`: the post-smoothing records its changes for
@@ -640,7 +675,7 @@ int cycle(mgwr_t h, Hier<R>& H, int l, int gamma, int nu1, int nu2, bool keep = 
   MGWR_TRY(defect_restrict(h, H, l));
   for (int g = 0; g < gamma; ++g)
     MGWR_TRY(cycle(h, H, l - 1, gamma, nu1, nu2, gamma > 1 && nu1 == 0));
-  MGWR_TRY(prolong_into(h, H, l));
+  MGWR_TRY(prolong_into(h, H, l, nu2 > 0));
   MGWR_TRY(smooth(h, H, l, nu2, keep));
   return MGWR_OK;
 }
@@ -821,7 +856,7 @@ int enqueue_plain(mgwr_t h, Hier<R>& H, int cyc, int nu1, int nu2, bool* exact) 
   MGWR_TRY(cycle(h, H, L, cyc, nu1, nu2));
   MGWR_TRY(clear_norms(h));
   if (H.rs[L] == R_DELTA) {
-    MGWR_TRY(defect_from_delta(h, H, L, h->norm_bits));
+    MGWR_TRY(defect_from_delta(h, H, L, h->norm_bits, false));
     *exact = false;
   } else {
     MGWR_TRY(defect(h, H, L, h->norm_bits));
@@ -845,7 +880,7 @@ int enqueue_iteration(mgwr_t h, int cyc, int nu1, int nu2, bool* exact, bool cop
   } else if (h->precision == MGWR_DD) {
     // double-float cycles on the defect equation from e = 0, the update of the
     // double-float iterate, its double-float defect as the next right-hand side
-    MGWR_CK(h, cudaMemsetAsync(h->hdd.u[L], 0, cnt * sizeof(mgwr::dd), h->stream));
+    h->hdd.uz[L] = 1;  // e = 0: the first cycle writes it without reading it
     h->hdd.rs[L] = R_ZERO_U;
     // the next inner cycle restricts the post-smoothing's defect only without
     // pre-smoothing; after the last one the outer defect is computed in full
@@ -859,7 +894,7 @@ int enqueue_iteration(mgwr_t h, int cyc, int nu1, int nu2, bool* exact, bool cop
     *exact = true;
   } else {
     const bool ddef = h->precision == MGWR_MIXED_DD;
-    MGWR_CK(h, cudaMemsetAsync(h->h32.u[L], 0, cnt * sizeof(float), h->stream));
+    h->h32.uz[L] = 1;  // e = 0: the first cycle writes it without reading it
     h->h32.rs[L] = R_ZERO_U;  // f32 holds the outer defect, e32 = 0
     for (int k = 0; k < step_cycles(h); ++k)
       MGWR_TRY(cycle(h, h->h32, L, cyc, nu1, nu2, nu1 == 0 && k + 1 < step_cycles(h)));
@@ -1540,8 +1575,9 @@ int mgwr_get_engine_split(mgwr_t h, int kernel_class, int level, int* split) {
       kernel_class >= MGWR_NUM_KERNEL_CLASSES || level < -1 || level >= h->nlev)
     return MGWR_E_INVAL;
   const int word = kernel_class == MGWR_K_SWEEP32 || kernel_class == MGWR_K_DEFECT32 ? 4 : 8;
-  *split = mgwr::effective_split(h->M, word,
-                                 split_of(h, kernel_class, level == -1 ? h->nlev - 1 : level));
+  const int l = level == -1 ? h->nlev - 1 : level;
+  int E = split_of(h, kernel_class, l);
+  *split = mgwr::effective_split(h->M, word, E);
   return MGWR_OK;
 }
 
@@ -2488,7 +2524,7 @@ int mgwr_smooth_restrict(mgwr_t h, int hierarchy, int level) {
   if (level == 0) return fail(h, MGWR_E_INVAL, "level 0 has no coarser level");
   MGWR_TRY(with_hier(h, hierarchy, [&](auto& H) {
     MGWR_TRY(smooth(h, H, level, 1));
-    return defect_restrict(h, H, level);
+    return restrict_delta_into(h, H, level, true);
   }));
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
   return check_staging(h);
@@ -2510,7 +2546,7 @@ int mgwr_restrict(mgwr_t h, int hierarchy, int level) {
   h->u_zero = false;
   MGWR_TRY(check_level(h, hierarchy, level));
   if (level == 0) return fail(h, MGWR_E_INVAL, "level 0 has no coarser level");
-  MGWR_TRY(with_hier(h, hierarchy, [&](auto& H) { return restrict_into(h, H, level, H.r[level]); }));
+  MGWR_TRY(with_hier(h, hierarchy, [&](auto& H) { return restrict_into(h, H, level, H.r[level], true); }));
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
   return MGWR_OK;
 }

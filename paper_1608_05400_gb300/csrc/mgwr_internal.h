@@ -98,10 +98,13 @@ inline size_t long_scratch_count(const LevelShape& ls) {
 // otherwise, may be null).
 // E: butterflies per thread of the FFT engine (engine_split; the launch shape
 // only, results are identical for every E).
+// zero_u (here and in the other forms below): u is zero; its memory is not read
+// (delta null).
 template <class R>
 cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t spec_stride,
                          const Cx<R>* tw, const R* zero, Cx<R>* scratch, const LevelShape& ls,
-                         int par, bool all_points, R hinv2, int E, cudaStream_t s);
+                         int par, bool all_points, R hinv2, int E, cudaStream_t s,
+                         bool zero_u = false);
 
 // launch_sweep<float> for 64 <= M <= kShortMaxM without all_points, E carrying
 // kStaged: a persistent grid (as many CTAs as fit on the GPU) walks the line
@@ -126,7 +129,7 @@ cudaError_t take_stage_timeout(bool* hit);
 // take_tc_timeout.
 cudaError_t launch_sweep_tc(const float* f, float* u, float* delta, const unsigned char* band,
                             size_t bstride, const LevelShape& ls, int par, float hinv2,
-                            cudaStream_t s);
+                            cudaStream_t s, bool zero_u = false);
 // Bytes of one Toeplitz band: three bf16 pieces of M rows x 32 columns.
 size_t tc_band_bytes(int M);
 // band + line * tc_band_bytes(M): the band of the inverse column kcol[line]
@@ -149,7 +152,7 @@ inline bool toep_length(int M) { return M >= 64 && M <= 1024; }
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
                               size_t cstride, const unsigned char* band, size_t bstride,
                               unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
-                              cudaStream_t s);
+                              cudaStream_t s, bool zero_u = false);
 size_t toep_band_bytes(int M);
 // Bytes of scratch the launches on a level of this shape need (bounded: larger
 // fields go through it in slabs).
@@ -172,7 +175,7 @@ constexpr int kRpSingle = 1, kRpPaired = 2, kRpResident = 4;
 cudaError_t launch_sweep_rp(const float* f, float* u, float* delta, const Cx<float>* spec,
                             size_t spec_stride, const Cx<float>* tw, const float* zero,
                             const LevelShape& ls, int par, float hinv2, int form,
-                            cudaStream_t s);
+                            cudaStream_t s, bool zero_u = false);
 // dst[c L ..] = the FP64 spectra src[c L ..] (length L = 2M, the shared-memory
 // engine's order) rounded to FP32 and permuted into the register-pass engine's
 // order (the sweeps' plans, or the carried defect's when `defect`), for
@@ -182,7 +185,8 @@ cudaError_t launch_spectra_rp(Cx<float>* dst, const Cx<double>* src, size_t line
 
 // Defect after a red-black step from the black half-sweep's delta: r = 0 on the
 // black points, r = hinv2 * sum of neighbour deltas on the red points
-// (parity red_par); |r|_inf of instance b folded into norm_bits[b].
+// (parity red_par); |r|_inf of instance b folded into norm_bits[b].  r null: only
+// the norm.
 template <class R>
 cudaError_t launch_defect_from_delta(const R* delta, R* r, const R* zero, const LevelShape& ls,
                                      int red_par, R hinv2, unsigned long long* norm_bits,
@@ -202,28 +206,36 @@ cudaError_t launch_defect(const R* u, const R* f, RO* r, const Cx<R>* tspec, siz
 template <class R>
 cudaError_t launch_sweep_long(const R* f, R* u, R* delta, const Cx<R>* spec, size_t spec_stride,
                               const Cx<R>* tw, Cx<R>* scratch, const LevelShape& ls, int par,
-                              bool all_points, R hinv2, int E, cudaStream_t s);
+                              bool all_points, R hinv2, int E, cudaStream_t s, bool zero_u);
 template <class R, class RO>
 cudaError_t launch_defect_long(const R* u, const R* f, RO* r, const Cx<R>* tspec,
                                size_t spec_stride, const Cx<R>* tw, Cx<R>* scratch,
                                const LevelShape& ls, R hinv2, unsigned long long* norm_bits,
                                int E, cudaStream_t s);
 
-// fc = full weighting of r (fine n -> coarse (n-1)/2), uc = 0.
+// fc = full weighting of r (fine n -> coarse (n-1)/2), uc = 0 when given.
 template <class R>
 cudaError_t launch_restrict(const R* r, R* fc, R* uc, const LevelShape& fine, cudaStream_t s);
 
 // fc = full weighting of the defect after a red-black step, formed from the
 // black half-sweep's changes delta (as launch_defect_from_delta would write
-// it, red points of parity red_par) without storing it; uc = 0.  Bitwise the
+// it, red points of parity red_par) without storing it; uc = 0 when given.  Bitwise the
 // same fc as launch_defect_from_delta followed by launch_restrict.
 template <class R>
 cudaError_t launch_restrict_delta(const R* delta, R* fc, R* uc, const R* zero, const LevelShape& fine,
                                   int red_par, R hinv2, cudaStream_t s);
 
-// u (fine, n) += linear / bilinear interpolation of uc (coarse (n-1)/2).
+// The same restriction for the 8-byte types with the sums regrouped over the
+// changes (equal up to rounding).
 template <class R>
-cudaError_t launch_prolong(R* u, const R* uc, const LevelShape& fine, cudaStream_t s);
+cudaError_t launch_restrict_changes(const R* delta, R* fc, const R* zero, const LevelShape& fine,
+                                    int red_par, R hinv2, cudaStream_t s);
+
+// u (fine, n) += linear / bilinear interpolation of uc (coarse (n-1)/2), at the
+// points of parity par, or all for par < 0; fresh: u is zero, its memory not read.
+template <class R>
+cudaError_t launch_prolong(R* u, const R* uc, const LevelShape& fine, int par, bool fresh,
+                           cudaStream_t s);
 
 // u += (double) e, elementwise.
 cudaError_t launch_refine(double* u, const float* e, size_t count, cudaStream_t s);

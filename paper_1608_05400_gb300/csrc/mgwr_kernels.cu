@@ -90,6 +90,7 @@ __device__ __forceinline__ void block_absmax(double amax, unsigned long long* no
 // its own equation exactly, so the defect is 0 there; at a red point the
 // equation was solved with the old black neighbours, so its defect is
 // h^-2 * sum over its black neighbours of (new - old) = h^-2 sum delta.
+// r null: only the norm.
 template <class R>
 __global__ void __launch_bounds__(kLineBlock)
     k_defect_from_delta(const R* __restrict__ delta, R* __restrict__ r, const R* __restrict__ zero,
@@ -98,19 +99,21 @@ __global__ void __launch_bounds__(kLineBlock)
   constexpr int W = Vec<R>::W;
   const LineMap<R> lm(log_tpl);
   delta += blockIdx.y * fstride;
-  r += blockIdx.y * fstride;
+  const bool store = r != nullptr;
+  if (store) r += blockIdx.y * fstride;
   if (norm_bits != nullptr) norm_bits += blockIdx.y;
   double amax = 0.0;
   if (lm.line < npts) {
     const int p = lm.line;
     const int i = d == 1 ? p : p % n, j = d == 1 ? 0 : p / n;
     const int par = d == 1 ? (i & 1) : ((i + j) & 1);
-    R* rp = r + (size_t)p * M;
+    R* rp = store ? r + (size_t)p * M : nullptr;
     if (par != red_par) {
       Vec<R> z;
 #pragma unroll
       for (int k = 0; k < W; ++k) z.v[k] = R(0);
-      for (int m = lm.m0; m < M; m += lm.step) vstore(rp + m, z);
+      if (store)
+        for (int m = lm.m0; m < M; m += lm.step) vstore(rp + m, z);
     } else {
       // neighbour lines, the zero line outside the grid; four reads, three
       // additions and one product per value
@@ -134,7 +137,7 @@ __global__ void __launch_bounds__(kLineBlock)
           out.v[k] = hinv2 * sum;
           amax = absmax_nan((double)Arith<R>::mag(out.v[k]), amax);
         }
-        vstore(rp + m, out);
+        if (store) vstore(rp + m, out);
       }
     }
   }
@@ -145,7 +148,8 @@ __global__ void __launch_bounds__(kLineBlock)
 // grid transfers on whole time lines (Algorithm 1; Sec. 3 and Sec. 6)
 // ---------------------------------------------------------------------------------
 
-// Full weighting, (1/4)[1 2 1] per dimension; also clears the coarse correction.
+// Full weighting, (1/4)[1 2 1] per dimension; also clears the coarse correction
+// uc when given.
 template <class R>
 __global__ void __launch_bounds__(kLineBlock)
     k_restrict(const R* __restrict__ r, R* __restrict__ fc, R* __restrict__ uc, int d, int n, int M,
@@ -154,12 +158,13 @@ __global__ void __launch_bounds__(kLineBlock)
   const LineMap<R> lm(log_tpl);
   r += blockIdx.y * fstride;
   fc += blockIdx.y * cstride;
-  uc += blockIdx.y * cstride;
+  const bool clear = uc != nullptr;
+  if (clear) uc += blockIdx.y * cstride;
   if (lm.line >= ncpts) return;
   const int nc = (n - 1) / 2;
   const int P = lm.line;
   R* fo = fc + (size_t)P * M;
-  R* uo = uc + (size_t)P * M;
+  R* uo = clear ? uc + (size_t)P * M : nullptr;
   Vec<R> z;
 #pragma unroll
   for (int k = 0; k < W; ++k) z.v[k] = R(0);
@@ -171,7 +176,7 @@ __global__ void __launch_bounds__(kLineBlock)
 #pragma unroll
       for (int k = 0; k < W; ++k) out.v[k] = R(0.25) * (a.v[k] + R(2) * b.v[k] + e.v[k]);
       vstore(fo + m, out);
-      vstore(uo + m, z);
+      if (clear) vstore(uo + m, z);
     }
   } else {
     const int I = P % nc, J = P / nc;
@@ -198,7 +203,7 @@ __global__ void __launch_bounds__(kLineBlock)
         for (int k = 0; k < W; ++k) out.v[k] = R(0.0625) * (out.v[k] + (a.v[k] + R(2) * b.v[k] + e.v[k]));
       }
       vstore(fo + m, out);
-      vstore(uo + m, z);
+      if (clear) vstore(uo + m, z);
     }
   }
 }
@@ -216,7 +221,7 @@ __device__ __forceinline__ dd mul_rounded(dd a, dd b) { return a * b; }
 // changes) at a red one, and the stencil sums them in k_restrict's order, so
 // fc is bitwise what k_defect_from_delta followed by k_restrict gives.  Reads
 // the black changes (half a fine field, neighbours shared through L2) instead
-// of writing and reading back a whole fine defect; also clears uc.
+// of writing and reading back a whole fine defect; also clears uc when given.
 template <class R>
 __global__ void __launch_bounds__(kLineBlock)
     k_restrict_delta(const R* __restrict__ delta, R* __restrict__ fc, R* __restrict__ uc,
@@ -226,12 +231,13 @@ __global__ void __launch_bounds__(kLineBlock)
   const LineMap<R> lm(log_tpl);
   delta += blockIdx.y * fstride;
   fc += blockIdx.y * cstride;
-  uc += blockIdx.y * cstride;
+  const bool clear = uc != nullptr;
+  if (clear) uc += blockIdx.y * cstride;
   if (lm.line >= ncpts) return;
   const int nc = (n - 1) / 2;
   const int P = lm.line;
   R* fo = fc + (size_t)P * M;
-  R* uo = uc + (size_t)P * M;
+  R* uo = clear ? uc + (size_t)P * M : nullptr;
   Vec<R> z;
 #pragma unroll
   for (int k = 0; k < W; ++k) z.v[k] = R(0);
@@ -265,7 +271,7 @@ __global__ void __launch_bounds__(kLineBlock)
 #pragma unroll
       for (int k = 0; k < W; ++k) out.v[k] = R(0.25) * (a.v[k] + R(2) * b.v[k] + e.v[k]);
       vstore(fo + m, out);
-      vstore(uo + m, z);
+      if (clear) vstore(uo + m, z);
     }
   } else {
     const int ci = 2 * (P % nc) + 1, cj = 2 * (P / nc) + 1;
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(kLineBlock)
         for (int k = 0; k < W; ++k) out.v[k] = R(0.0625) * (out.v[k] + (a.v[k] + R(2) * b.v[k] + e.v[k]));
       }
       vstore(fo + m, out);
-      vstore(uo + m, z);
+      if (clear) vstore(uo + m, z);
     }
   }
 }
@@ -309,7 +315,8 @@ __global__ void __launch_bounds__(kLineBlock)
   constexpr int W = Vec<R>::W;
   delta += blockIdx.y * fstride;
   fc += blockIdx.y * cstride;
-  uc += blockIdx.y * cstride;
+  const bool clear = uc != nullptr;
+  if (clear) uc += blockIdx.y * cstride;
   const int nc = (n - 1) / 2;
   const int MV = M / W;                        // time vectors per line
   const int runs = (nc + kRowRun - 1) / kRowRun;  // walks per coarse row
@@ -359,10 +366,107 @@ __global__ void __launch_bounds__(kLineBlock)
         out.v[k] = R(0.0625) * (out.v[k] + (l2.v[k] + R(2) * c2.v[k] + q2.v[k]));
       const size_t P = (size_t)row * nc + p;
       vstore(fc + P * M + m, out);
-      vstore(uc + P * M + m, z);
+      if (clear) vstore(uc + P * M + m, z);
       l0 = q0;
       l1 = q1;
       l2 = q2;
+    }
+  }
+}
+
+// The same restriction with its sums regrouped over the black changes, for the
+// 8-byte types, whose additions bound it (FP64: two a clock and SM; double-float:
+// about 20 FP32 operations each).  With red points at even i + j, the coarse
+// point at fine (i, j) takes
+//   h^-2 / 16 (6 V(i) + V(i-2) + V(i+2) + H(i-1) + H(i+1)),
+//   V(x) = delta(x, j-1) + delta(x, j+1),
+//   H(x) = 6 delta(x, j) + delta(x, j-2) + delta(x, j+2):
+// walking a coarse row, five loads and nine operations per coarse value, where
+// the fine defects and their stencil take about 30 operations in two passes over
+// the field.  2-D 255 x 255, M = 1024, FP64 solve: defects and restrictions 20.4 ->
+// 12.0 ms, 6.5 of them the norms of the twelve convergence checks.  In 1-D: half the sum of the two changes beside a red coarse
+// point, or a quarter of [1 2 1] at a black one (both colour orders occur).
+template <class R>
+__global__ void __launch_bounds__(kLineBlock)
+    k_restrict_changes(const R* __restrict__ delta, R* __restrict__ fc, const R* __restrict__ zero,
+                       int d, int n, int M, int red_par, R hinv2, size_t fstride,
+                       size_t cstride) {
+  constexpr int W = Vec<R>::W;
+  delta += blockIdx.y * fstride;
+  fc += blockIdx.y * cstride;
+  const int nc = (n - 1) / 2;
+  const int MV = M / W;
+  if (d == 1) {
+    const size_t items = (size_t)nc * MV;
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < items;
+         x += (size_t)gridDim.x * blockDim.x) {
+      const int m = (int)(x % MV) * W;
+      const int P = (int)(x / MV), i = 2 * P + 1;
+      Vec<R> out;
+      if (red_par == 1) {
+        const Vec<R> a = vload(delta + (size_t)(i - 1) * M + m), b = vload(delta + (size_t)(i + 1) * M + m);
+        const R w = R(0.5) * hinv2;
+#pragma unroll
+        for (int k = 0; k < W; ++k) out.v[k] = w * (a.v[k] + b.v[k]);
+      } else {
+        const Vec<R> a = vload((i > 1 ? delta + (size_t)(i - 2) * M : zero) + m),
+                     b = vload(delta + (size_t)i * M + m),
+                     e = vload((i + 2 < n ? delta + (size_t)(i + 2) * M : zero) + m);
+        const R w = R(0.25) * hinv2;
+#pragma unroll
+        for (int k = 0; k < W; ++k) out.v[k] = w * (a.v[k] + R(2) * b.v[k] + e.v[k]);
+      }
+      vstore(fc + (size_t)P * M + m, out);
+    }
+    return;
+  }
+  const int runs = (nc + kRowRun - 1) / kRowRun;
+  const size_t items = (size_t)nc * runs * MV;
+  const R w = R(0.0625) * hinv2;
+  for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < items;
+       x += (size_t)gridDim.x * blockDim.x) {
+    const int m = (int)(x % MV) * W;
+    const size_t rest = x / MV;
+    const int run = (int)(rest % runs);
+    const int row = (int)(rest / runs);
+    const int j = 2 * row + 1;
+    const int p0 = run * kRowRun;
+    const int p1 = p0 + kRowRun < nc ? p0 + kRowRun : nc;
+    const size_t nM = (size_t)n * M;
+    auto at = [&](int i, int jj) { return delta + ((size_t)i + (size_t)jj * n) * M + m; };
+    auto V = [&](int i) -> Vec<R> {  // odd i
+      Vec<R> v;
+      if (i < 0 || i >= n) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) v.v[k] = R(0);
+        return v;
+      }
+      const R* c = at(i, j - 1);
+      const Vec<R> a = vload(c), b = vload(c + 2 * nM);
+#pragma unroll
+      for (int k = 0; k < W; ++k) v.v[k] = a.v[k] + b.v[k];
+      return v;
+    };
+    auto H = [&](int i) -> Vec<R> {  // even i, 0 .. n - 1
+      const Vec<R> c = vload(at(i, j));
+      const Vec<R> a = vload(j > 1 ? at(i, j - 2) : zero + m), b = vload(j + 2 < n ? at(i, j + 2) : zero + m);
+      Vec<R> v;
+#pragma unroll
+      for (int k = 0; k < W; ++k) v.v[k] = R(6) * c.v[k] + (a.v[k] + b.v[k]);
+      return v;
+    };
+    Vec<R> vl = V(2 * p0 - 1), vc = V(2 * p0 + 1), hl = H(2 * p0);
+    for (int p = p0; p < p1; ++p) {
+      const int i = 2 * p + 1;
+      const Vec<R> vr = V(i + 2), hr = H(i + 1);
+      Vec<R> out;
+#pragma unroll
+      for (int k = 0; k < W; ++k)
+        out.v[k] = w * (R(6) * vc.v[k] + ((vl.v[k] + vr.v[k]) + (hl.v[k] + hr.v[k])));
+      vstore(fc + ((size_t)row * nc + p) * M + m, out);
+      vl = vc;
+      vc = vr;
+      hl = hr;
     }
   }
 }
@@ -395,20 +499,30 @@ struct Taps {
   }
 };
 
+// Interpolation and correction.  par >= 0: the points of that parity alone (a
+// smoothing step that follows overwrites the other colour from these, so its
+// correction would never be read); npts counts the points.  fresh: u is zero (its
+// memory not read).
 template <class R>
 __global__ void __launch_bounds__(kLineBlock)
     k_prolong(R* __restrict__ u, const R* __restrict__ uc, int d, int n, int M, int log_tpl,
-              int npts, size_t fstride, size_t cstride) {
+              int npts, int par, bool fresh, size_t fstride, size_t cstride) {
   constexpr int W = Vec<R>::W;
   const LineMap<R> lm(log_tpl);
   u += blockIdx.y * fstride;
   uc += blockIdx.y * cstride;
   if (lm.line >= npts) return;
   const int nc = (n - 1) / 2;
-  const int p = lm.line;
+  int pi = 0, pj = 0, p = lm.line;
+  if (par >= 0) {
+    p = colour_point(lm.line, d, n, par, pi, pj);
+  } else {
+    pi = d == 1 ? p : p % n;
+    pj = d == 1 ? 0 : p / n;
+  }
   R* up = u + (size_t)p * M;
-  const Taps tx(d == 1 ? p : p % n, nc);
-  const Taps ty(d == 1 ? 1 : p / n, nc);  // 1-D: a single tap of weight 1 in y
+  const Taps tx(pi, nc);
+  const Taps ty(d == 1 ? 1 : pj, nc);  // 1-D: a single tap of weight 1 in y
   const size_t row0 = d == 1 ? 0 : (size_t)ty.i0 * nc, row1 = d == 1 ? 0 : (size_t)ty.i1 * nc;
   const R* a = uc + ((size_t)tx.i0 + row0) * M;
   const R* b = uc + ((size_t)tx.i1 + row0) * M;
@@ -430,9 +544,15 @@ __global__ void __launch_bounds__(kLineBlock)
 #pragma unroll
       for (int k = 0; k < W; ++k) sum.v[k] = sum.v[k] + vs.v[k];
     }
-    Vec<R> cur = vload_rw(up + m);
+    Vec<R> cur;
+    if (fresh) {
 #pragma unroll
-    for (int k = 0; k < W; ++k) cur.v[k] = unit ? cur.v[k] + sum.v[k] : cur.v[k] + w * sum.v[k];
+      for (int k = 0; k < W; ++k) cur.v[k] = unit ? sum.v[k] : w * sum.v[k];
+    } else {
+      cur = vload_rw(up + m);
+#pragma unroll
+      for (int k = 0; k < W; ++k) cur.v[k] = unit ? cur.v[k] + sum.v[k] : cur.v[k] + w * sum.v[k];
+    }
     vstore(up + m, cur);
   }
 }
@@ -447,8 +567,8 @@ constexpr int kProlongRun = 16;
 
 template <class R>
 __global__ void __launch_bounds__(kLineBlock)
-    k_prolong_rows(R* __restrict__ u, const R* __restrict__ uc, int n, int M, size_t fstride,
-                   size_t cstride) {
+    k_prolong_rows(R* __restrict__ u, const R* __restrict__ uc, int n, int M, int par, bool fresh,
+                   size_t fstride, size_t cstride) {
   constexpr int W = Vec<R>::W;
   u += blockIdx.y * fstride;
   uc += blockIdx.y * cstride;
@@ -490,7 +610,9 @@ __global__ void __launch_bounds__(kLineBlock)
       v1 = b1;
     };
     const int i_end = (run + 1) * kProlongRun < n ? (run + 1) * kProlongRun : n;
-    for (int i = run * kProlongRun; i < i_end; ++i) {
+    // the points of parity par (kProlongRun is even), or all
+    const int i_step = par >= 0 ? 2 : 1;
+    for (int i = run * kProlongRun + (par >= 0 ? (par ^ j) & 1 : 0); i < i_end; i += i_step) {
       const Taps tx(i, nc);
       Vec<R> l0, l1, r0, r1;
       column(tx.i0, l0, l1);  // a, c
@@ -508,9 +630,15 @@ __global__ void __launch_bounds__(kLineBlock)
       const bool unit = !tx.half && !ty.half;
       const R w = R((tx.half ? 0.5 : 1.0) * (ty.half ? 0.5 : 1.0));
       R* up = u + ((size_t)i + (size_t)j * n) * M + m;
-      Vec<R> cur = vload_rw(up);
+      Vec<R> cur;
+      if (fresh) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) cur.v[k] = unit ? cur.v[k] + sum.v[k] : cur.v[k] + w * sum.v[k];
+        for (int k = 0; k < W; ++k) cur.v[k] = unit ? sum.v[k] : w * sum.v[k];
+      } else {
+        cur = vload_rw(up);
+#pragma unroll
+        for (int k = 0; k < W; ++k) cur.v[k] = unit ? cur.v[k] + sum.v[k] : cur.v[k] + w * sum.v[k];
+      }
       vstore(up, cur);
     }
   }
@@ -873,8 +1001,22 @@ cudaError_t launch_restrict_delta(const R* delta, R* fc, R* uc, const R* zero, c
 }
 
 template <class R>
-cudaError_t launch_prolong(R* u, const R* uc, const LevelShape& ls, cudaStream_t s) {
-  const int npts = ls.d == 1 ? ls.n : ls.n * ls.n;
+cudaError_t launch_restrict_changes(const R* delta, R* fc, const R* zero, const LevelShape& ls,
+                                    int red_par, R hinv2, cudaStream_t s) {
+  const int nc = (ls.n - 1) / 2;
+  const int ncpts = ls.d == 1 ? nc : nc * nc;
+  if (ncpts == 0 || ls.batch == 0) return cudaSuccess;
+  const size_t items = (size_t)nc * (ls.d == 1 ? 1 : (nc + kRowRun - 1) / kRowRun) *
+                       (ls.M / Vec<R>::W);
+  k_restrict_changes<R><<<dim3(elementwise_grid(items), ls.batch), kLineBlock, 0, s>>>(
+      delta, fc, zero, ls.d, ls.n, ls.M, red_par, hinv2, ls.field_stride(), (size_t)ncpts * ls.M);
+  return counted(cudaGetLastError());
+}
+
+template <class R>
+cudaError_t launch_prolong(R* u, const R* uc, const LevelShape& ls, int par, bool fresh,
+                           cudaStream_t s) {
+  const int npts = par >= 0 ? colour_count(ls.d, ls.n, par) : ls.d == 1 ? ls.n : ls.n * ls.n;
   const int nc = (ls.n - 1) / 2;
   const size_t cstride = (size_t)(ls.d == 1 ? nc : nc * nc) * ls.M;
   if (ls.batch == 0) return cudaSuccess;
@@ -886,14 +1028,14 @@ cudaError_t launch_prolong(R* u, const R* uc, const LevelShape& ls, cudaStream_t
     const size_t items =
         (size_t)ls.n * ((ls.n + kProlongRun - 1) / kProlongRun) * (ls.M / Vec<R>::W);
     k_prolong_rows<R><<<dim3(elementwise_grid(items), ls.batch), kLineBlock, 0, s>>>(
-        u, uc, ls.n, ls.M, ls.field_stride(), cstride);
+        u, uc, ls.n, ls.M, par, fresh, ls.field_stride(), cstride);
     return counted(cudaGetLastError());
   }
   int log_tpl;
   unsigned blocks;
   line_grid<R>(ls.M, npts, &log_tpl, &blocks);
-  k_prolong<R><<<dim3(blocks, ls.batch), kLineBlock, 0, s>>>(u, uc, ls.d, ls.n, ls.M, log_tpl, npts,
-                                                      ls.field_stride(), cstride);
+  k_prolong<R><<<dim3(blocks, ls.batch), kLineBlock, 0, s>>>(
+      u, uc, ls.d, ls.n, ls.M, log_tpl, npts, par, fresh, ls.field_stride(), cstride);
   return counted(cudaGetLastError());
 }
 
@@ -1056,13 +1198,18 @@ cudaError_t launch_round_cx(Cx<float>* dst, const Cx<double>* src, size_t count,
   template cudaError_t launch_defect_from_delta<R>(const R*, R*, const R*, const LevelShape&,  \
                                                    int, R, unsigned long long*, cudaStream_t); \
   template cudaError_t launch_restrict<R>(const R*, R*, R*, const LevelShape&, cudaStream_t);  \
-  template cudaError_t launch_prolong<R>(R*, const R*, const LevelShape&, cudaStream_t);     \
+  template cudaError_t launch_prolong<R>(R*, const R*, const LevelShape&, int, bool,         \
+                                         cudaStream_t);                                      \
   template cudaError_t launch_restrict_delta<R>(const R*, R*, R*, const R*, const LevelShape&, \
                                                 int, R, cudaStream_t);
 MGWR_INST_R(double)
 MGWR_INST_R(float)
 MGWR_INST_R(dd)
 #undef MGWR_INST_R
+template cudaError_t launch_restrict_changes<double>(const double*, double*, const double*,
+                                                     const LevelShape&, int, double, cudaStream_t);
+template cudaError_t launch_restrict_changes<dd>(const dd*, dd*, const dd*, const LevelShape&, int,
+                                                 dd, cudaStream_t);
 
 
 }  // namespace mgwr

@@ -60,7 +60,7 @@ template <class R, int MODE, int E>
 __global__ void __launch_bounds__(long_threads<E>(), 1)
     k_long_forward(const R* __restrict__ f, const R* __restrict__ u, Cx<R>* __restrict__ scratch,
                    const Cx<R>* __restrict__ tw, int d, int n, int M, int P, int par,
-                   int all_points, R hinv2, int npts, int npairs, size_t fstride) {
+                   int all_points, bool zero_u, R hinv2, int npts, int npairs, size_t fstride) {
   extern __shared__ unsigned char smem_raw[];
   const int pair = blockIdx.x / P, j = blockIdx.x - pair * P, inst = blockIdx.y;
   f += inst * fstride;
@@ -81,10 +81,10 @@ __global__ void __launch_bounds__(long_threads<E>(), 1)
     Cx<R> x{R(0), R(0)};
     if constexpr (MODE == 0) {
       x.x = f[pAM + m];
-      if (!all_points) x.x = x.x + hinv2 * neighbour_sum(u, d, n, iA, jA, pAM, M, m);
+      if (!all_points && !zero_u) x.x = x.x + hinv2 * neighbour_sum(u, d, n, iA, jA, pAM, M, m);
       if (hasB) {
         x.y = f[pBM + m];
-        if (!all_points) x.y = x.y + hinv2 * neighbour_sum(u, d, n, iB, jB, pBM, M, m);
+        if (!all_points && !zero_u) x.y = x.y + hinv2 * neighbour_sum(u, d, n, iB, jB, pBM, M, m);
       }
     } else {
       x.x = u[pAM + m];
@@ -232,11 +232,11 @@ template <class R, int E>
 cudaError_t sweep_long_launch(dim3 grid, size_t smem, cudaStream_t s, const R* f, R* u, R* delta,
                               const Cx<R>* spec, size_t spec_stride, const Cx<R>* tw,
                               Cx<R>* scratch, int d, int n, int M, int P, int par, int all_points,
-                              R hinv2, int npts, int npairs, size_t fstride) {
+                              bool zero_u, R hinv2, int npts, int npairs, size_t fstride) {
   cudaError_t e = prepare_smem(k_long_forward<R, 0, E>, smem);
   if (e != cudaSuccess) return e;
   k_long_forward<R, 0, E><<<grid, long_threads<E>(), smem, s>>>(
-      f, u, scratch, tw, d, n, M, P, par, all_points, hinv2, npts, npairs, fstride);
+      f, u, scratch, tw, d, n, M, P, par, all_points, zero_u, hinv2, npts, npairs, fstride);
   e = counted(cudaGetLastError());
   if (e != cudaSuccess) return e;
   e = prepare_smem(k_long_inverse<R, R, 0, E>, smem);
@@ -250,7 +250,7 @@ cudaError_t sweep_long_launch(dim3 grid, size_t smem, cudaStream_t s, const R* f
 template <class R>
 cudaError_t launch_sweep_long(const R* f, R* u, R* delta, const Cx<R>* spec, size_t spec_stride,
                               const Cx<R>* tw, Cx<R>* scratch, const LevelShape& ls, int par,
-                              bool all_points, R hinv2, int E, cudaStream_t s) {
+                              bool all_points, R hinv2, int E, cudaStream_t s, bool zero_u) {
   const int d = ls.d, n = ls.n, M = ls.M, P = M / kLongB;
   const int npts = all_points ? (d == 1 ? n : n * n) : colour_count(d, n, par);
   const int npairs = (npts + 1) / 2;
@@ -261,9 +261,10 @@ cudaError_t launch_sweep_long(const R* f, R* u, R* delta, const Cx<R>* spec, siz
   const size_t fstride = ls.field_stride();
   if (effective_split(M, 8, E) == 2)
     return sweep_long_launch<R, 2>(grid, smem, s, f, u, delta, spec, spec_stride, tw, scratch, d,
-                                   n, M, P, par, all_points ? 1 : 0, hinv2, npts, npairs, fstride);
+                                   n, M, P, par, all_points ? 1 : 0, zero_u, hinv2, npts, npairs,
+                                   fstride);
   return sweep_long_launch<R, 1>(grid, smem, s, f, u, delta, spec, spec_stride, tw, scratch, d, n,
-                                 M, P, par, all_points ? 1 : 0, hinv2, npts, npairs, fstride);
+                                 M, P, par, all_points ? 1 : 0, zero_u, hinv2, npts, npairs, fstride);
 }
 
 template <class R, class RO, int E>
@@ -274,7 +275,7 @@ cudaError_t defect_long_launch(dim3 grid, size_t smem, cudaStream_t s, const R* 
   cudaError_t e = prepare_smem(k_long_forward<R, 1, E>, smem);
   if (e != cudaSuccess) return e;
   k_long_forward<R, 1, E><<<grid, long_threads<E>(), smem, s>>>(
-      f, u, scratch, tw, d, n, M, P, 0, 1, hinv2, npts, npairs, fstride);
+      f, u, scratch, tw, d, n, M, P, 0, 1, false, hinv2, npts, npairs, fstride);
   e = counted(cudaGetLastError());
   if (e != cudaSuccess) return e;
   e = prepare_smem(k_long_inverse<R, RO, 1, E>, smem);
@@ -320,14 +321,14 @@ cudaError_t launch_spectra_long(Cx<double>* spec, const double* lines, int count
 template cudaError_t launch_sweep_long<double>(const double*, double*, double*, const Cx<double>*,
                                                size_t, const Cx<double>*, Cx<double>*,
                                                const LevelShape&, int, bool, double, int,
-                                               cudaStream_t);
+                                               cudaStream_t, bool);
 template cudaError_t launch_sweep_long<dd>(const dd*, dd*, dd*, const Cx<dd>*, size_t,
                                            const Cx<dd>*, Cx<dd>*, const LevelShape&, int, bool,
-                                           dd, int, cudaStream_t);
+                                           dd, int, cudaStream_t, bool);
 template cudaError_t launch_sweep_long<float>(const float*, float*, float*, const Cx<float>*,
                                               size_t, const Cx<float>*, Cx<float>*,
                                               const LevelShape&, int, bool, float, int,
-                                              cudaStream_t);
+                                              cudaStream_t, bool);
 #define MGWR_INST_LONG_DEFECT(R, RO)                                                          \
   template cudaError_t launch_defect_long<R, RO>(const R*, const R*, RO*, const Cx<R>*,        \
                                                  size_t, const Cx<R>*, Cx<R>*,                 \

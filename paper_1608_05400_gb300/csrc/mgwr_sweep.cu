@@ -12,7 +12,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<R>(BLOCK, E))
     k_sweep(const R* __restrict__ f, R* __restrict__ u, R* __restrict__ delta,
             const Cx<R>* __restrict__ spec, const Cx<R>* __restrict__ tw,
             const R* __restrict__ zero, int d, int n, int M, int logL, int par, int all_points,
-            R hinv2, int npts, int npairs, size_t fstride, size_t sstride) {
+            bool zero_u, R hinv2, int npts, int npairs, size_t fstride, size_t sstride) {
   extern __shared__ unsigned char smem_raw[];
   // instance of a batch: blockIdx.y
   f += blockIdx.y * fstride;
@@ -51,8 +51,8 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<R>(BLOCK, E))
   if constexpr (sizeof(R) == 4) {
     neighbour_lines(u, zero, d, n, iA, jA, pAM, M, qA);
     neighbour_lines(u, zero, d, n, iB, jB, pBM, M, qB);
-    if (!valid || all_points) qA[0] = qA[1] = qA[2] = qA[3] = zero;
-    if (!hasB || all_points) qB[0] = qB[1] = qB[2] = qB[3] = zero;
+    if (!valid || all_points || zero_u) qA[0] = qA[1] = qA[2] = qA[3] = zero;
+    if (!hasB || all_points || zero_u) qB[0] = qB[1] = qB[2] = qB[3] = zero;
   }
 
   auto load = [&](int m) -> Cx<R> {
@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<R>(BLOCK, E))
       return Cx<R>{fA[m] + hinv2 * (qA[0][m] + qA[1][m]), fB[m] + hinv2 * (qB[0][m] + qB[1][m])};
     } else {  // bounds tested per access: fewer live registers
       Cx<R> b{fA[m], fB[m]};
-      if (valid && !all_points) b.x = b.x + hinv2 * neighbour_sum(u, d, n, iA, jA, pAM, M, m);
-      if (hasB && !all_points) b.y = b.y + hinv2 * neighbour_sum(u, d, n, iB, jB, pBM, M, m);
+      if (valid && !all_points && !zero_u) b.x = b.x + hinv2 * neighbour_sum(u, d, n, iA, jA, pAM, M, m);
+      if (hasB && !all_points && !zero_u) b.y = b.y + hinv2 * neighbour_sum(u, d, n, iB, jB, pBM, M, m);
       return b;
     }
   };
@@ -94,28 +94,29 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<R>(BLOCK, E))
 template <class R, int BLOCK, class SH, int E>
 cudaError_t sweep_launch(dim3 grid, size_t smem, cudaStream_t s, const R* f, R* u, R* delta,
                          const Cx<R>* spec, const Cx<R>* tw, const R* zero, int d, int n, int M,
-                         int logL, int par, bool all_points, R hinv2, int npts, int npairs,
+                         int logL, int par, bool all_points, bool zero_u, R hinv2, int npts, int npairs,
                          size_t fstride, size_t sstride) {
   cudaError_t e = prepare_smem(k_sweep<R, BLOCK, SH, E>, smem);
   if (e != cudaSuccess) return e;
   k_sweep<R, BLOCK, SH, E><<<grid, BLOCK, smem, s>>>(f, u, delta, spec, tw, zero, d, n, M, logL,
-                                                     par, all_points, hinv2, npts, npairs, fstride,
-                                                     sstride);
+                                                     par, all_points, zero_u, hinv2, npts, npairs,
+                                                     fstride, sstride);
   return cudaSuccess;
 }
 
 template <class R>
 cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t spec_stride,
                          const Cx<R>* tw, const R* zero, Cx<R>* scratch, const LevelShape& ls,
-                         int par, bool all_points, R hinv2, int E, cudaStream_t s) {
+                         int par, bool all_points, R hinv2, int E, cudaStream_t s,
+                         bool zero_u) {
   if (ls.M > kShortMaxM)
     return launch_sweep_long(f, u, delta, spec, spec_stride, tw, scratch, ls, par, all_points,
-                             hinv2, E, s);
+                             hinv2, E, s, zero_u);
   const int d = ls.d, n = ls.n, M = ls.M;
   const int L = 2 * M, logL = ilog2(L);
   E = effective_split(M, (int)sizeof(R) == 4 ? 4 : 8, E);
   if constexpr (sizeof(R) == 4) {
-    if ((E & kStaged) && !all_points)
+    if ((E & kStaged) && !all_points && !zero_u)
       return launch_sweep_staged(f, u, delta, spec, spec_stride, tw, zero, ls, par, hinv2, E, s);
   }
   E &= ~(kStaged | kTensor | kRadix);
@@ -133,7 +134,7 @@ cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t s
   const dim3 grid((unsigned)((npairs + groups - 1) / groups), (unsigned)ls.batch);
   cudaError_t e = cudaErrorInvalidValue;
 #define MGWR_SWEEP_ARGS                                                                     \
-  grid, smem, s, f, u, delta, spec, tw, zero, d, n, M, logL, par, all_points, hinv2, npts, \
+  grid, smem, s, f, u, delta, spec, tw, zero, d, n, M, logL, par, all_points, zero_u, hinv2, npts, \
       npairs, fstride, spec_stride
   if constexpr (sizeof(R) == 4) {
     switch (logL * 8 + E) {
@@ -171,13 +172,13 @@ cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t s
 
 template cudaError_t launch_sweep<double>(const double*, double*, double*, const Cx<double>*,
                                           size_t, const Cx<double>*, const double*, Cx<double>*,
-                                          const LevelShape&, int, bool, double, int, cudaStream_t);
+                                          const LevelShape&, int, bool, double, int, cudaStream_t, bool);
 template cudaError_t launch_sweep<float>(const float*, float*, float*, const Cx<float>*, size_t,
                                          const Cx<float>*, const float*, Cx<float>*,
-                                         const LevelShape&, int, bool, float, int, cudaStream_t);
+                                         const LevelShape&, int, bool, float, int, cudaStream_t, bool);
 
 template cudaError_t launch_sweep<dd>(const dd*, dd*, dd*, const Cx<dd>*, size_t, const Cx<dd>*,
                                       const dd*, Cx<dd>*, const LevelShape&, int, bool, dd, int,
-                                      cudaStream_t);
+                                      cudaStream_t, bool);
 
 }  // namespace mgwr

@@ -7,10 +7,12 @@ namespace mgwr {
 
 namespace {
 
+// ZERO: u is zero and not read: b = f (a build of its own: as a run-time branch
+// the choice slowed every 256-step half-sweep by a third).
 // PAIRED: the first pass takes adjacent butterflies two at a time, with 8-byte
 // gathers and stores (rp::convolve2), else one at a time (rp::convolve); the
 // tuner picks per level (faster for 256-step lines, slower for 1024 and 4096).
-template <int LOGL, int R0, int R1, int R2, int R3, int T, bool PAIRED>
+template <int LOGL, int R0, int R1, int R2, int R3, int T, bool PAIRED, bool ZERO>
 __global__ void __launch_bounds__(kRpBlock, (rp::Plan<LOGL, R0, R1, R2, R3, T>::MIN_BLOCKS))
     k_sweep_rp(const float* __restrict__ f, float* __restrict__ u, float* __restrict__ delta,
                const Cx<float>* __restrict__ spec, const Cx<float>* __restrict__ tw,
@@ -48,6 +50,7 @@ __global__ void __launch_bounds__(kRpBlock, (rp::Plan<LOGL, R0, R1, R2, R3, T>::
 
   if constexpr (!PAIRED) {
     auto load = [&](int m) -> C {
+      if constexpr (ZERO) return C{fA[m], fB[m]};
       if (d == 2)
         return C{fA[m] + hinv2 * ((qA[0][m] + qA[1][m]) + (qA[2][m] + qA[3][m])),
                  fB[m] + hinv2 * ((qB[0][m] + qB[1][m]) + (qB[2][m] + qB[3][m]))};
@@ -73,6 +76,7 @@ __global__ void __launch_bounds__(kRpBlock, (rp::Plan<LOGL, R0, R1, R2, R3, T>::
   auto ld2 = [](const float* p, int m) { return *reinterpret_cast<const float2*>(p + m); };
   auto load2 = [&](int m) -> rp::Pair2 {
     const float2 a = ld2(fA, m), b = ld2(fB, m);
+    if constexpr (ZERO) return rp::Pair2{C{a.x, b.x}, C{a.y, b.y}};
     const float2 a0 = ld2(qA[0], m), a1 = ld2(qA[1], m), b0 = ld2(qB[0], m), b1 = ld2(qB[1], m);
     float2 sa{a0.x + a1.x, a0.y + a1.y}, sb{b0.x + b1.x, b0.y + b1.y};
     if (d == 2) {
@@ -119,7 +123,7 @@ __global__ void __launch_bounds__(kRpBlock, (rp::Plan<LOGL, R0, R1, R2, R3, T>::
 // loaded once; the black half-sweep loads the old values of a butterfly's
 // outputs before its first store.  The same arithmetic as the
 // paired k_sweep_rp: bitwise the same results.
-template <int LOGL, int R0, int R1, int R2, int R3, int T>
+template <int LOGL, int R0, int R1, int R2, int R3, int T, bool ZERO>
 __global__ void __launch_bounds__(kRpResBlock, 1)
     k_sweep_rp_res(const float* __restrict__ f, float* __restrict__ u, float* __restrict__ delta,
                    const Cx<float>* __restrict__ spec, const Cx<float>* __restrict__ tw,
@@ -167,6 +171,7 @@ __global__ void __launch_bounds__(kRpResBlock, 1)
     const bool shared = qB[0] == qA[1] && hasB;
     auto load2 = [&](int m) -> rp::Pair2 {
       const float2 a = ld2(fA, m), b = ld2(fB, m);
+      if constexpr (ZERO) return rp::Pair2{C{a.x, b.x}, C{a.y, b.y}};
       const float2 a0 = ld2(qA[0], m), a1 = ld2(qA[1], m), b1 = ld2(qB[1], m);
       const float2 b0 = shared ? a1 : ld2(qB[0], m);
       float2 sa{a0.x + a1.x, a0.y + a1.y}, sb{b0.x + b1.x, b0.y + b1.y};
@@ -238,14 +243,16 @@ __global__ void k_spectra_rp(Cx<float>* __restrict__ dst, const Cx<double>* __re
 template <int LOGL, int R0, int R1, int R2, int R3, int T, bool PAIRED>
 cudaError_t sweep_rp_launch(dim3 grid, cudaStream_t s, const float* f, float* u, float* delta,
                             const Cx<float>* spec, const Cx<float>* tw, const float* zero, int d,
-                            int n, int M, int par, float hinv2, int npts, int npairs,
+                            int n, int M, int par, bool zero_u, float hinv2, int npts, int npairs,
                             size_t fstride, size_t sstride) {
   using P = rp::Plan<LOGL, R0, R1, R2, R3, T>;
   const size_t smem = (size_t)(kRpBlock / T) * P::SMEM * sizeof(Cx<float>);
-  cudaError_t e = prepare_smem(k_sweep_rp<LOGL, R0, R1, R2, R3, T, PAIRED>, smem);
+  const auto kern = zero_u ? k_sweep_rp<LOGL, R0, R1, R2, R3, T, PAIRED, true>
+                           : k_sweep_rp<LOGL, R0, R1, R2, R3, T, PAIRED, false>;
+  cudaError_t e = prepare_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  k_sweep_rp<LOGL, R0, R1, R2, R3, T, PAIRED><<<grid, kRpBlock, smem, s>>>(
-      f, u, delta, spec, tw, zero, d, n, M, par, hinv2, npts, npairs, fstride, sstride);
+  kern<<<grid, kRpBlock, smem, s>>>(f, u, delta, spec, tw, zero, d, n, M, par, hinv2, npts, npairs,
+                                    fstride, sstride);
   return cudaSuccess;
 }
 
@@ -255,21 +262,23 @@ cudaError_t sweep_rp_launch(dim3 grid, cudaStream_t s, const float* f, float* u,
 template <int LOGL, int R0, int R1, int R2, int R3, int T>
 cudaError_t sweep_rp_res_launch(int batch, cudaStream_t s, const float* f, float* u, float* delta,
                                 const Cx<float>* spec, const Cx<float>* tw, const float* zero,
-                                int d, int n, int M, int par, float hinv2, int npts, int npairs,
-                                size_t fstride, size_t sstride) {
+                                int d, int n, int M, int par, bool zero_u, float hinv2, int npts,
+                                int npairs, size_t fstride, size_t sstride) {
   using P = rp::Plan<LOGL, R0, R1, R2, R3, T>;
   using TB = rp::SharedTables<LOGL, R0, R1, R2, R3>;
   constexpr int PAIRS = kRpResBlock / T;
   constexpr size_t smem = (size_t)PAIRS * P::SMEM * sizeof(Cx<float>) + TB::BYTES;
   static_assert(smem <= 227 * 1024, "resident sweep exceeds the shared memory of a block");
-  cudaError_t e = prepare_smem(k_sweep_rp_res<LOGL, R0, R1, R2, R3, T>, smem);
+  const auto kern = zero_u ? k_sweep_rp_res<LOGL, R0, R1, R2, R3, T, true>
+                           : k_sweep_rp_res<LOGL, R0, R1, R2, R3, T, false>;
+  cudaError_t e = prepare_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const int need = (npairs + PAIRS - 1) / PAIRS;
   int per = sm_count() / batch;
   if (per < 1) per = 1;
   const dim3 grid((unsigned)(need < per ? need : per), (unsigned)batch);
-  k_sweep_rp_res<LOGL, R0, R1, R2, R3, T><<<grid, kRpResBlock, smem, s>>>(
-      f, u, delta, spec, tw, zero, d, n, M, par, hinv2, npts, npairs, fstride, sstride);
+  kern<<<grid, kRpResBlock, smem, s>>>(f, u, delta, spec, tw, zero, d, n, M, par, hinv2, npts,
+                                       npairs, fstride, sstride);
   return cudaSuccess;
 }
 
@@ -278,7 +287,7 @@ cudaError_t sweep_rp_res_launch(int batch, cudaStream_t s, const float* f, float
 cudaError_t launch_sweep_rp(const float* f, float* u, float* delta, const Cx<float>* spec,
                             size_t spec_stride, const Cx<float>* tw, const float* zero,
                             const LevelShape& ls, int par, float hinv2, int form,
-                            cudaStream_t s) {
+                            cudaStream_t s, bool zero_u) {
   const int d = ls.d, n = ls.n, M = ls.M;
   if (!radix_length(M)) return cudaErrorInvalidValue;
   const int logL = ilog2(2 * M);
@@ -293,15 +302,15 @@ cudaError_t launch_sweep_rp(const float* f, float* u, float* delta, const Cx<flo
     const dim3 grid((unsigned)((npairs + kRpBlock / T - 1) / (kRpBlock / T)), (unsigned)ls.batch); \
     if (form == kRpResident)                                                                 \
       e = sweep_rp_res_launch<LG, A, B, C, D, T>(ls.batch, s, f, u, delta, spec, tw, zero, d, \
-                                                 n, M, par, hinv2, npts, npairs, fstride,    \
+                                                 n, M, par, zero_u, hinv2, npts, npairs, fstride, \
                                                  spec_stride);                               \
     else if (form == kRpPaired)                                                              \
       e = sweep_rp_launch<LG, A, B, C, D, T, true>(grid, s, f, u, delta, spec, tw, zero, d, n,  \
-                                                   M, par, hinv2, npts, npairs, fstride,     \
+                                                   M, par, zero_u, hinv2, npts, npairs, fstride, \
                                                    spec_stride);                             \
     else                                                                                     \
       e = sweep_rp_launch<LG, A, B, C, D, T, false>(grid, s, f, u, delta, spec, tw, zero, d, n, \
-                                                    M, par, hinv2, npts, npairs, fstride,    \
+                                                    M, par, zero_u, hinv2, npts, npairs, fstride, \
                                                     spec_stride);                            \
     break;                                                                                   \
   }

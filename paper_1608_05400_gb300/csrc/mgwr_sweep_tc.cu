@@ -115,7 +115,7 @@ __constant__ int kPieceB[6] = {0, 1, 0, 2, 1, 0};
 template <int M>
 __global__ void __launch_bounds__(kThreads, 2)
     k_sweep_tc(const float* __restrict__ f, float* __restrict__ u, float* __restrict__ delta,
-               const unsigned char* __restrict__ band, int d, int n, int par, float hinv2,
+               const unsigned char* __restrict__ band, int d, int n, int par, bool zero_u, float hinv2,
                int npts, int tiles_per_inst, size_t fstride, size_t bstride) {
   constexpr int kA = kTileRows * kChunk * 2;  // bytes per piece of a b-values chunk
   constexpr int kB = M * kChunk * 2;          // bytes per piece of the Kt band
@@ -151,8 +151,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (k < npts) {
       int i = 0, j = 0;
       p = colour_point(k, d, n, par, i, j);
-      m = 16u | (i > 0 ? 1u : 0u) | (i < n - 1 ? 2u : 0u);
-      if (d == 2) m |= (j > 0 ? 4u : 0u) | (j < n - 1 ? 8u : 0u);
+      m = 16u;
+      if (!zero_u) m |= (i > 0 ? 1u : 0u) | (i < n - 1 ? 2u : 0u);
+      if (d == 2 && !zero_u) m |= (j > 0 ? 4u : 0u) | (j < n - 1 ? 8u : 0u);
     }
     rowp[threadIdx.x] = p;
     rowm[threadIdx.x] = m;
@@ -342,7 +343,8 @@ namespace {
 
 template <int M>
 cudaError_t tc_launch(const float* f, float* u, float* delta, const unsigned char* band,
-                      size_t bstride, const LevelShape& ls, int par, float hinv2, cudaStream_t s) {
+                      size_t bstride, const LevelShape& ls, int par, float hinv2, cudaStream_t s,
+                      bool zero_u) {
   const int npts = colour_count(ls.d, ls.n, par);
   if (npts == 0 || ls.batch == 0) return cudaSuccess;
   const int tiles = (npts + kTileRows - 1) / kTileRows;
@@ -358,7 +360,7 @@ cudaError_t tc_launch(const float* f, float* u, float* delta, const unsigned cha
   auto kern = k_sweep_tc<M>;
   cudaError_t e = prepare_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)grid, kThreads, smem, s>>>(f, u, delta, band, ls.d, ls.n, par, hinv2, npts,
+  kern<<<(unsigned)grid, kThreads, smem, s>>>(f, u, delta, band, ls.d, ls.n, par, zero_u, hinv2, npts,
                                               tiles, ls.field_stride(), bstride);
   return cudaSuccess;
 }
@@ -391,12 +393,12 @@ __global__ void k_band_bf16x3(const double* __restrict__ kcol, unsigned char* __
 
 cudaError_t launch_sweep_tc(const float* f, float* u, float* delta, const unsigned char* band,
                             size_t bstride, const LevelShape& ls, int par, float hinv2,
-                            cudaStream_t s) {
+                            cudaStream_t s, bool zero_u) {
   cudaError_t e = cudaErrorInvalidValue;
   switch (ls.M) {
-    case 64: e = tc_launch<64>(f, u, delta, band, bstride, ls, par, hinv2, s); break;
-    case 128: e = tc_launch<128>(f, u, delta, band, bstride, ls, par, hinv2, s); break;
-    case 256: e = tc_launch<256>(f, u, delta, band, bstride, ls, par, hinv2, s); break;
+    case 64: e = tc_launch<64>(f, u, delta, band, bstride, ls, par, hinv2, s, zero_u); break;
+    case 128: e = tc_launch<128>(f, u, delta, band, bstride, ls, par, hinv2, s, zero_u); break;
+    case 256: e = tc_launch<256>(f, u, delta, band, bstride, ls, par, hinv2, s, zero_u); break;
     default: break;
   }
   if (e != cudaSuccess) return e;

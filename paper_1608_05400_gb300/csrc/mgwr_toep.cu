@@ -214,6 +214,7 @@ struct Geometry {
   int group0, groups;      // the slab: groups group0 .. group0 + groups - 1 of all instances
   size_t fstride;          // values of one instance's field
   size_t bstride;          // bytes from one instance's band to the next
+  bool zero_u;             // u is zero: no neighbour sums
 };
 
 // b of steps m .. m + W - 1 of point p (line start `base`, neighbours by flag).
@@ -272,8 +273,9 @@ __global__ void __launch_bounds__(512, 3)
     int i = 0, j = 0;
     const int p = colour_point(k, G.d, G.n, G.par, i, j);
     const size_t base = inst * G.fstride + (size_t)p * M;
-    gather_steps<8>(f, u, base + 8 * (threadIdx.x / LPB), M, (size_t)G.n * M, i > 0,
-                    i < G.n - 1, G.d == 2 && j > 0, G.d == 2 && j < G.n - 1, hinv2, b);
+    gather_steps<8>(f, u, base + 8 * (threadIdx.x / LPB), M, (size_t)G.n * M,
+                    i > 0 && !G.zero_u, i < G.n - 1 && !G.zero_u, G.d == 2 && j > 0 && !G.zero_u,
+                    G.d == 2 && j < G.n - 1 && !G.zero_u, hinv2, b);
 #pragma unroll
     for (int q = 0; q < 8; ++q) ef = max(ef, exp_field(b[q]));
   } else {
@@ -333,8 +335,9 @@ __global__ void __launch_bounds__(256)
   cols += inst * cstride;
   for (int m = 2 * threadIdx.x; m < t0 + OB; m += 512) {
     double b[2];
-    gather_steps<2>(f, u, base + m, M, (size_t)G.n * M, i > 0, i < G.n - 1, G.d == 2 && j > 0,
-                    G.d == 2 && j < G.n - 1, hinv2, b);
+    gather_steps<2>(f, u, base + m, M, (size_t)G.n * M, i > 0 && !G.zero_u,
+                    i < G.n - 1 && !G.zero_u, G.d == 2 && j > 0 && !G.zero_u,
+                    G.d == 2 && j < G.n - 1 && !G.zero_u, hinv2, b);
     sb[m] = b[0];
     sb[m + 1] = b[1];
     const double2 c = __ldg(reinterpret_cast<const double2*>(cols + m));
@@ -811,7 +814,7 @@ size_t toep_scratch_bytes(const LevelShape& ls) {
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
                               size_t cstride, const unsigned char* band, size_t bstride,
                               unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
-                              cudaStream_t s) {
+                              cudaStream_t s, bool zero_u) {
   if (!toep_length(ls.M)) return cudaErrorInvalidValue;
   const int npts = colour_count(ls.d, ls.n, par);
   if (npts == 0 || ls.batch == 0) return cudaSuccess;
@@ -823,6 +826,7 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
   G.npts = npts;
   G.fstride = ls.field_stride();
   G.bstride = bstride;
+  G.zero_u = zero_u;
   const long long lines = (long long)npts * ls.batch;
   if (lines * ls.M * ls.M / 2 <= kDirectWork && lines <= 65535) {
     G.per_inst = G.group0 = G.groups = 0;
