@@ -13,7 +13,8 @@
 // E and F the exponents of the largest |b| of the line and |k| of the column.
 // s_p, the sum of the products with i + j = p for p = 0..7, is an FP32
 // accumulator of integers; a segment of the sum is as long as keeps it within
-// 2^24, so every s_p is exact.  Segments are added in two 64-bit integers per
+// 2^24 for any b (bounded at set-up with the column's own digits), so every s_p is
+// exact.  Segments are added in two 64-bit integers per
 // value and the total is rounded to FP64 once.  What is dropped, the products
 // with i + j > 7, is about 2^-59 (largest |k|) (largest |b|); the half-sweep's
 // error against 64-bit sums is that of the final rounding (about 1e-16 of the
@@ -76,14 +77,16 @@ constexpr int kThreads = kIssuer + 32 * kIssuers;
 
 __host__ __device__ constexpr int cores(int M) { return (M < kTile ? kTile : M) / 8 + 15; }
 __host__ __device__ constexpr size_t slice_bytes(int M) { return (size_t)cores(M) * 128; }
-// band blob: the slices, then { first slices by lag (4 bits per 64 lags), F, fold shift }
-__host__ __device__ constexpr size_t blob_bytes(int M) { return kSlices * slice_bytes(M) + 16; }
+// band blob: the slices, then BandHead
+__host__ __device__ constexpr size_t blob_bytes(int M) { return kSlices * slice_bytes(M) + 32; }
 
 struct BandHead {
   unsigned long long first;
   int F;
   short shift;   // low bits dropped when the two sums are joined: |y| < 2^(62 + shift) units
   short chunks;  // chunks from the diagonal down that have a nonzero slice
+  unsigned starts;  // bit c: a segment starts with chunk c
+  unsigned pad;
 };
 
 __device__ __forceinline__ const BandHead* band_head(const unsigned char* blob, int M) {
@@ -109,9 +112,12 @@ __device__ __forceinline__ int chunk_core(int M, int c) { return (chunk_lag0(M, 
 __device__ __forceinline__ int first_slice(unsigned long long first, int c) {
   return (int)(first >> (4 * (c >> 1))) & 15;
 }
-// Chunks of a segment starting with slice i0: an order sums at most 8 - i0
-// products a step, each at most 2^14, so 1024 / (8 - i0) steps stay within 2^24.
-__device__ __forceinline__ int segment_chunks(int i0) { return 32 / (kSlices - i0); }
+// the chunk after the segment that starts with chunk c
+__device__ __forceinline__ int segment_end(unsigned starts, int c, int nc) {
+  const unsigned later = c + 1 < 32 ? starts >> (c + 1) : 0u;
+  const int end = later != 0 ? c + __ffs((int)later) : nc;
+  return end < nc ? end : nc;
+}
 
 // exponent field of |x| (1 for zero and subnormals, 2047 for inf and NaN)
 __device__ __forceinline__ int exp_field(double x) {
@@ -150,6 +156,8 @@ __global__ void __launch_bounds__(256)
   __shared__ short dig[kSlices][1024];
   __shared__ int s_ef, s_last[kSlices];
   __shared__ double s_sum[8];
+  // per chunk: most that one step's digits add to |s_7| and, less, to |s_2|
+  __shared__ int s_prefix[1025], s_scan[8], s_all[32], s_top[32];
   const double* k = cols + (size_t)blockIdx.x * M;
   unsigned char* out = blob + (size_t)blockIdx.x * blob_bytes(M);
   if (threadIdx.x == 0) s_ef = 1;
@@ -183,6 +191,52 @@ __global__ void __launch_bounds__(256)
     *reinterpret_cast<__half*>(out + i * slice_bytes(M) + g * 128 + r * 16 + c * 2) =
         __int2half_rn(v);
   }
+  // A chunk adds to |s_7| at most sum_{i < 7} 128 W_i + 64 W_7 (the leading digit of b
+  // is at most 64) and to |s_2| at most 128 (W_0 + W_1) + 64 W_2, W_i the largest sum
+  // of the 32 consecutive |K_i| that a row of its window multiplies.
+  const int chunks = M / kChunk;
+  if (threadIdx.x < 32) s_all[threadIdx.x] = s_top[threadIdx.x] = 0;
+  for (int i = 0; i < kSlices; ++i) {
+    __syncthreads();
+    int own[4], acc = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int m = 4 * threadIdx.x + q;
+      acc += m < M ? abs((int)dig[i][m]) : 0;
+      own[q] = acc;
+    }
+    int incl = acc;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if ((threadIdx.x & 31) >= o) incl += up;
+    }
+    if ((threadIdx.x & 31) == 31) s_scan[threadIdx.x >> 5] = incl;
+    __syncthreads();
+    int before = incl - acc;
+    for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) before += s_scan[w];
+    if (threadIdx.x == 0) s_prefix[0] = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (4 * threadIdx.x + q < M) s_prefix[4 * threadIdx.x + q + 1] = before + own[q];
+    __syncthreads();
+    // eight threads per chunk; row r multiplies lags chunk_lag0 - 31 + r .. chunk_lag0 + r
+    const int c = threadIdx.x >> 3;
+    int most = 0;
+    if (c < chunks)
+      for (int r = threadIdx.x & 7; r < kTile; r += 8) {
+        const int hi = min(M, max(0, chunk_lag0(M, c) + r + 1));
+        const int lo = min(M, max(0, chunk_lag0(M, c) + r + 1 - kChunk));
+        most = max(most, s_prefix[hi] - s_prefix[lo]);
+      }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    if (c < chunks && (threadIdx.x & 7) == 0) {
+      s_all[c] += most * (i == kSlices - 1 ? 64 : 128);
+      if (i < 3) s_top[c] += most * (i == 2 ? 64 : 128);
+    }
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     unsigned long long first = 0;
     const int pairs = M < kTile ? 1 : M / kChunk / 2;
@@ -203,6 +257,19 @@ __global__ void __launch_bounds__(256)
     int live = 0;
     while (live < pairs && first_slice(first, 2 * live) < kSlices) ++live;
     h->chunks = (short)(2 * live);
+    // segments: within 2^24 for every order, and 256 |s_2| + |s_3| within 2^31
+    unsigned starts = 1;
+    int all = 0, top = 0;
+    for (int c = 0; c < chunks; ++c) {
+      if (c > 0 && (all + s_all[c] > (1 << 24) || top + s_top[c] > 8000000)) {
+        starts |= 1u << c;
+        all = top = 0;
+      }
+      all += s_all[c];
+      top += s_top[c];
+    }
+    h->starts = starts;
+    h->pad = 0;
   }
 }
 
@@ -596,8 +663,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       const unsigned long long first =
           (unsigned long long)uniform((unsigned)(f64 >> 32)) << 32 | uniform((unsigned)f64);
       const int nc = min(tile_chunks(M, tau), (int)uniform((unsigned)head->chunks));
+      const unsigned starts = uniform(head->starts);
       for (int c = 0; ok && c < nc; ++seg) {
-        const int end = min(nc, c + segment_chunks(first_slice(first, c)));
+        const int end = segment_end(starts, c, nc);
         const int a = seg & 1;
         const unsigned dst = tmem_u + (unsigned)(a * kCols);
         if (seg >= 2) ok = warp_wait(&acc_empty[a], (unsigned)((seg / 2 - 1) & 1));
@@ -637,6 +705,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const BandHead* head = band_head(band + inst * G.bstride, M);
       const unsigned long long first = head->first;
       const int shift = head->shift;
+      const unsigned starts = head->starts;
       const int nc = min(tile_chunks(M, tau), (int)head->chunks);
       // lane x holds the point and exponent of line x of this quarter
       const int k = (G.group0 + g - inst * G.per_inst) * NL + mine + (lane & (kMine - 1));
@@ -694,7 +763,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[a]);
         ++seg;
-        c += segment_chunks(i0);
+        c = segment_end(starts, c, nc);
       }
       if (!ok) break;
       const int t = kTile * tau + 32 * (warp & 3) + lane;
