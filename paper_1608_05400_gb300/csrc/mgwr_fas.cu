@@ -20,6 +20,7 @@
 // The history sums are direct (O(M^2) per line, as the scheme is written):
 // the paper's nonlinear tables use M <= 256, and M is limited to 1024 here, so
 // both kernels stay within the default 48 KB of dynamic shared memory.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -255,9 +256,144 @@ __global__ void __launch_bounds__(BLOCK)
   }
 }
 
-// out = base + sign * N_h(u) on every point (one block per line), and the
+// k_fas_fixed's iteration with the convolution as FP64 sums, one line per cluster
+// of C blocks of M threads.  The transform of a pair costs about 78 M clocks of one
+// SM's FP64 pipe and runs on as many SMs as there are pairs (coarse levels: a few);
+// the sums cost M^2 / 4 clocks of it and spread over the cluster, M^2 / (4 C).
+// Block `rank` owns the steps t = rank mod C (equal shares of the triangle): it forms
+// their right-hand sides and hands them to the cluster's other blocks through
+// distributed shared memory (two buffers, one cluster barrier an iteration), then
+// sums its outputs with C threads each.  Settled per line by k_fas_fixed's rule; the
+// largest change and value travel with the next iteration's right-hand sides, so
+// that all blocks decide alike.  With the neighbours fixed the right-hand side
+// f + sigma v - phi(v) is a cubic in v whose sigma terms cancel: three operations.
+// M = 256, one half-sweep of the 255-point grid: 59 us
+// against 106; the coarser levels 41 .. 25 us.
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(1024)
+    k_fas_fixed_sums(double* __restrict__ u, const double* __restrict__ f,
+                     const double* __restrict__ kcol, int n, int M, double hinv, double hinv2,
+                     double c, double sigma, int coef, int parity, int all_points, int max_it,
+                     int* __restrict__ status, unsigned long long* __restrict__ iterations) {
+  namespace cg = cooperative_groups;
+  extern __shared__ double sums_sm[];
+  // per buffer and rank: largest change, largest value (bits of non-negative doubles,
+  // which order like them; compared as integers, off the FP64 pipe)
+  __shared__ unsigned long long most[2][C][2];
+  __shared__ unsigned long long red[2][32];
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int rank = C == 1 ? 0 : (int)cluster.block_rank();
+  double* const sk = sums_sm;          // the inverse column
+  double* const sb = sums_sm + M;      // two buffers of right-hand sides
+  double* const sv = sums_sm + 3 * M;  // this block's outputs
+  const int tid = threadIdx.x;
+  const int k = blockIdx.x / C;
+  const int i = all_points ? k : 2 * k + parity;
+  const int own = M / C;
+  const bool owner = tid < own;
+  const int t = tid * C + rank;
+  double* const line = u + (size_t)i * M;
+  double v = 0.0, fm = 0.0, P = 0.0, Q = 0.0;
+  if (owner) {
+    v = line[t];
+    fm = f[(size_t)i * M + t];
+    if (!all_points && i + 1 < n) P = line[M + t];
+    if (!all_points && i > 0) Q = line[t - M];
+  }
+  sk[tid] = kcol[tid];
+  // b = b0 + b1 v + b2 v^2 + b3 v^3 for D(v) = 1 + kappa v^2
+  const double kappa = coef == MGWR_FAS_D_POROUS ? 1.0 : 0.0;
+  const double b3 = -kappa * hinv2, b2 = 0.5 * kappa * hinv2 * (P + Q);
+  const double b1 = -0.5 * kappa * hinv2 * (P * P + Q * Q);
+  const double b0 = fm + (c >= 0.0 ? c * P : -c * Q) * hinv +
+                    0.5 * hinv2 * ((2.0 + kappa * P * P) * P + (2.0 + kappa * Q * Q) * Q);
+  // magnitude bits, 0 for NaN (as fmax ignores it)
+  auto mag = [](double x) {
+    const unsigned long long m = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+    return m > 0x7FF0000000000000ull ? 0ull : m;
+  };
+  // the output this thread helps to sum
+  const int o = tid / C, lane = tid % C, to = o * C + rank;
+  bool settled = false;
+  double d_prev = 0.0;
+  int it = 0;
+  for (;; ++it) {
+    const int buf = it & 1;
+    if (owner) {
+      const double b = fma(fma(fma(b3, v, b2), v, b1), v, b0);
+      for (int r = 0; r < C; ++r)
+        (C == 1 ? sb : cluster.map_shared_rank(sb, r))[buf * M + t] = b;
+    }
+    if (C == 1)
+      __syncthreads();
+    else
+      cluster.sync();
+    if (it > 0) {
+      unsigned long long dm = 0, wm = 0;
+      for (int r = 0; r < C; ++r) {
+        dm = max(dm, most[buf][r][0]);
+        wm = max(wm, most[buf][r][1]);
+      }
+      const double d = __longlong_as_double((long long)dm), w = __longlong_as_double((long long)wm);
+      settled = w <= DBL_MAX && (d <= 4e-15 * w || (d <= 1e-12 * w && d >= 0.5 * d_prev));
+      d_prev = d;
+      if (settled || it == max_it) break;
+    }
+    const double* const b = sb + buf * M;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int s = lane; s < to; s += 4 * C) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (s + q * C < to) a[q] = fma(sk[to - s - q * C], b[s + q * C], a[q]);
+    }
+    double y = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+    for (int x = C / 2; x > 0; x >>= 1) y += __shfl_xor_sync(0xffffffffu, y, x);
+    y = fma(sk[0], b[to], y);  // the largest product last
+    if (lane == 0) sv[o] = y;
+    __syncthreads();
+    unsigned long long d = 0, w = 0;
+    if (owner) {
+      const double next = sv[tid];
+      d = mag(next - v);
+      w = mag(next);
+      v = next;
+    }
+    for (int x = 16; x > 0; x >>= 1) {
+      d = max(d, __shfl_xor_sync(0xffffffffu, d, x));
+      w = max(w, __shfl_xor_sync(0xffffffffu, w, x));
+    }
+    if ((tid & 31) == 0) {
+      red[0][tid >> 5] = d;
+      red[1][tid >> 5] = w;
+    }
+    __syncthreads();
+    if (tid < C) {  // thread r tells rank r
+      d = w = 0;
+      for (int x = 0; x < (own + 31) / 32; ++x) {
+        d = max(d, red[0][x]);
+        w = max(w, red[1][x]);
+      }
+      unsigned long long* const to_rank =
+          C == 1 ? &most[0][0][0] : cluster.map_shared_rank(&most[0][0][0], tid);
+      to_rank[((buf ^ 1) * C + rank) * 2] = d;
+      to_rank[((buf ^ 1) * C + rank) * 2 + 1] = w;
+    }
+  }
+  if (owner) line[t] = v;
+  if (tid == 0 && rank == 0) {
+    if (!settled) atomicOr(status, 2);
+    atomicAdd(iterations, (unsigned long long)it);  // line iterations
+  }
+}
+
+// out = base + sign * N_h(u) on every point (gridDim.y blocks per line, block y the
+// steps y mod gridDim.y: coarse levels have fewer lines than SMs), and the
 // max-norm of out into *norm_bits (the bits of a non-negative double; a
-// non-finite value counts as +inf).  Dynamic shared memory: 2 * M doubles.
+// non-finite value counts as +inf).  Eight threads share a history sum; the
+// spatial terms are formed by whole warps afterwards.  Dynamic shared memory: 3 * M
+// doubles.  h is a power of two, so its reciprocals are exact.  M = 256, mean over the levels: 13 us, 20.7 with
+// one block per line and one thread per sum.
 __global__ void __launch_bounds__(kApplyThreads)
     k_fas_apply(const double* __restrict__ u, const double* __restrict__ r,
                 const double* __restrict__ base, double* __restrict__ out, int n, int M,
@@ -265,6 +401,7 @@ __global__ void __launch_bounds__(kApplyThreads)
                 unsigned long long* __restrict__ norm_bits) {
   extern __shared__ double sm[];
   __shared__ double wmax[kApplyThreads / 32];
+  constexpr int kLanes = 8;
   double* rs = sm;
   double* line = sm + M;
   const int i = blockIdx.x;
@@ -274,19 +411,37 @@ __global__ void __launch_bounds__(kApplyThreads)
     line[j] = u[row + j];
   }
   __syncthreads();
-  const double h2 = h * h;
+  double* const sums = sm + 2 * M;
+  const double hinv = 1.0 / h, hinv2 = hinv * hinv;
+  const int lane = threadIdx.x % kLanes;
+  const int share = (M - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;
+  // whole warps run each pass (the sums end in shuffles)
+  for (int o0 = 0; o0 < share; o0 += kApplyThreads / kLanes) {
+    const int o = o0 + threadIdx.x / kLanes;
+    const int m = o < share ? o * (int)gridDim.y + (int)blockIdx.y : -1;
+    double t0 = 0.0, t1 = 0.0;
+    for (int j = lane; j <= m; j += 2 * kLanes) {
+      t0 = fma(rs[m - j], line[j], t0);
+      if (j + kLanes <= m) t1 = fma(rs[m - j - kLanes], line[j + kLanes], t1);
+    }
+    double t = t0 + t1;
+#pragma unroll
+    for (int x = kLanes / 2; x > 0; x >>= 1) t += __shfl_xor_sync(0xffffffffu, t, x);
+    if (m >= 0 && lane == 0) sums[o] = t;
+  }
+  __syncthreads();
   double local = 0.0;
-  for (int m = threadIdx.x; m < M; m += blockDim.x) {
-    double t = 0.0;
-    for (int j = 0; j <= m; ++j) t = fma(rs[m - j], line[j], t);
+  for (int o = threadIdx.x; o < share; o += kApplyThreads) {
+    const int m = o * (int)gridDim.y + (int)blockIdx.y;
+    const double t = sums[o];
     const double w0 = line[m];
     const double wp = i + 1 < n ? u[row + M + m] : 0.0;
     const double wm = i > 0 ? u[row - M + m] : 0.0;
     const double D0 = coef_D(coef, w0);
     const double a_plus = 0.5 * (coef_D(coef, wp) + D0);
     const double a_minus = 0.5 * (coef_D(coef, wm) + D0);
-    const double diffusion = (a_plus * (wp - w0) - a_minus * (w0 - wm)) / h2;
-    const double convection = c >= 0.0 ? c * (wp - w0) / h : c * (w0 - wm) / h;
+    const double diffusion = (a_plus * (wp - w0) - a_minus * (w0 - wm)) * hinv2;
+    const double convection = c >= 0.0 ? c * (wp - w0) * hinv : c * (w0 - wm) * hinv;
     const double val = base[row + m] + sign * (t - (diffusion + convection));
     out[row + m] = val;
     const double a = fabs(val);
@@ -302,16 +457,19 @@ __global__ void __launch_bounds__(kApplyThreads)
   }
 }
 
-// Full weighting (1/4)[1 2 1] of two fine fields (n = 2 nc + 1 lines) at once.
+// Full weighting (1/4)[1 2 1] of two fine fields (n = 2 nc + 1 lines) at once, the
+// first to two places (R u and the coarse iterate that starts from it).
 __global__ void k_fas_restrict2(const double* __restrict__ a, double* __restrict__ ac,
-                                const double* __restrict__ b, double* __restrict__ bc, int nc,
-                                int M) {
+                                double* __restrict__ ac2, const double* __restrict__ b,
+                                double* __restrict__ bc, int nc, int M) {
   const size_t total = (size_t)nc * M;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
        idx += (size_t)gridDim.x * blockDim.x) {
     const size_t J = idx / M, m = idx % M;
     const size_t f0 = 2 * J * M + m;  // fine line 2J, then 2J+1 and 2J+2
-    ac[idx] = 0.25 * ((a[f0] + 2.0 * a[f0 + M]) + a[f0 + 2 * M]);
+    const double x = 0.25 * ((a[f0] + 2.0 * a[f0 + M]) + a[f0 + 2 * M]);
+    ac[idx] = x;
+    ac2[idx] = x;
     bc[idx] = 0.25 * ((b[f0] + 2.0 * b[f0 + M]) + b[f0 + 2 * M]);
   }
 }
@@ -368,6 +526,10 @@ struct mgwr_fas {
   std::vector<double> sigma;
   size_t line_smem = 0, apply_smem = 0;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  // one cycle and the norm of its defect as a CUDA graph (about 45 launches at 255
+  // points), captured by the second cycle of a solve, for one set of settings
+  cudaGraphExec_t graph = nullptr;
+  long long graph_key = -1, graph_kernels = 0;
   std::string err;
 };
 
@@ -409,10 +571,33 @@ cudaError_t launch_line(mgwr_fas* h, int l, int parity, int all_points) {
   if (fixed_point(h)) {
     const int L = 2 * h->M, logL = mgwr::ilog2(L);
     const double hl = level_h(l);
+    int* st = reinterpret_cast<int*>(h->flags + 1);
+    // blocks per line: as many as keep one line's cluster per SM group
+    const int sms = mgwr::sm_count();
+    const int C = count * 8 <= sms ? 8 : count * 4 <= sms ? 4 : count * 2 <= sms ? 2 : 1;
+    // clocks an iteration takes an SM's FP64 pipe: the sums (and about 3000 of
+    // right-hand sides and barriers) against the transform of one pair
+    const long long M = h->M;
+    const long long sums = (M * M / (4 * C) + 3000) * ((count * C + sms - 1) / sms);
+    const long long transform = 78 * M * ((((long long)count + 1) / 2 + sms - 1) / sms);
+    if (sums < transform) {
+      const size_t smem = sizeof(double) * (size_t)(3 * M + M / C);
+#define MGWR_SUMS_LAUNCH(CC)                                                                      \
+  mgwr::k_fas_fixed_sums<CC><<<(unsigned)(count * CC), (unsigned)M, smem, h->stream>>>(           \
+      h->u[l], h->f[l], h->kcol + (size_t)l * M, n, (int)M, 1.0 / hl, 1.0 / (hl * hl), h->c,      \
+      h->sigma[l], h->coef, parity, all_points, kFixedMaxIt, st, h->flags + 2)
+      switch (C) {
+        case 8: MGWR_SUMS_LAUNCH(8); break;
+        case 4: MGWR_SUMS_LAUNCH(4); break;
+        case 2: MGWR_SUMS_LAUNCH(2); break;
+        default: MGWR_SUMS_LAUNCH(1); break;
+      }
+#undef MGWR_SUMS_LAUNCH
+      return mgwr::counted(cudaGetLastError());
+    }
     const unsigned grid = (unsigned)((count + 1) / 2);
     const size_t smem = mgwr::Pad<double>::len(L) * sizeof(Cx<double>);
     const Cx<double>* ks = h->kspec + (size_t)l * L;
-    int* st = reinterpret_cast<int*>(h->flags + 1);
 #define MGWR_FIXED_LAUNCH(B)                                                                    \
   mgwr::k_fas_fixed<B><<<grid, B, smem, h->stream>>>(h->u[l], h->f[l], ks, h->tw, n, h->M, logL, \
                                                      1.0 / hl, 1.0 / (hl * hl), h->c,           \
@@ -436,7 +621,14 @@ cudaError_t launch_line(mgwr_fas* h, int l, int parity, int all_points) {
 
 cudaError_t launch_apply(mgwr_fas* h, int l, const double* u, const double* base, double* out,
                          double sign, bool norm) {
-  mgwr::k_fas_apply<<<level_n(l), mgwr::kApplyThreads, h->apply_smem, h->stream>>>(
+  // blocks per line: two blocks per SM where the lines are fewer, at least 16 steps each
+  const int lines = level_n(l);
+  int split = 2 * mgwr::sm_count() / lines;
+  if (split > h->M / 16) split = h->M / 16;
+  if (split > 16) split = 16;
+  if (split < 1) split = 1;
+  const dim3 grid((unsigned)lines, (unsigned)split);
+  mgwr::k_fas_apply<<<grid, mgwr::kApplyThreads, h->apply_smem, h->stream>>>(
       u, h->r, base, out, level_n(l), h->M, level_h(l), h->c, h->coef, sign,
       norm ? h->flags : nullptr);
   return mgwr::counted(cudaGetLastError());
@@ -466,14 +658,11 @@ cudaError_t fas_cycle(mgwr_fas* h, int l, int nu1, int nu2, int gamma) {
   const int nc = level_n(l - 1);
   // ubar = R u, R r (into the coarse defect field, free until the coarse cycle)
   mgwr::k_fas_restrict2<<<grid_for((size_t)nc * h->M), 256, 0, h->stream>>>(
-      h->u[l], h->ubar[l - 1], h->rr[l], h->rr[l - 1], nc, h->M);
+      h->u[l], h->ubar[l - 1], h->u[l - 1], h->rr[l], h->rr[l - 1], nc, h->M);
   if ((e = mgwr::counted(cudaGetLastError())) != cudaSuccess) return e;
   // f_c = N_2h(ubar) + R r; the coarse iterate starts from ubar
   if ((e = launch_apply(h, l - 1, h->ubar[l - 1], h->rr[l - 1], h->f[l - 1], 1.0, false)) !=
       cudaSuccess)
-    return e;
-  if ((e = cudaMemcpyAsync(h->u[l - 1], h->ubar[l - 1], field_bytes(h, l - 1),
-                           cudaMemcpyDeviceToDevice, h->stream)) != cudaSuccess)
     return e;
   for (int g = 0; g < gamma; ++g)
     if ((e = fas_cycle(h, l - 1, nu1, nu2, gamma)) != cudaSuccess) return e;
@@ -504,15 +693,67 @@ cudaError_t clear_norm(mgwr_fas* h) {
   return cudaMemsetAsync(h->flags, 0, sizeof(unsigned long long), h->stream);
 }
 
+// The max-norm a defect left, and the failure of a line solve since the last clear.
+int read_norm(mgwr_fas* h, double* norm) {
+  bool failed = false;
+  int s = read_flags(h, norm, &failed);
+  if (s == MGWR_OK && failed)
+    s = fas_fail(h, MGWR_E_NUMERIC, "a line solve did not settle (Newton's method or the whole-line fixed point)");
+  return s;
+}
+
 int defect_norm(mgwr_fas* h, int l, double* norm) {
   int s = fas_cuda(h, clear_norm(h), "clear norm");
   if (s == MGWR_OK)
     s = fas_cuda(h, launch_apply(h, l, h->u[l], h->f[l], h->rr[l], -1.0, true), "defect");
-  bool failed = false;
-  if (s == MGWR_OK) s = read_flags(h, norm, &failed);
-  if (s == MGWR_OK && failed)
-    s = fas_fail(h, MGWR_E_NUMERIC, "a line solve did not settle (Newton's method or the whole-line fixed point)");
-  return s;
+  return s == MGWR_OK ? read_norm(h, norm) : s;
+}
+
+// The launches of one cycle from the finest level and of its defect's norm.
+cudaError_t enqueue_cycle(mgwr_fas* h, int nu1, int nu2, int gamma) {
+  const int L = h->nlev - 1;
+  cudaError_t e = fas_cycle(h, L, nu1, nu2, gamma);
+  if (e == cudaSuccess) e = clear_norm(h);
+  if (e == cudaSuccess) e = launch_apply(h, L, h->u[L], h->f[L], h->rr[L], -1.0, true);
+  return e;
+}
+
+void drop_graph(mgwr_fas* h) {
+  if (h->graph) cudaGraphExecDestroy(h->graph);
+  h->graph = nullptr;
+  h->graph_key = -1;
+}
+
+// enqueue_cycle as a graph replay, captured on first use; the launches themselves
+// where the stream cannot be captured.
+cudaError_t replay_cycle(mgwr_fas* h, int nu1, int nu2, int gamma) {
+  const long long key =
+      (((long long)h->order * 4 + h->smoother) * 4 + gamma) * 1024 + nu1 * 32 + nu2;
+  if (h->graph_key != key) {
+    drop_graph(h);
+    if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();
+      return enqueue_cycle(h, nu1, nu2, gamma);
+    }
+    const long long before = mgwr::launch_counter();
+    cudaError_t e = enqueue_cycle(h, nu1, nu2, gamma);
+    cudaGraph_t g = nullptr;
+    const cudaError_t end = cudaStreamEndCapture(h->stream, &g);
+    const long long kernels = mgwr::launch_counter() - before;
+    mgwr::add_launches(-kernels);  // captured, not run
+    if (e == cudaSuccess) e = end;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&h->graph, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) {
+      h->graph = nullptr;
+      return e;
+    }
+    h->graph_key = key;
+    h->graph_kernels = kernels;
+  }
+  const cudaError_t e = cudaGraphLaunch(h->graph, h->stream);
+  if (e == cudaSuccess) mgwr::add_launches(h->graph_kernels);
+  return e;
 }
 
 double* field_of(mgwr_fas* h, int l, int which) {
@@ -525,6 +766,7 @@ double* field_of(mgwr_fas* h, int l, int which) {
 }
 
 void release(mgwr_fas* h) {
+  drop_graph(h);
   auto fr = [](double* p) { if (p) cudaFree(p); };
   for (auto* v : {&h->u, &h->f, &h->rr, &h->ubar})
     for (double* p : *v) fr(p);
@@ -568,7 +810,7 @@ int mgwr_fas_create(int n, int M, double T, double alpha, double c, int coeffici
   while (level_n(h->nlev) < n) ++h->nlev;
   ++h->nlev;  // levels 0..nlev-1 with level_n(nlev-1) = n
   h->line_smem = sizeof(double) * (size_t)(1 + mgwr::kLineWarps) * M;
-  h->apply_smem = sizeof(double) * 2 * (size_t)M;
+  h->apply_smem = sizeof(double) * 3 * (size_t)M;
   auto bail = [&](int code) {
     release(h);
     delete h;
@@ -605,7 +847,7 @@ int mgwr_fas_create(int n, int M, double T, double alpha, double c, int coeffici
     h->ubar.push_back(ub);
   }
   if (!ok) return bail(MGWR_E_NOMEM);
-  // (1 + kLineWarps) * 1024 and 2 * 1024 doubles: within the default 48 KB
+  // (1 + kLineWarps) * 1024 and 3 * 1024 doubles: within the default 48 KB
   static_assert((1 + mgwr::kLineWarps) * mgwr::kFasMaxM * sizeof(double) <= 48 * 1024,
                 "k_fas_line shared memory");
   cudaError_t e = cudaSuccess;
@@ -828,9 +1070,10 @@ int mgwr_fas_solve(mgwr_fas_t h, int cycle, int nu1, int nu2, double tol, int ma
   st.relres = 1.0;
   s = fas_cuda(h, cudaEventRecord(h->ev0, h->stream), "event");
   while (s == MGWR_OK && st.cycles < max_cycles && st.relres > tol) {
-    s = fas_cuda(h, fas_cycle(h, L, nu1, nu2, cycle), "cycle");
+    s = fas_cuda(h, st.cycles == 0 ? enqueue_cycle(h, nu1, nu2, cycle)
+                                   : replay_cycle(h, nu1, nu2, cycle), "cycle");
     double nrm = 0.0;
-    if (s == MGWR_OK) s = defect_norm(h, L, &nrm);
+    if (s == MGWR_OK) s = read_norm(h, &nrm);
     if (s != MGWR_OK) break;
     ++st.cycles;
     st.relres = nrm / r0;

@@ -270,3 +270,26 @@ def test_fixed_point_non_finite_rhs_is_reported():
         assert e.value.status == G.MGWR_E_NUMERIC
         g.set_rhs(np.ones((n, M)))
         assert g.solve(1, 0, 1, tol=1e-10, max_cycles=30).relres <= 1e-10
+
+
+# lines per cluster size of the whole-line smoother (8, 4, 2 and 1 blocks per line, more lines
+# than SMs, and the transform where it is cheaper), both colours, against the time march: each
+# solves the same line equations to rounding (the fixed point stops within 4e-15 of a line, or
+# where it no longer falls within 1e-12)
+@pytest.mark.parametrize("n,M,c", [(31, 128, 2.0), (63, 256, -1.0), (127, 128, 1.0),
+                                   (255, 128, -1.0), (511, 128, 1.0), (31, 1024, 1.0),
+                                   (255, 1024, 1.0)])
+def test_whole_line_smoother_equals_the_march_for_every_cluster_size(n, M, c):
+    u0 = inputs.random_field(n, M, seed=41, scale=0.3)
+    f = inputs.random_field(n, M, seed=42, scale=50.0)
+    out = []
+    for smoother in (G.MGWR_FAS_SMOOTHER_FIXED, G.MGWR_FAS_SMOOTHER_MARCH):
+        with G.FAS(n, M, 1.0, 0.6, c=c) as s:
+            s.set_smoother(smoother)
+            s.set_rhs(f)
+            s.set_initial(u0)
+            l = s.num_levels() - 1
+            for colour in (G.MGWR_RED, G.MGWR_BLACK):
+                s.smooth(l, colour)
+            out.append(s.field_get(l, G.MGWR_U))
+    assert np.abs(out[0] - out[1]).max() <= 1e-12 * np.abs(out[1]).max()
