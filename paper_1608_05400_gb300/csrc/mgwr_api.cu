@@ -102,6 +102,7 @@ struct mgwr_handle {
   // sliced bands of the inverse columns (FP64 half-sweeps on the tensor cores,
   // lines of 64 .. 1024 steps) and the scratch of their digits
   unsigned char* toep_band = nullptr;
+  unsigned char* toep_tband = nullptr;  // the same of the Toeplitz columns (FP64 defects)
   unsigned char* toep_scratch = nullptr;
   double* c_dev = nullptr;      // batch
   Hier<double> h64;
@@ -371,9 +372,12 @@ int ensure_toep(mgwr_t h) {
   const size_t lines = (size_t)h->B * h->nlev;
   if (h->toep_scratch == nullptr)
     MGWR_TRY(dev_alloc(h, &h->toep_scratch, mgwr::toep_scratch_bytes(shape(h, h->nlev - 1))));
+  if (h->toep_tband == nullptr)
+    MGWR_TRY(dev_alloc(h, &h->toep_tband, mgwr::toep_band_bytes(h->M) * (size_t)h->B));
   unsigned char* band = nullptr;
   MGWR_TRY(dev_alloc(h, &band, mgwr::toep_band_bytes(h->M) * lines));
   MGWR_CK(h, mgwr::launch_toep_band(h->kcol, band, h->M, lines, h->stream));
+  MGWR_CK(h, mgwr::launch_toep_band(h->r, h->toep_tband, h->M, (size_t)h->B, h->stream));
   h->toep_band = band;
   return MGWR_OK;
 }
@@ -586,15 +590,32 @@ const R* changes(const Hier<R>& H, int l) {
   return H.from_zero[l] ? H.u[l] : H.dl[l];
 }
 
-// Full defect r = f - (T_M (x) I + A_h) u with one FFT convolution per line.
+// The FP64 defect of level l in FP64 into H64's r.
+int defect64(mgwr_t h, int l, unsigned long long* norm_bits) {
+  Hier<double>& H = h->h64;
+  if (h->toep_band != nullptr && mgwr::toep_defect(shape(h, l)))
+    MGWR_CK(h, mgwr::launch_defect_toep(H.u[l], H.f[l], H.r[l], h->toep_tband, h->toep_scratch,
+                                        shape(h, l), h->hinv2[l], norm_bits, h->stream));
+  else
+    MGWR_CK(h, (mgwr::launch_defect<double, double>(
+                   H.u[l], H.f[l], H.r[l], H.tspec, (size_t)h->L, H.tw, H.zero,
+                   scratch_for<double>(h), shape(h, l), h->hinv2[l], norm_bits,
+                   split_of(h, MGWR_K_DEFECT64, l), h->stream)));
+  return MGWR_OK;
+}
+
+// Full defect r = f - (T_M (x) I + A_h) u with one convolution per line.
 template <class R>
 int defect(mgwr_t h, Hier<R>& H, int l, unsigned long long* norm_bits) {
   const int pm = prof_begin(h, defect_class<R>(),
                             (double)(points(h, l) * h->B));
-  MGWR_CK(h, (mgwr::launch_defect<R, R>(H.u[l], H.f[l], H.r[l], H.tspec, (size_t)h->L, H.tw,
-                                         H.zero, scratch_for<R>(h), shape(h, l), R(h->hinv2[l]), norm_bits,
-                                         split_of(h, defect_class<R>(), l),
-                                         h->stream)));
+  if constexpr (std::is_same<R, double>::value)
+    MGWR_TRY(defect64(h, l, norm_bits));
+  else
+    MGWR_CK(h, (mgwr::launch_defect<R, R>(H.u[l], H.f[l], H.r[l], H.tspec, (size_t)h->L, H.tw,
+                                           H.zero, scratch_for<R>(h), shape(h, l), R(h->hinv2[l]),
+                                           norm_bits, split_of(h, defect_class<R>(), l),
+                                           h->stream)));
   prof_end(h, pm);
   H.rs[l] = R_CURRENT;
   return MGWR_OK;
@@ -815,11 +836,7 @@ int finest_defect_norms(mgwr_t h, std::vector<double>& norms, bool to_h32) {
   } else {
     const int pm = prof_begin(h, MGWR_K_DEFECT64, (double)(points(h, L) * h->B));
     MGWR_TRY(ensure_field(h, &h->h64.r[L], level_count(h, L)));
-    MGWR_CK(h, (mgwr::launch_defect<double, double>(h->h64.u[L], h->h64.f[L], h->h64.r[L],
-                                                     h->h64.tspec, (size_t)h->L, h->h64.tw,
-                                                     h->h64.zero, scratch_for<double>(h), shape(h, L), h->hinv2[L], h->norm_bits,
-                                                    split_of(h, MGWR_K_DEFECT64, L),
-                                                     h->stream)));
+    MGWR_TRY(defect64(h, L, h->norm_bits));
     h->h64.rs[L] = R_CURRENT;
     prof_end(h, pm);
   }
@@ -1146,7 +1163,7 @@ int tune_hierarchy(mgwr_t h, Hier<R>& H, int cls_sweep, int cls_defect) {
     const LevelShape ls = tune_sample(h, l);
     st = ensure_field(h, &H.u[l], level_count(h, l));
     if (st == MGWR_OK) st = ensure_field(h, &H.f[l], level_count(h, l));
-    // FP64 sweeps on the tensor cores have one launch shape
+    // FP64 sweeps on the tensor cores have one launch shape (so have their defects)
     const bool fixed = std::is_same<R, double>::value && h->toep_band != nullptr;
     if (st == MGWR_OK && !fixed)
       st = tune_class(h, cls_sweep, l, sizeof(R) == 4 ? 4 : 8, [&](int E) {
@@ -1162,7 +1179,7 @@ int tune_hierarchy(mgwr_t h, Hier<R>& H, int cls_sweep, int cls_defect) {
         if (e != cudaSuccess) return e;
         return level_sweep(h, H, l, H.f[l], out, dlt, ls, parity(h, MGWR_BLACK), E);
       });
-    if (st == MGWR_OK)
+    if (st == MGWR_OK && !(fixed && mgwr::toep_defect(shape(h, l))))
       st = tune_class(h, cls_defect, l, sizeof(R) == 4 ? 4 : 8, [&](int E) {
         return mgwr::launch_defect<R, R>(H.u[l], H.f[l], out, H.tspec, (size_t)h->L, H.tw,
                                          H.zero, scratch_for<R>(h), ls, R(h->hinv2[l]), nullptr,
@@ -1297,6 +1314,8 @@ int refresh_derived(mgwr_t h) {
   if (h->toep_band != nullptr)
     MGWR_CK(h, mgwr::launch_toep_band(h->kcol, h->toep_band, h->M, (size_t)h->B * h->nlev,
                                       h->stream));
+  if (h->toep_band != nullptr)
+    MGWR_CK(h, mgwr::launch_toep_band(h->r, h->toep_tband, h->M, (size_t)h->B, h->stream));
   if (h->tspec_dd != nullptr)
     MGWR_CK(h, mgwr::launch_split_cx(h->tspec_dd, h->h64.tspec, (size_t)h->B * h->L, h->stream));
   if (h->hdd.ready)
@@ -2679,7 +2698,7 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
     total += r512(16 * B * ((pts[0] + 1) / 2) * L);
   if (precision == MGWR_FP64) {
     if (mgwr::toep_length(M))  // sliced bands and digits of the tensor-core sweeps
-      total += r512(mgwr::toep_band_bytes(M) * B * nlev) +
+      total += r512(mgwr::toep_band_bytes(M) * B * nlev) + r512(mgwr::toep_band_bytes(M) * B) +
                r512(mgwr::toep_scratch_bytes(LevelShape{d, n, M, batch}));
     for (size_t l = 0; l < nlev; ++l) total += (l + 1 < nlev ? 4 : 3) * r512(8 * B * pts[l] * M);
   } else if (precision == MGWR_DD) {

@@ -153,6 +153,15 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
                               size_t cstride, const unsigned char* band, size_t bstride,
                               unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
                               cudaStream_t s, bool zero_u = false);
+// The FP64 defect r = f - (T_M (x) I + A_h) u with the time term as sliced products
+// (bands of the instances' Toeplitz columns, toep_band_bytes(M) apart), for the
+// shapes toep_defect names (the transform's single launch is cheaper below);
+// norm_bits as in launch_defect.
+bool toep_defect(const LevelShape& ls);
+cudaError_t launch_defect_toep(const double* u, const double* f, double* r,
+                               const unsigned char* band, unsigned char* scratch,
+                               const LevelShape& ls, double hinv2, unsigned long long* norm_bits,
+                               cudaStream_t s);
 size_t toep_band_bytes(int M);
 // Bytes of scratch the launches on a level of this shape need (bounded: larger
 // fields go through it in slabs).

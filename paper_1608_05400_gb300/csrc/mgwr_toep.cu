@@ -1,6 +1,7 @@
 // FP64 Toeplitz products of whole time lines (64 .. 1024 steps): the FP64
 // smoother's half-sweep (Sec. 3 Eq. red-black, Sec. 6 Eq. red-black_2d) and
-// one-point solve, u_p = k * b_p with b_p = f_p + h^-2 sum of neighbour lines.
+// one-point solve, u_p = k * b_p with b_p = f_p + h^-2 sum of neighbour lines, and
+// the time term T_M u_p of the FP64 defect.
 //
 // GB300 issues two FP64 operations per clock and SM, so the FFT form of the
 // product (about 78 FP64 instructions per value at M = 1024) keeps that pipe
@@ -276,13 +277,19 @@ __global__ void __launch_bounds__(256)
 // ---- gather ---------------------------------------------------------------------
 
 struct Geometry {
-  int d, n, M, par, npts;  // npts: lines of the colour per instance
+  int d, n, M, par, npts;  // npts: lines of the colour (par < 0: of the grid) per instance
   int per_inst;            // groups of NL lines per instance
   int group0, groups;      // the slab: groups group0 .. group0 + groups - 1 of all instances
   size_t fstride;          // values of one instance's field
   size_t bstride;          // bytes from one instance's band to the next
   bool zero_u;             // u is zero: no neighbour sums
 };
+
+// the k-th line of a launch
+__device__ __forceinline__ int launch_point(const Geometry& G, int k, int& i, int& j) {
+  if (G.par >= 0) return colour_point(k, G.d, G.n, G.par, i, j);
+  return k;  // every point; its place in the grid is not needed
+}
 
 // b of steps m .. m + W - 1 of point p (line start `base`, neighbours by flag).
 template <int W>
@@ -321,7 +328,8 @@ __device__ __forceinline__ void gather_steps(const double* __restrict__ f,
 // steps.  LPB = 4 or 8 writes whole 32-byte sectors; small grids take fewer lines
 // per block, so that the FP64 sums of a line (four operations a value, two a clock
 // and SM: what bounds this kernel) spread over the SMs.
-template <int NL, int LPB>
+// PLAIN: b is the line of f itself (the defect's time term of a field).
+template <int NL, int LPB, bool PLAIN>
 __global__ void __launch_bounds__(512, 3)
     k_toep_gather(const double* __restrict__ f, const double* __restrict__ u,
                   const unsigned char* __restrict__ band, unsigned char* __restrict__ dig,
@@ -338,11 +346,12 @@ __global__ void __launch_bounds__(512, 3)
   int ef = 1;
   if (k < G.npts) {
     int i = 0, j = 0;
-    const int p = colour_point(k, G.d, G.n, G.par, i, j);
+    const int p = launch_point(G, k, i, j);
     const size_t base = inst * G.fstride + (size_t)p * M;
-    gather_steps<8>(f, u, base + 8 * (threadIdx.x / LPB), M, (size_t)G.n * M,
-                    i > 0 && !G.zero_u, i < G.n - 1 && !G.zero_u, G.d == 2 && j > 0 && !G.zero_u,
-                    G.d == 2 && j < G.n - 1 && !G.zero_u, hinv2, b);
+    const bool sums = !PLAIN && !G.zero_u;
+    gather_steps<8>(f, u, base + 8 * (threadIdx.x / LPB), M, (size_t)G.n * M, sums && i > 0,
+                    sums && i < G.n - 1, sums && G.d == 2 && j > 0,
+                    sums && G.d == 2 && j < G.n - 1, hinv2, b);
 #pragma unroll
     for (int q = 0; q < 8; ++q) ef = max(ef, exp_field(b[q]));
   } else {
@@ -712,7 +721,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int p = -1, e = 0;
       if (k < G.npts) {
         int i = 0, j = 0;
-        p = colour_point(k, G.d, G.n, G.par, i, j);
+        p = launch_point(G, k, i, j);
         e = lexp[g * NL + mine + (lane & (kMine - 1))];
       }
       long long hi[kMine], lo[kMine];
@@ -805,14 +814,14 @@ int slab_groups(int M, int NL, int groups) {
   return (int)((groups + slabs - 1) / slabs);
 }
 
-template <int NL>
+template <int NL, bool PLAIN>
 cudaError_t gather_launch(const double* f, const double* u, const unsigned char* band,
                           unsigned char* dig, int* lexp, const Geometry& G, double hinv2,
                           cudaStream_t s) {
   const int M = G.M;
 #define MGWR_GATHER(LPB)                                                                  \
-  k_toep_gather<NL, LPB><<<(unsigned)(G.groups * (NL / LPB)), LPB * M / 8, 0, s>>>(f, u, band, dig, \
-                                                                                lexp, G, hinv2)
+  k_toep_gather<NL, LPB, PLAIN><<<(unsigned)(G.groups * (NL / LPB)), LPB * M / 8, 0, s>>>( \
+      f, u, band, dig, lexp, G, hinv2)
   if (M >= 256 && G.groups * (NL / 4) < 2 * sm_count()) {
     MGWR_GATHER(1);
   } else if (M == 128 && G.groups * (NL / 8) < 2 * sm_count()) {
@@ -832,7 +841,8 @@ cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigne
   const int M = G.M;
   unsigned char* dig = scratch;
   int* lexp = reinterpret_cast<int*>(scratch + (size_t)G.groups * NL * M * kLineValue);
-  cudaError_t e = gather_launch<NL>(f, u, band, dig, lexp, G, hinv2, s);
+  cudaError_t e = G.par >= 0 ? gather_launch<NL, false>(f, u, band, dig, lexp, G, hinv2, s)
+                             : gather_launch<NL, true>(f, u, band, dig, lexp, G, hinv2, s);
   if (e != cudaSuccess) return e;
   Items items;
   items.groups = G.groups;
@@ -860,6 +870,69 @@ cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigne
 // 31 lines (4.1 M) 23 against 21 us.
 constexpr long long kDirectWork = 1ll << 22;
 
+// Every line of a launch, in slabs of groups.
+cudaError_t product(const double* f, double* u, double* delta, const unsigned char* band,
+                    unsigned char* scratch, Geometry G, int batch, double hinv2, cudaStream_t s) {
+  const int NL = lines_per_group(G.M, G.npts, batch);
+  G.per_inst = (G.npts + NL - 1) / NL;
+  const int total = G.per_inst * batch;
+  const int step = slab_groups(G.M, NL, total);
+  for (int g0 = 0; g0 < total; g0 += step) {
+    G.group0 = g0;
+    G.groups = total - g0 < step ? total - g0 : step;
+    const cudaError_t e = NL == 32 ? slab_launch<32>(f, u, delta, band, scratch, G, hinv2, s)
+                                   : slab_launch<16>(f, u, delta, band, scratch, G, hinv2, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// r = f - r - h^-2 sum (u_p - u_q), r holding T_M u; every difference formed before the
+// sum.  A group of threads per line, 16-byte accesses.  Nine FP64 operations a value
+// bound it (66.6 million values: 1.0 ms of the pipe).
+__global__ void __launch_bounds__(256)
+    k_defect_finish(const double* __restrict__ u, const double* __restrict__ f,
+                    double* __restrict__ r, int d, int n, int M, int log_tpl, int npts,
+                    double hinv2, unsigned long long* __restrict__ norm_bits, size_t fstride) {
+  __shared__ double red[8];
+  const int tpl = 1 << log_tpl;
+  const int p = blockIdx.x * (256 >> log_tpl) + (threadIdx.x >> log_tpl);
+  u += blockIdx.y * fstride;
+  f += blockIdx.y * fstride;
+  r += blockIdx.y * fstride;
+  double amax = 0.0;
+  if (p < npts) {
+    const int i = d == 1 ? p : p % n, j = d == 1 ? 0 : p / n;
+    const bool w = i > 0, e = i < n - 1, s = d == 2 && j > 0, t = d == 2 && j < n - 1;
+    const size_t nM = (size_t)n * M;
+    auto ld = [](const double* q) { return *reinterpret_cast<const double2*>(q); };
+    for (int m = 2 * (threadIdx.x & (tpl - 1)); m < M; m += 2 * tpl) {
+      const size_t at = (size_t)p * M + m;
+      const double2 c = ld(u + at), fv = ld(f + at), y = ld(r + at);
+      const double2 z = make_double2(0.0, 0.0);
+      const double2 qw = w ? ld(u + at - M) : z, qe = e ? ld(u + at + M) : z;
+      double2 sum = make_double2((c.x - qw.x) + (c.x - qe.x), (c.y - qw.y) + (c.y - qe.y));
+      if (d == 2) {
+        const double2 qs = s ? ld(u + at - nM) : z, qt = t ? ld(u + at + nM) : z;
+        sum.x += (c.x - qs.x) + (c.x - qt.x);
+        sum.y += (c.y - qs.y) + (c.y - qt.y);
+      }
+      const double2 out = make_double2((fv.x - y.x) - hinv2 * sum.x, (fv.y - y.y) - hinv2 * sum.y);
+      *reinterpret_cast<double2*>(r + at) = out;
+      amax = absmax_nan(fabs(out.x), absmax_nan(fabs(out.y), amax));
+    }
+  }
+  if (norm_bits == nullptr) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) amax = absmax_nan(__shfl_xor_sync(0xffffffffu, amax, o), amax);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int x = 1; x < 8; ++x) amax = absmax_nan(red[x], amax);
+    atomic_max_nonneg(norm_bits + blockIdx.y, amax);
+  }
+}
+
 }  // namespace
 
 size_t toep_band_bytes(int M) { return blob_bytes(M); }
@@ -871,8 +944,8 @@ cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, siz
 }
 
 size_t toep_scratch_bytes(const LevelShape& ls) {
-  // no slab of any colour or group size holds more lines than this
-  const size_t pts = (size_t)colour_count(ls.d, ls.n, 0);
+  // no slab of any launch or group size holds more lines than this
+  const size_t pts = (size_t)(ls.d == 1 ? ls.n : ls.n * ls.n);
   size_t lines = ((pts + 31) / 32 * 32) * ls.batch;
   const size_t per = (size_t)ls.M * kLineValue;
   const size_t most = kSlabBytes / per + 32;
@@ -915,18 +988,36 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
 #undef MGWR_DIRECT
     return counted(cudaGetLastError());
   }
-  const int NL = lines_per_group(ls.M, npts, ls.batch);
-  G.per_inst = (npts + NL - 1) / NL;
-  const int total = G.per_inst * ls.batch;
-  const int step = slab_groups(ls.M, NL, total);
-  for (int g0 = 0; g0 < total; g0 += step) {
-    G.group0 = g0;
-    G.groups = total - g0 < step ? total - g0 : step;
-    const cudaError_t e = NL == 32 ? slab_launch<32>(f, u, delta, band, scratch, G, hinv2, s)
-                                   : slab_launch<16>(f, u, delta, band, scratch, G, hinv2, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return product(f, u, delta, band, scratch, G, ls.batch, hinv2, s);
+}
+
+bool toep_defect(const LevelShape& ls) {
+  const long long lines = (long long)(ls.d == 1 ? ls.n : ls.n * ls.n) * ls.batch;
+  return toep_length(ls.M) && lines * ls.M * ls.M / 2 > kDirectWork;
+}
+
+cudaError_t launch_defect_toep(const double* u, const double* f, double* r,
+                               const unsigned char* band, unsigned char* scratch,
+                               const LevelShape& ls, double hinv2, unsigned long long* norm_bits,
+                               cudaStream_t s) {
+  if (!toep_length(ls.M)) return cudaErrorInvalidValue;
+  if (ls.batch == 0) return cudaSuccess;
+  Geometry G;
+  G.d = ls.d;
+  G.n = ls.n;
+  G.M = ls.M;
+  G.par = -1;
+  G.npts = ls.d == 1 ? ls.n : ls.n * ls.n;
+  G.fstride = ls.field_stride();
+  G.bstride = blob_bytes(ls.M);
+  G.zero_u = false;
+  const cudaError_t e = product(u, r, nullptr, band, scratch, G, ls.batch, 0.0, s);
+  if (e != cudaSuccess) return e;
+  const int per = ls.M / 2, tpl = per < 64 ? per : 64;
+  const unsigned blocks = (unsigned)((G.npts + 256 / tpl - 1) / (256 / tpl));
+  k_defect_finish<<<dim3(blocks, (unsigned)ls.batch), 256, 0, s>>>(
+      u, f, r, ls.d, ls.n, ls.M, ilog2(tpl), G.npts, hinv2, norm_bits, G.fstride);
+  return counted(cudaGetLastError());
 }
 
 cudaError_t take_toep_timeout(bool* hit) {
