@@ -38,17 +38,17 @@
 // slice that is not zero from a lag on is recorded per 64 lags at set-up, and
 // the slices before it are neither loaded nor multiplied (on a fine level about
 // half the products remain).
-// Lines are processed in slabs whose digits stay in L2 between the kernels.
+// Lines are processed in slabs, which bounds the digits' memory.
 //
 // Warp roles in k_toep_mma: warps 0-15 fold and store (tcgen05.ld), warp 16 loads
 // chunks of digits by bulk copies into a ring, warps 17 and 18 issue the MMAs; the
 // accumulator is double-buffered (2 x 8 NL columns).  Every wait is bounded.
 //
-// Measured (2-D, finest half-sweep, alpha = 0.5; slabs of 64 MB): 255 x 255, M =
-// 1024: FFT form 4.8 ms; 8 slabs of k_toep_gather 43 us (28 us of it FP64 sums at
-// the pipe's rate) and k_toep_mma 88 us: 1.05 ms.  Without its MMAs k_toep_mma takes
-// 69 us (folding: seven conversions a value and segment at a quarter of the rate,
-// tcgen05.ld latency, and the hand-overs of about 18 chunks an item).
+// Measured (2-D, finest half-sweep, alpha = 0.5; 255 x 255, M = 1024): FFT form
+// 4.8 ms; k_toep_gather 0.34 ms (0.22 ms of it FP64 sums at the pipe's rate) and
+// k_toep_mma 0.58 ms.  What k_toep_mma takes is folding (seven conversions a value and
+// segment at a quarter of the rate, tcgen05.ld latency) and the hand-overs of about
+// 18 chunks an item: without its MMAs it is a fifth faster.
 //
 // Where there are too few lines to fill the chip the product is a sum of FP64
 // products (k_toep_direct): one launch, 6 us for one line of 512 steps (FFT form
@@ -796,8 +796,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                  : "memory");
 }
 
-// Bytes of a slab's digits: what stays in L2 (129 MB) from one kernel to the next.
-constexpr size_t kSlabBytes = size_t(64) << 20;
+// Bytes of a slab's digits.  Both kernels are bound by arithmetic, so writing the digits
+// to HBM and reading them back costs nothing, while every slab leaves SMs idle at the
+// end of two launches: 255 x 255 x 1024 solves with slabs of 32, 64, 128, 256 and 600 MB
+// (the last: one slab) take 101, 87, 82.3, 79.2 and 78.8 ms.
+constexpr size_t kSlabBytes = size_t(256) << 20;
 constexpr size_t kLineValue = 2 * kSlices;  // bytes of digits per value
 
 // Lines per group: 32, or 16 while that leaves SMs without an item.
