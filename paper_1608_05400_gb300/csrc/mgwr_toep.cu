@@ -51,8 +51,8 @@
 // 18 chunks an item: without its MMAs it is a fifth faster.
 //
 // Where there are too few lines to fill the chip the product is a sum of FP64
-// products (k_toep_direct): one launch, 6 us for one line of 512 steps (FFT form
-// 26 us, the tensor-core pair 22 us).
+// products (k_toep_direct): one launch, 4.5 us for one line of 512 steps (FFT form
+// 26 us, the tensor-core pair 17 us).
 #include <cuda_fp16.h>
 
 #include <climits>
@@ -394,22 +394,27 @@ __global__ void __launch_bounds__(512, 3)
 }
 
 // Few lines: the product as FP64 sums.  A block holds OB output steps of one
-// line, 256 / OB threads per step; b up to the last of them in shared memory.
+// line from its end and OB from its start (so all blocks sum the same number of
+// terms); a warp's lanes are the steps (and 32 / OB phases of the sum), its eight
+// warps share the sum, and b up to the last step is in shared memory.  FP64 issue
+// bounds it (two operations a clock and SM).  With the lanes of a step reducing by
+// shuffles, and one tile a block, the reductions took as much of the pipe as the
+// products: 16 lines of 512 steps 13.6 us, now 7.7 us; 25 lines 16.6, now 11.6 us.
 template <int OB>
 __global__ void __launch_bounds__(256)
     k_toep_direct(const double* __restrict__ f, double* __restrict__ u, double* __restrict__ delta,
                   const double* __restrict__ cols, size_t cstride, Geometry G, double hinv2) {
-  constexpr int LPO = 256 / OB;
-  __shared__ double sb[1024], sk[1024];
-  const int inst = blockIdx.y / G.npts;
-  const int k = blockIdx.y - inst * G.npts;
+  constexpr int kTerms = 256 / OB;  // terms of the sums that the block takes at a time
+  __shared__ double sb[1024], sk[1024], part[512];
   const int M = G.M;
-  const int t0 = (gridDim.x - 1 - blockIdx.x) * OB;  // longest sums first
+  const int inst = blockIdx.x / G.npts;
+  const int k = blockIdx.x - inst * G.npts;
   int i = 0, j = 0;
   const int p = colour_point(k, G.d, G.n, G.par, i, j);
   const size_t base = inst * G.fstride + (size_t)p * M;
+  const int first[2] = {M - OB - (int)blockIdx.y * OB, (int)blockIdx.y * OB};
   cols += inst * cstride;
-  for (int m = 2 * threadIdx.x; m < t0 + OB; m += 512) {
+  for (int m = 2 * threadIdx.x; m < first[0] + OB; m += 512) {
     double b[2];
     gather_steps<2>(f, u, base + m, M, (size_t)G.n * M, i > 0 && !G.zero_u,
                     i < G.n - 1 && !G.zero_u, G.d == 2 && j > 0 && !G.zero_u,
@@ -421,21 +426,37 @@ __global__ void __launch_bounds__(256)
     sk[m + 1] = c.y;
   }
   __syncthreads();
-  const int t = t0 + threadIdx.x / LPO;
-  const int lane = threadIdx.x % LPO;
-  double a[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int s = lane; s < t; s += 4 * LPO) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (s + q * LPO < t) a[q] = fma(sk[t - s - q * LPO], sb[s + q * LPO], a[q]);
+  for (int h = 0; h < 2; ++h) {
+    const int t0 = first[h], t = t0 + threadIdx.x % OB;
+    double a[2] = {0.0, 0.0};
+    int s = threadIdx.x / OB;
+#pragma unroll 2
+    for (; s + kTerms < t0; s += 2 * kTerms) {
+      a[0] = fma(sk[t - s], sb[s], a[0]);
+      a[1] = fma(sk[t - s - kTerms], sb[s + kTerms], a[1]);
+    }
+    for (; s < t0 + OB; s += kTerms)
+      if (s < t) a[0] = fma(sk[t - s], sb[s], a[0]);
+    part[256 * h + threadIdx.x] = a[0] + a[1];
   }
-  double y = (a[0] + a[1]) + (a[2] + a[3]);
+  __syncthreads();
+  if (threadIdx.x >= 64) return;
+  const int lane = threadIdx.x & 31, h = threadIdx.x >> 5;
+  const int t = (h == 0 ? first[0] : first[1]) + lane % OB;
+  double y[8];
 #pragma unroll
-  for (int o = LPO / 2; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-  y = fma(sk[0], sb[t], y);  // the largest product last
-  if (lane == 0) {
-    if (delta != nullptr) delta[base + t] = y - u[base + t];
-    u[base + t] = y;
+  for (int w = 0; w < 8; ++w) y[w] = part[256 * h + 32 * w + lane];
+#pragma unroll
+  for (int x = 4; x > 0; x >>= 1)
+#pragma unroll
+    for (int w = 0; w < x; ++w) y[w] += y[w + x];
+#pragma unroll
+  for (int o = OB; o < 32; o <<= 1) y[0] += __shfl_xor_sync(0xffffffffu, y[0], o);
+  y[0] = fma(sk[0], sb[t], y[0]);  // the largest product last
+  if (lane < OB) {
+    if (delta != nullptr) delta[base + t] = y[0] - u[base + t];
+    u[base + t] = y[0];
   }
 }
 
@@ -867,11 +888,33 @@ cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigne
   return counted(cudaGetLastError());
 }
 
-// Multiply-adds up to which the FP64 sums run (the chip does 304 a clock, 14000
-// clocks in all).  Measured at M = 512: 25 lines (3.3 M) 17 us by sums, 21 us by
-// the tensor-core pair, which takes as long for any grid up to one item per SM;
-// 31 lines (4.1 M) 23 against 21 us.
-constexpr long long kDirectWork = 1ll << 22;
+// Few lines: the FP64 sums (about 4 us + 2 us a million multiply-adds) instead of
+// the tensor-core pair (11.6, 12.5, 14.3, 17.8 and 23.3 us at M = 64 .. 1024 for any
+// grid up to one item per SM, and a second launch).  Measured, sums against pair
+// without that launch: M = 64, 481 lines (1.0 M) 7.5 / 11.5 us; M = 256, 128 lines
+// (4.2 M) 14.0 / 14.3; M = 512, 32 lines (4.2 M) 12.5 / 17.8, 64 lines (8.4 M) 22.7 /
+// 17.8; M = 1024, 16 lines (8.4 M) 21.3 / 23.3, 32 lines 40 / 23.3.
+bool few_lines(long long lines, int M) {
+  return lines * M * M / 2 <= (1ll << 21) + (1ll << 13) * M;
+}
+
+// Steps per tile of the FP64 sums: the one whose rounds of blocks (one per SM) take
+// least, a block costing its tile's sums and about five steps' worth for the rest
+// (M = 512, tiles of 8, 16, 32: 4 lines 4.7, 5.6, 7.6 us; 8 lines 6.3, 5.7, 7.6;
+// 16 lines 10.3, 8.4, 7.7; 25 lines 14.1, 11.6, 12.6).
+int direct_tile(long long lines, int M) {
+  int best = 0;
+  long long least = 0;
+  for (int tile = 8; tile <= 32; tile *= 2) {
+    const long long rounds = (lines * (M / (2 * tile)) + sm_count() - 1) / sm_count();
+    const long long cost = rounds * (tile + 5);
+    if (best == 0 || cost < least) {
+      best = tile;
+      least = cost;
+    }
+  }
+  return best;
+}
 
 // Every line of a launch, in slabs of groups.
 cudaError_t product(const double* f, double* u, double* delta, const unsigned char* band,
@@ -973,18 +1016,16 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
   G.bstride = bstride;
   G.zero_u = zero_u;
   const long long lines = (long long)npts * ls.batch;
-  if (lines * ls.M * ls.M / 2 <= kDirectWork && lines <= 65535) {
+  if (few_lines(lines, ls.M)) {
     G.per_inst = G.group0 = G.groups = 0;
-    // fewest steps a block (shortest sums per block, but every block gathers its
-    // line up to its last step) with at most two blocks per SM; by the instance's
-    // lines, so that a batch sums as one instance does
-    const long long values = (long long)npts * ls.M, blocks = 2 * sm_count();
 #define MGWR_DIRECT(OB)                                                                     \
-  k_toep_direct<OB><<<dim3(ls.M / OB, (unsigned)lines), 256, 0, s>>>(f, u, delta, cols, cstride, \
-                                                                     G, hinv2)
-    if (values / 8 <= blocks)
+  k_toep_direct<OB><<<dim3((unsigned)lines, ls.M / (2 * OB)), 256, 0, s>>>(f, u, delta, cols, \
+                                                                           cstride, G, hinv2)
+    // by one instance's lines, so that a batch sums as one instance does
+    const int tile = direct_tile(npts, ls.M);
+    if (tile == 8)
       MGWR_DIRECT(8);
-    else if (values / 16 <= blocks)
+    else if (tile == 16)
       MGWR_DIRECT(16);
     else
       MGWR_DIRECT(32);
@@ -994,9 +1035,10 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
   return product(f, u, delta, band, scratch, G, ls.batch, hinv2, s);
 }
 
+// Few lines keep the transform's defect (one launch).
 bool toep_defect(const LevelShape& ls) {
   const long long lines = (long long)(ls.d == 1 ? ls.n : ls.n * ls.n) * ls.batch;
-  return toep_length(ls.M) && lines * ls.M * ls.M / 2 > kDirectWork;
+  return toep_length(ls.M) && lines * ls.M * ls.M / 2 > (1ll << 22);
 }
 
 cudaError_t launch_defect_toep(const double* u, const double* f, double* r,

@@ -4,8 +4,8 @@ FP64 sums where the lines are few) against sums in extended precision.
 Bounds, against S = sum |k| |b| of a value (b the gathered line, k the inverse column):
   * sliced: b keeps 59 bits below its largest operand, the dropped products are below
     2^-59 (largest |k|) (largest |b|), the total is rounded once: 4e-16 of the largest S and b.
-  * FP64 sums: b rounded five times, at most 32 products a thread in four chains, five shuffles:
-    about twenty roundings, 20 * 2^-53 = 2.3e-15.
+  * FP64 sums: b rounded five times, at most M / 16 products a thread in a chain of sums, eight
+    sums of the chains' results and two of what is left: (M / 16 + 15) * 2^-53.
 """
 import numpy as np
 import pytest
@@ -15,6 +15,14 @@ from paper_1608_05400_gb300 import mgwr as G
 
 pytestmark = pytest.mark.gpu
 Q = np.longdouble
+
+
+def _sums(lines, M):  # the rule that takes few lines to the FP64 sums
+    return lines * M * M // 2 <= (1 << 21) + (1 << 13) * M
+
+
+def _bound(lines, M):
+    return (M / 16 + 15) * 2.0 ** -53 if _sums(lines, M) else 4e-16
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -59,7 +67,7 @@ def _check(s, d, n, M, colour, u, f, batch, sample, bound):
             assert float(err.max()) <= bound * float(scale.max()), (b, p, float(err.max() / scale.max()))
 
 
-# (d, n, M, batch): the two forms on both sides of their boundary (2^22 products), groups of 16
+# (d, n, M, batch): the two forms on both sides of their boundary, groups of 16
 # and of 32 lines, partly filled groups, several slabs, the shortest and the longest lines, and
 # instances with columns of their own
 @pytest.mark.parametrize("d,n,M,batch", [
@@ -82,7 +90,7 @@ def test_half_sweep_against_extended_sums(d, n, M, batch, data):
         u, f = (rng.uniform(-1, 1, (batch, N, M)) * 10.0 ** rng.uniform(-12, 0, (batch, N, M))
                 for _ in range(2))
     lines = len(_points(d, n, G.MGWR_BLACK if n == 1 and d == 1 else G.MGWR_RED)) * batch
-    bound = 2.3e-15 if lines * M * M // 2 <= 1 << 22 else 4e-16
+    bound = _bound(lines, M)
     alphas = 0.45 if batch == 1 else list(np.linspace(0.15, 0.95, batch))
     with G.Solver(d, n, M, 1.0, alphas) as s:
         colour = G.MGWR_RED
@@ -128,3 +136,37 @@ def test_infinities_and_nan_reach_the_solver(bad):
             s.field_set(G.MGWR_H64, l, G.MGWR_U, np.zeros_like(f))
             s.smooth(G.MGWR_H64, l, G.MGWR_RED)
             assert not np.isfinite(s.field_get(G.MGWR_H64, l, G.MGWR_U)[n // 2]).all()
+
+
+# one, three and the most lines of the FP64 sums, which take tiles of 8, 16 and 32 steps between
+# them; f alone (u = 0) so that the reference is a plain convolution
+@pytest.mark.parametrize("M", [64, 128, 256, 512, 1024])
+def test_sums_at_the_edges_of_their_tiles(M):
+    sizes = [3, 7, 15, 31, 63, 127, 255, 511, 1023]
+    few = [n for n in sizes if _sums(n // 2, M)]
+    for n in (few[0], few[1], few[2], few[-2], few[-1]):
+        f = inputs.random_field(n, M, n)
+        with G.Solver(1, n, M, 1.0, 0.35) as s:
+            _check(s, 1, n, M, G.MGWR_RED, np.zeros((1, n, M)), f[None], 1, (0.0, 0.5, 1.0),
+                   _bound(n // 2, M))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("n,M", [(4095, 64), (511, 256), (127, 1024)])
+def test_non_finite_values_stay_in_their_line_of_a_sliced_sweep(n, M, bad):
+    assert not _sums(n // 2, M)
+    f = inputs.random_field(n, M, 5)
+    hit = n // 2 | 1
+    f[hit, M // 3] = bad
+    with G.Solver(1, n, M, 1.0, 0.5) as s:
+        l = s.num_levels() - 1
+        s.field_set(G.MGWR_H64, l, G.MGWR_F, f)
+        s.field_set(G.MGWR_H64, l, G.MGWR_U, np.zeros_like(f))
+        s.smooth(G.MGWR_H64, l, G.MGWR_RED)
+        got = s.field_get(G.MGWR_H64, l, G.MGWR_U)
+        assert not np.isfinite(got[hit]).all()
+        assert np.isfinite(np.delete(got, hit, axis=0)).all()
+        with pytest.raises(G.MGWRError) as e:
+            s.set_rhs(f)
+            s.solve(1, 1, 1, tol=1e-10, max_cycles=5)
+        assert e.value.status == G.MGWR_E_NUMERIC
