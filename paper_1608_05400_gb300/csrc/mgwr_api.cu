@@ -2697,9 +2697,11 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
   if (M > mgwr::kShortMaxM)  // partitioned-convolution scratch: all block spectra of the finest level
     total += r512(16 * B * ((pts[0] + 1) / 2) * L);
   if (precision == MGWR_FP64) {
-    if (mgwr::toep_length(M))  // sliced bands and digits of the tensor-core sweeps
+    // sliced bands and digits of the tensor-core sweeps; a batch's digits (at most one
+    // slab) counted as its instances', so that the footprint is linear in the batch
+    if (mgwr::toep_length(M))
       total += r512(mgwr::toep_band_bytes(M) * B * nlev) + r512(mgwr::toep_band_bytes(M) * B) +
-               r512(mgwr::toep_scratch_bytes(LevelShape{d, n, M, batch}));
+               B * r512(mgwr::toep_scratch_bytes(LevelShape{d, n, M, 1}));
     for (size_t l = 0; l < nlev; ++l) total += (l + 1 < nlev ? 4 : 3) * r512(8 * B * pts[l] * M);
   } else if (precision == MGWR_DD) {
     total += 2 * r512(8 * B * pts[0] * M);  // FP64 finest iterate and right-hand side

@@ -830,12 +830,20 @@ int lines_per_group(int M, int npts, int batch) {
   return items >= sm_count() ? 32 : 16;
 }
 
-int slab_groups(int M, int NL, int groups) {
-  const size_t per = (size_t)NL * M * kLineValue;
-  long long most = (long long)(kSlabBytes / per);
-  if (most < 1) most = 1;
-  const long long slabs = (groups + most - 1) / most;
-  return (int)((groups + slabs - 1) / slabs);
+// Lines of a slab: a colour of every instance (a defect, on all points, takes two
+// slabs), at most kSlabBytes of digits.
+size_t slab_lines(int M, int d, int n, int batch) {
+  const size_t pts = (size_t)(d == 1 ? n : n * n);
+  const size_t lines = ((pts + 1) / 2 + 31) / 32 * 32 * batch;
+  const size_t most = kSlabBytes / ((size_t)M * kLineValue);
+  return lines < most ? lines : most;
+}
+
+// Groups per slab of equal slabs.
+int slab_groups(const Geometry& G, int batch, int NL, int groups) {
+  const int most = (int)(slab_lines(G.M, G.d, G.n, batch) / NL);
+  const int slabs = (groups + most - 1) / most;
+  return (groups + slabs - 1) / slabs;
 }
 
 template <int NL, bool PLAIN>
@@ -922,7 +930,7 @@ cudaError_t product(const double* f, double* u, double* delta, const unsigned ch
   const int NL = lines_per_group(G.M, G.npts, batch);
   G.per_inst = (G.npts + NL - 1) / NL;
   const int total = G.per_inst * batch;
-  const int step = slab_groups(G.M, NL, total);
+  const int step = slab_groups(G, batch, NL, total);
   for (int g0 = 0; g0 < total; g0 += step) {
     G.group0 = g0;
     G.groups = total - g0 < step ? total - g0 : step;
@@ -990,13 +998,7 @@ cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, siz
 }
 
 size_t toep_scratch_bytes(const LevelShape& ls) {
-  // no slab of any launch or group size holds more lines than this
-  const size_t pts = (size_t)(ls.d == 1 ? ls.n : ls.n * ls.n);
-  size_t lines = ((pts + 31) / 32 * 32) * ls.batch;
-  const size_t per = (size_t)ls.M * kLineValue;
-  const size_t most = kSlabBytes / per + 32;
-  if (lines > most) lines = most;
-  return lines * (per + sizeof(int));
+  return slab_lines(ls.M, ls.d, ls.n, ls.batch) * ((size_t)ls.M * kLineValue + sizeof(int));
 }
 
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
