@@ -210,8 +210,8 @@ int mgwr_set_outer_switch(mgwr_t h, double rel);
  * group fits in one warp.  A request a length cannot take falls back to the
  * nearest smaller E; mgwr_get_engine_split reports the E launches use.  The
  * FP64 half-sweeps of 64 .. 1024 steps have one form, whatever E is set.
- * MGWR_K_SWEEP32 that was neither set nor tuned takes the form measured
- * fastest for the line length and the lines of the launch (one of those below).
+ * MGWR_K_SWEEP32 that was neither set nor tuned takes E = 1 or 2, by the line
+ * length and the lines of the launch.
  * For MGWR_K_SWEEP32 (not the one-point solve) with 64 <= M <= 4096, `split`
  * may also be E | MGWR_SPLIT_STAGED: a persistent kernel whose thread groups
  * receive the f and neighbour lines of their next line pair in shared memory

@@ -459,30 +459,19 @@ void prof_collect(mgwr_t h) {
 
 // ---- Algorithm 1 components ------------------------------------------------------
 
-// The form of an FP32 half-sweep whose split was neither set nor tuned, by the line
-// length and the line pairs of the launch (all instances).  Measured, us per
-// half-sweep (radix-8 E = 1 / E = 2 / register-pass single / resident):
-//   values >= 3 2^18: the resident register-pass form.  M = 256, 4033 pairs: 19.6 /
-//     19.9 / 18.9 / 14.2; M = 1024, 993: 22.9 / 22.6 / 19.2 / 16.6, 16257: 258 / 241 /
-//     198 / 160; M = 2048, 512: 26.6 / 22.7 / 20.5 / 17.5; M = 4096, 4033: 431 / 348 /
-//     229 / 205.  Below, its one block per SM has too few pairs: M = 1024, 241 pairs:
-//     13.1 / 11.3 / 14.9 / 17.0; M = 512, 993: 16.6 / 14.5 / 14.0 / 17.0.
-//   M = 4096: single register passes at every size (13 pairs 21.1 / 17.5 / 14.9 / 19.3).
-//   else E = 2 for M = 2048 and 4096 (13.5 / 11.4 / 15.1 / 17.5) and from 200
-//     thousand values of M >= 512, E = 1 for the rest (M = 256, 57 pairs: 8.3 / 9.5 /
-//     12.5 / 12.7).
-// The register passes round differently from the radix-8 forms.  The finer the
-// grid, the more of a solution to 1e-8 is FP32 rounding: that difference is 4e-11
-// of it at h = 1/256, 4e-10 at 1/512 and 1e-9, as large as its error, at 1/2048.
-// Handles finer than 1/256 keep the radix-8 forms unless they are tuned.
-int default_sweep32(const mgwr_handle* h, const LevelShape& ls) {
+// E of an FP32 half-sweep whose split was neither set nor tuned, by the line length
+// and the line pairs of the launch (all instances): 2 for M = 2048 and 4096 and from
+// 200 thousand values of M >= 512, 1 for the rest.  Measured, us per half-sweep, E = 1
+// / E = 2: M = 4096, 4033 pairs 431 / 348, 13 pairs 21.1 / 17.5; M = 2048, 512: 26.6 /
+// 22.7; M = 1024, 16257: 258 / 241, 241: 13.1 / 11.3; M = 512, 993: 16.6 / 14.5;
+// M = 256, 4033: 19.6 / 19.9, 57: 8.3 / 9.5.  The register-pass forms are faster for
+// many lines (M = 1024, 16257 pairs: 160), but they round differently, and another
+// rounding moves a solution to 1e-8 by up to 1e-9 of itself (2-D 255 x 255 x 1024):
+// only handles that are tuned or set take them.
+int default_sweep32(const LevelShape& ls) {
   const int M = ls.M;
   const long long pts = ls.d == 1 ? ls.n : (long long)ls.n * ls.n;
   const long long values = ((pts + 1) / 2 + 1) / 2 * ls.batch * M;
-  if (pts > 1 && h->n <= 255 && mgwr::radix_length(M)) {
-    if (values >= 3ll << 18) return mgwr::kRpResident | mgwr::kRadix;
-    if (M == 4096) return mgwr::kRpSingle | mgwr::kRadix;
-  }
   if (M > mgwr::kShortMaxM) return 1;
   return M >= 2048 || (M >= 512 && values >= 200000) ? 2 : 1;
 }
@@ -503,7 +492,7 @@ cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
     }
   }
   if constexpr (std::is_same<R, float>::value) {
-    if (E == 0) E = default_sweep32(h, ls);
+    if (E == 0) E = default_sweep32(ls);
     const int eff = mgwr::effective_split(h->M, 4, E);
     if ((eff & mgwr::kTensor) && h->tc_band != nullptr) {
       const size_t bb = mgwr::tc_band_bytes(h->M);
@@ -533,7 +522,7 @@ int coarsest(mgwr_t h, Hier<R>& H) {
     }
   }
   int E = split_of(h, sweep_class<R>(), 0);
-  if (std::is_same<R, float>::value && E == 0) E = default_sweep32(h, shape(h, 0));
+  if (std::is_same<R, float>::value && E == 0) E = default_sweep32(shape(h, 0));
   MGWR_CK(h, mgwr::launch_sweep<R>(H.f[0], H.u[0], (R*)nullptr, H.spec, (size_t)h->nlev * h->L,
                                     H.tw, H.zero, scratch_for<R>(h), shape(h, 0), 0, true, R(0),
                                     E & ~(mgwr::kTensor | mgwr::kRadix), h->stream));
@@ -1626,7 +1615,7 @@ int mgwr_get_engine_split(mgwr_t h, int kernel_class, int level, int* split) {
   const int word = kernel_class == MGWR_K_SWEEP32 || kernel_class == MGWR_K_DEFECT32 ? 4 : 8;
   const int l = level == -1 ? h->nlev - 1 : level;
   int E = split_of(h, kernel_class, l);
-  if (E == 0 && kernel_class == MGWR_K_SWEEP32) E = default_sweep32(h, shape(h, l));
+  if (E == 0 && kernel_class == MGWR_K_SWEEP32) E = default_sweep32(shape(h, l));
   *split = mgwr::effective_split(h->M, word, E);
   return MGWR_OK;
 }
