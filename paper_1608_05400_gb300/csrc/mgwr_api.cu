@@ -104,6 +104,7 @@ struct mgwr_handle {
   unsigned char* toep_band = nullptr;
   unsigned char* toep_tband = nullptr;  // the same of the Toeplitz columns (FP64 defects)
   unsigned char* toep_scratch = nullptr;
+  bool toep_off = false;  // no memory for them
   double* c_dev = nullptr;      // batch
   Hier<double> h64;
   Hier<float> h32;
@@ -253,7 +254,7 @@ int check_staging(mgwr_t h) {
   bool hit = false;
   if (h->toep_band != nullptr) {
     MGWR_CK(h, mgwr::take_toep_timeout(&hit));
-    if (hit) return fail(h, MGWR_E_CUDA, "sliced sweep: wait for its copies or MMAs gave up");
+    if (hit) return fail(h, MGWR_E_CUDA, "sliced product: wait for its copies or MMAs gave up");
   }
   MGWR_CK(h, mgwr::take_stage_timeout(&hit));
   if (hit) return fail(h, MGWR_E_CUDA, "staged sweep: wait for bulk copies gave up");
@@ -368,17 +369,29 @@ int ensure_h32(mgwr_t h) {
 // The sliced bands of the FP64 half-sweeps on the tensor cores and their
 // scratch (before any capture that runs them).
 int ensure_toep(mgwr_t h) {
-  if (h->toep_band != nullptr || !mgwr::toep_length(h->M)) return MGWR_OK;
+  if (h->toep_band != nullptr || h->toep_off || !mgwr::toep_length(h->M)) return MGWR_OK;
   const size_t lines = (size_t)h->B * h->nlev;
-  if (h->toep_scratch == nullptr)
-    MGWR_TRY(dev_alloc(h, &h->toep_scratch, mgwr::toep_scratch_bytes(shape(h, h->nlev - 1))));
-  if (h->toep_tband == nullptr)
-    MGWR_TRY(dev_alloc(h, &h->toep_tband, mgwr::toep_band_bytes(h->M) * (size_t)h->B));
-  unsigned char* band = nullptr;
-  MGWR_TRY(dev_alloc(h, &band, mgwr::toep_band_bytes(h->M) * lines));
-  MGWR_CK(h, mgwr::launch_toep_band(h->kcol, band, h->M, lines, h->stream));
-  MGWR_CK(h, mgwr::launch_toep_band(h->r, h->toep_tband, h->M, (size_t)h->B, h->stream));
-  h->toep_band = band;
+  unsigned char* part[3] = {};
+  const size_t bytes[3] = {mgwr::toep_scratch_bytes(shape(h, h->nlev - 1)),
+                           mgwr::toep_band_bytes(h->M) * (size_t)h->B,
+                           mgwr::toep_band_bytes(h->M) * lines};
+  for (int k = 0; k < 3; ++k) {
+    if (dev_alloc(h, &part[k], bytes[k]) == MGWR_OK) continue;
+    // no room: this handle keeps the transforms
+    for (unsigned char* p : part) {
+      if (p == nullptr) continue;
+      cudaFreeAsync(p, h->stream);
+      h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)p));
+    }
+    h->err.clear();
+    h->toep_off = true;
+    return MGWR_OK;
+  }
+  MGWR_CK(h, mgwr::launch_toep_band(h->kcol, part[2], h->M, lines, h->stream));
+  MGWR_CK(h, mgwr::launch_toep_band(h->r, part[1], h->M, (size_t)h->B, h->stream));
+  h->toep_scratch = part[0];
+  h->toep_tband = part[1];
+  h->toep_band = part[2];
   return MGWR_OK;
 }
 
