@@ -95,10 +95,10 @@ FP64_FMA_PER_CLK_PER_SM = 2
 SMS = 152
 # FP32 lanes of a GB300 SM (4 partitions x 32)
 FP32_LANES_PER_SM = 128
-# DRAM bytes (read + write) per smoothed line of k_sweep<double> from an ncu
-# capture of the finest-level half-sweep of the default workload (772.5 MB for
-# 32,513 lines of 1024 doubles; profiles/k_sweep_fp64_2d_255x255_M1024.md).
-SWEEP64_DRAM_BYTES_PER_LINE_M1024 = 23758.0
+# DRAM bytes (read + write) per smoothed line of the FP64 half-sweep as sliced products,
+# from an ncu capture of k_toep_gather (132.2 + 89.8 MB) and k_toep_mma (199.4 + 36.6 MB) on
+# 8064 lines of 1024 steps (profiles/k_toep_fp64_2d_127x127_M1024.md).
+SWEEP64_DRAM_BYTES_PER_LINE_M1024 = 56800.0
 # DRAM bytes per line of further kernels from single-kernel ncu captures (see
 # profiles/), by kernel class and M
 # (k_defect<double, float>: 1059.1 MB read + 254.9 MB written for 16,129 lines of 4096,
@@ -348,8 +348,9 @@ CLASS_KERNELS = {
 
 def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
     """Roofline of one kernel class from its summed event-timed launches: the
-    FP64 kernels against the FP64 ALU peak (GB300 runs FP64 at 1/64 of FP32),
-    the FP32 and line kernels against HBM with the FP32-issue view beside."""
+    FP64 kernels against the FP64 ALU peak (GB300 runs FP64 at 1/64 of FP32) or,
+    where lines of 64 .. 1024 steps run as sliced products, against the tensor
+    peak; the FP32 and line kernels against HBM with the FP32-issue view beside."""
     secs = p["ms"] * 1e-3
     name, word, kind = CLASS_KERNELS.get(cls, (cls, 8, "line"))
     long = M > 4096
@@ -376,7 +377,17 @@ def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
            "avg_launch_ms": p["ms"] / max(p["launches"], 1),
            "lines_per_launch": p["lines"] / max(p["launches"], 1),
            "bytes_per_line": bytes_per_line, "flops_per_line": per_line}
-    if cls in ("sweep64", "defect64"):
+    if cls in ("sweep64", "defect64") and 64 <= M <= 1024:
+        # 36 products of 8-bit slices per multiply-add of the triangle, in blocks of 128
+        # steps, those of zero slices at far lags included
+        per_line = 36.0 * M * (M + 128)
+        achieved, peak = p["lines"] * per_line / secs / 1e12, float(pk.get("bf16_tflops", 1900.0))
+        out.update({"kernel": "k_toep_gather + k_toep_mma (k_toep_direct on levels of few lines)",
+                    "flops_per_line": per_line, "bound": "tensor", "achieved": achieved,
+                    "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                    "peak_source": "measured (MEASURED_PEAKS.json bf16_tflops)",
+                    "hbm_view": {"achieved_gbs": hbm, "peak_gbs": hbm_peak, "frac": hbm / hbm_peak}})
+    elif cls in ("sweep64", "defect64"):
         peak = fp64_peak_tflops(pk)
         achieved = flops / secs / 1e12
         out.update({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -557,7 +568,7 @@ def run_nonlinear(args):
     sm_max = float(pk.get("sm_max_mhz", 2070.0))
     peak = SMS * FP64_FMA_PER_CLK_PER_SM * 2 * sm_max * 1e6 / 1e12
     fixed = line_iters > 0
-    flops = (line_iters * (conv_flops_per_line(Mw) + 20 * Mw) if fixed
+    flops = (line_iters * (Mw * (Mw + 1) + 20 * Mw) if fixed
              else lines * fas_line_flops(Mw))
     achieved = flops / (line_ms * 1e-3) / 1e12
 
@@ -604,13 +615,13 @@ def run_nonlinear(args):
         "solve": {"cycles": stats[-1].cycles, "relres": stats[-1].relres,
                   "factor": stats[-1].factor},
         "gpu_launches": launches,
-        "roofline": {"kernel": "k_fas_fixed" if fixed else "k_fas_line", "bound": "alu",
+        "roofline": {"kernel": "k_fas_fixed_sums" if fixed else "k_fas_line", "bound": "alu",
                      "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                      "peak_source": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x max SM clock",
                      "avg_launch_ms": line_ms, "lines_per_launch": lines,
                      "fixed_point_iterations_per_line": line_iters / lines if fixed else None,
-                     "note": ("whole-line fixed point: one FP64 FFT convolution per line and "
+                     "note": ("whole-line fixed point: FP64 sums of a line over a cluster of blocks per "
                               "iteration, a few hundred lines per launch (latency-bound)") if fixed
                      else "latency-bound: one warp per line marches M dependent Newton solves"},
         "clocks": clk.summary(),
