@@ -367,3 +367,21 @@ def test_solve_from_zero_skips_nothing_it_needs(precision):
     anchor = 2.0 ** -40 if precision == G.MGWR_MIXED else 0.0
     assert abs(out[0][3] - out[1][3]) <= 1e-6 * out[1][3] + anchor
     assert rel(out[0][0], direct.time_stepping(d, n, M, 1.0, 0.6, f)) <= (1e-11 if precision == G.MGWR_FP64 else 1e-8)
+
+
+# the norm of a convergence check (formed from the black changes, never stored) is the defect's:
+# lines shorter and longer than a group of threads, one red point, odd and even rows, a batch
+@pytest.mark.parametrize("d,n,M,batch", [(1, 3, 4, 1), (1, 63, 64, 1), (1, 127, 2048, 1),
+                                         (2, 3, 32, 1), (2, 31, 128, 3), (2, 15, 1024, 1)])
+def test_norm_of_a_check_is_that_of_the_full_defect(d, n, M, batch):
+    N = n ** d
+    f = np.stack([inputs.random_field(N, M, 40 + b) for b in range(batch)])
+    with G.Solver(d, n, M, 1.0, 0.6 if batch == 1 else [0.3, 0.6, 0.9]) as s:
+        l = s.num_levels() - 1
+        s.set_rhs(f if batch > 1 else f[0])
+        st = s.solve(1, 1, 1, tol=1e-14, max_cycles=2, allow_noconv=True)
+        s.defect(G.MGWR_H64, l)
+        r = s.field_get(G.MGWR_H64, l, G.MGWR_R).reshape(batch, -1)
+    per = np.abs(r).max(axis=1) / np.abs(f).reshape(batch, -1).max(axis=1)
+    # the full defect's rounding is below 1e-15 (8 / h^2) max |u| <= 1e-15 * max |f|-sized sums
+    assert abs(st.relres - per.max()) <= 1e-12
