@@ -262,8 +262,9 @@ __global__ void __launch_bounds__(BLOCK)
 // the sums cost M^2 / 4 clocks of it and spread over the cluster, M^2 / (4 C).
 // Block `rank` owns the steps t = rank mod C (equal shares of the triangle): it forms
 // their right-hand sides and hands them to the cluster's other blocks through
-// distributed shared memory (two buffers, one cluster barrier an iteration), then
-// sums its outputs with C threads each.  Settled per line by k_fas_fixed's rule; the
+// distributed shared memory (two buffers, one cluster barrier an iteration, one before
+// the first store, split so that it spans the loads), then sums its outputs with C
+// threads each.  Settled per line by k_fas_fixed's rule; the
 // largest change and value travel with the next iteration's right-hand sides, so
 // that all blocks decide alike.  With the neighbours fixed the right-hand side
 // f + sigma v - phi(v) is a cubic in v whose sigma terms cancel: three operations.
@@ -282,6 +283,9 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(1024)
   __shared__ unsigned long long most[2][C][2];
   __shared__ unsigned long long red[2][32];
   const cg::cluster_group cluster = cg::this_cluster();
+  // Another block's shared memory may be written only once that block runs: every
+  // block arrives here, and waits for the others before its first such store.
+  if (C > 1) cluster.barrier_arrive();
   const int rank = C == 1 ? 0 : (int)cluster.block_rank();
   double* const sk = sums_sm;          // the inverse column
   double* const sb = sums_sm + M;      // two buffers of right-hand sides
@@ -316,6 +320,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(1024)
   const int o = tid / C, lane = tid % C, to = o * C + rank;
   bool settled = false;
   double d_prev = 0.0;
+  if (C > 1) cluster.barrier_wait();
   int it = 0;
   for (;; ++it) {
     const int buf = it & 1;

@@ -293,3 +293,32 @@ def test_whole_line_smoother_equals_the_march_for_every_cluster_size(n, M, c):
                 s.smooth(l, colour)
             out.append(s.field_get(l, G.MGWR_U))
     assert np.abs(out[0] - out[1]).max() <= 1e-12 * np.abs(out[1]).max()
+
+
+# the first right-hand sides that the blocks of a cluster hand to one another, with the blocks'
+# starts spread by other work on the device: every repetition gives the same bits (8, 4 and 2
+# blocks per line)
+@pytest.mark.parametrize("n,M", [(7, 128), (31, 128), (63, 256), (127, 128)])
+def test_whole_line_smoother_repeats_its_bits_beside_other_work(n, M):
+    import torch
+    u0 = inputs.random_field(n, M, seed=43, scale=0.3)
+    f = inputs.random_field(n, M, seed=44, scale=50.0)
+    noise = torch.rand(1 << 22, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with G.FAS(n, M, 1.0, 0.6, c=1.0) as s:
+        s.set_smoother(G.MGWR_FAS_SMOOTHER_FIXED)
+        l = s.num_levels() - 1
+        out = []
+        for _ in range(12):
+            s.set_rhs(f)
+            s.set_initial(u0)
+            with torch.cuda.stream(side):
+                for _ in range(8):
+                    noise = noise * 0.5 + 0.25
+            for colour in (G.MGWR_RED, G.MGWR_BLACK):
+                s.smooth(l, colour)
+            out.append(s.field_get(l, G.MGWR_U))
+    torch.cuda.synchronize()
+    for o in out[1:]:
+        np.testing.assert_array_equal(o, out[0])
