@@ -26,9 +26,15 @@
 //                 written as fp16 in the layout the MMA reads (16 bytes a value);
 //  k_toep_mma     one CTA per SM.  An item is NL lines x 128 output steps: the
 //                 MMA's 128 rows are output steps, its columns the lines, once
-//                 per slice j, so one instruction multiplies slice i of the
-//                 column with slices 0 .. 7-i of the lines (N = NL (8 - i)) and
-//                 the accumulator columns of order i + j are adjacent.
+//                 per order p = i + j.  The orders 0 .. 3 and 4 .. 7 are an
+//                 accumulator each: one instruction multiplies slice i of the
+//                 column with the slices j = p - i of the lines for the four
+//                 orders of an accumulator (N = 4 NL; slices j < 0 are a pad of
+//                 zeros before the lines' slices).
+// The PTX ISA orders two tcgen05.mma only where both have the same accumulator and
+// the same shape (and come from one thread); others may overlap and lose a sum.  So
+// every MMA of an accumulator has one shape and one issuing thread.  The zeros cost
+// 48 blocks of four orders where the triangle i + j <= 7 has 36.
 // Because the time index of a chunk of 32 steps is stored reversed, element
 // (row, kk) of the Toeplitz operand depends on row + kk only, so its 8 x 8 core
 // matrices depend on one index and all blocks of all lags are windows into one
@@ -73,7 +79,8 @@ constexpr int kChunk = 32;     // time steps per shared-memory chunk (two K = 16
 constexpr int kMaxStages = 8;  // chunks in flight, as many as shared memory holds
 constexpr int kFoldThreads = 512;
 constexpr int kLoader = 512, kIssuer = 544;  // first threads of warps 16 and 17
-constexpr int kIssuers = kChunk / 16;         // one warp per K step of a chunk
+constexpr int kOrders = 4;                    // orders of an accumulator
+constexpr int kIssuers = kSlices / kOrders;   // one warp per accumulator
 constexpr int kThreads = kIssuer + 32 * kIssuers;
 
 __host__ __device__ constexpr int cores(int M) { return (M < kTile ? kTile : M) / 8 + 15; }
@@ -470,7 +477,7 @@ __device__ __forceinline__ uint64_t operand(unsigned addr, unsigned lead, unsign
 }
 
 // FP32 accumulator, fp16 A and B, both K-major, 128 rows, `n` columns.
-__device__ __forceinline__ uint32_t mma_shape(int n) {
+__device__ __forceinline__ constexpr uint32_t mma_shape(int n) {
   return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
 }
 
@@ -571,14 +578,22 @@ struct Items {
   }
 };
 
+// Zeros before a chunk's digits in shared memory: the slices j = p - i of an
+// accumulator's orders run from -(kOrders - 1) (order 0 of slice kOrders - 1, order
+// kOrders of slice 2 kOrders - 1) to kSlices - 1.
+static_assert(kSlices == 2 * kOrders, "slices reach from -(kOrders - 1) to kSlices - 1");
+__host__ __device__ constexpr int pad_bytes(int NL) { return (kOrders - 1) * NL * kChunk * 2; }
+
 template <int NL>
 __global__ void __launch_bounds__(kThreads, 1)
     k_toep_mma(double* __restrict__ u, double* __restrict__ delta,
                const unsigned char* __restrict__ band, const unsigned char* __restrict__ dig,
                const int* __restrict__ lexp, Geometry G, Items items, int stages) {
-  constexpr int kCols = kSlices * NL;               // columns of one accumulator
+  constexpr int kCols = kSlices * NL;               // columns of the accumulators of a segment
   constexpr unsigned kTmem = 2 * kCols;             // 512 or 256
   constexpr int kStage = kCols * kChunk * 2;        // bytes of a chunk's digits
+  constexpr int kPad = pad_bytes(NL);               // zeros before them: slices -3 .. -1
+  constexpr int kSlot = kPad + kStage;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // band: full / empty; chunk ring: full / empty; accumulators: full / empty
   __shared__ __align__(8) uint64_t bars[2 + 2 * kMaxStages + 4];
@@ -623,6 +638,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int c = (warp >> 2) * 4; c < 2 * kCols; c += 16) tmem_clear4(at + (unsigned)c);
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     tc_fence_before();
+    for (int x = threadIdx.x; x < stages * (kPad / 16); x += kFoldThreads) {
+      const int slot = x / (kPad / 16);
+      *reinterpret_cast<uint4*>(sRing + slot * kSlot + (x - slot * (kPad / 16)) * 16) =
+          make_uint4(0u, 0u, 0u, 0u);
+    }
+    fence_proxy_async_smem();
   }
   __syncthreads();
   tc_fence_after();
@@ -654,7 +675,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!ok) break;
           const unsigned bytes = (unsigned)((kSlices - i0) * NL * kChunk * 2);
           mbar_arrive_expect_tx(&full[slot], bytes);
-          bulk_copy_g2s(sRing + slot * kStage, src, bytes, &full[slot]);
+          bulk_copy_g2s(sRing + slot * kSlot + kPad, src, bytes, &full[slot]);
           ++chunks;
           if (++slot == stages) slot = 0, ++round;
         }
@@ -668,17 +689,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else if (warp >= kIssuer / 32) {
-    // Each issuer takes one K step of every chunk: waits and bookkeeping take a warp
-    // longer than the small MMAs of a step.  Accumulators start at zero (cleared by
-    // the warps that read them), so the order of the MMAs is free.  A whole warp
-    // walks the items (uniform control flow), one lane issues.
+    // Each issuer takes one accumulator, both K steps of every chunk (the order of an
+    // accumulator's MMAs is its thread's; waits and bookkeeping of one warp for both
+    // would leave the tensor cores idle).  Accumulators start at zero (cleared by the
+    // warps that read them).  A whole warp walks the items (uniform control flow), one
+    // lane issues.
     const bool lead = elect_one();
+    const int half = warp - kIssuer / 32;
     const unsigned tmem_u = uniform(tmem);
     int cur = -1, bands = 0, seg = 0, slot = 0, round = 0, last = -1, last_round = 0;
     const unsigned sb = (unsigned)slice_bytes(M) >> 4;
-    const unsigned kx = (unsigned)(warp - kIssuer / 32) * 16;  // operand offset of the K step
-    const uint64_t opA = operand(0, 128, 128) + ((smem_u32(sBand) >> 4) + kx);
-    const uint64_t opB = operand(0, 128, 512) + ((smem_u32(sRing) >> 4) + kx);
+    const uint64_t opA = operand(0, 128, 128) + (smem_u32(sBand) >> 4);
+    // slice `kOrders half` of the first slot: the window of slice i = 0
+    const uint64_t opB = operand(0, 128, 512) +
+                         ((smem_u32(sRing) + (unsigned)(kPad + half * kOrders * NL * kChunk * 2)) >> 4);
+    constexpr uint32_t kShape = mma_shape(kOrders * NL);
+    constexpr unsigned kWindow = NL * kChunk * 2 / 16;  // one slice on, in 16-byte units
     for (int it = 0; ok && items.get(it, g, tau); ++it) {
       const int inst = (G.group0 + g) / G.per_inst;
       if (inst != cur) {
@@ -697,7 +723,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int c = 0; ok && c < nc; ++seg) {
         const int end = segment_end(starts, c, nc);
         const int a = seg & 1;
-        const unsigned dst = tmem_u + (unsigned)(a * kCols);
+        const unsigned dst = tmem_u + (unsigned)(a * kCols + half * kOrders * NL);
         if (seg >= 2) ok = warp_wait(&acc_empty[a], (unsigned)((seg / 2 - 1) & 1));
         for (; ok && c < end; ++c) {
           ok = warp_wait(&full[slot], (unsigned)(round & 1));
@@ -706,11 +732,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (lead) {
             const int i0 = first_slice(first, c);
             const uint64_t da = opA + (unsigned)chunk_core(M, c) * 8;
-            const uint64_t db = opB + (unsigned)slot * (kStage / 16);
+            const uint64_t db = opB + (unsigned)slot * (kSlot / 16);
 #pragma unroll
-            for (int i = 0; i < kSlices; ++i)
-              if (i >= i0)
-                mma_f16(dst + i * NL, da + (uint64_t)(i * sb), db, mma_shape(NL * (kSlices - i)), 1u);
+            for (int k = 0; k < kChunk / 16; ++k)  // 16 steps: two cores of either operand
+#pragma unroll
+              for (int i = 0; i < kSlices; ++i)
+                if (i >= i0 && i < kOrders * (half + 1))
+                  mma_f16(dst, da + (uint64_t)(i * sb + k * 16), db - (uint64_t)(i * kWindow) + k * 16,
+                          kShape, 1u);
             mma_commit(&empty[slot]);
             if (c + 1 == end) mma_commit(&acc_full[a]);
           }
@@ -882,13 +911,13 @@ cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigne
   items.dealt = G.groups < 4 * sm_count();
   const long long count = items.dealt ? (long long)G.groups * items.tiles : G.groups;
   const unsigned grid = (unsigned)(count < sm_count() ? count : sm_count());
-  constexpr size_t kStage = (size_t)kSlices * NL * kChunk * 2;
+  constexpr size_t kSlot = (size_t)pad_bytes(NL) + (size_t)kSlices * NL * kChunk * 2;
   const size_t band_bytes = kSlices * slice_bytes(M);
-  int stages = (int)((226 * 1024 - band_bytes) / kStage);
+  int stages = (int)((226 * 1024 - band_bytes) / kSlot);
   if (stages > kMaxStages) stages = kMaxStages;
   // at least half the SM's shared memory and one byte: one CTA per SM, whose
   // accumulators take its tensor memory (NL = 32)
-  size_t smem = band_bytes + stages * kStage;
+  size_t smem = band_bytes + stages * kSlot;
   if (smem < 116 * 1024) smem = 116 * 1024;
   e = prepare_smem(k_toep_mma<NL>, smem);
   if (e != cudaSuccess) return e;

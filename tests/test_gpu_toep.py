@@ -170,3 +170,29 @@ def test_non_finite_values_stay_in_their_line_of_a_sliced_sweep(n, M, bad):
             s.set_rhs(f)
             s.solve(1, 1, 1, tol=1e-10, max_cycles=5)
         assert e.value.status == G.MGWR_E_NUMERIC
+
+
+# every launch sums the same whole numbers: the bits of a half-sweep, its changes and a defect
+# repeat, and lines with the same data agree with one another (each line length, groups of 16
+# and of 32 lines, columns with and without slices that vanish at far lags)
+@pytest.mark.parametrize("n,M", [(4095, 64), (1023, 128), (511, 256), (127, 512), (511, 512),
+                                 (127, 1024), (1023, 1024)])
+def test_sliced_products_repeat_their_bits(n, M):
+    assert not _sums(n // 2, M)
+    line = inputs.random_field(1, M, 6, scale=(n + 1.0) ** 2)[0]
+    f = np.tile(line, (n, 1))
+    with G.Solver(1, n, M, 1.0, 0.4) as s:
+        l = s.num_levels() - 1
+        s.field_set(G.MGWR_H64, l, G.MGWR_F, f)
+        seen = []
+        for _ in range(25):
+            s.field_set(G.MGWR_H64, l, G.MGWR_U, np.zeros_like(f))
+            s.smooth(G.MGWR_H64, l, G.MGWR_RED)
+            u = s.field_get(G.MGWR_H64, l, G.MGWR_U)
+            s.defect(G.MGWR_H64, l)
+            seen.append((u, s.field_get(G.MGWR_H64, l, G.MGWR_R)))
+    for u, r in seen:
+        np.testing.assert_array_equal(u, seen[0][0])
+        np.testing.assert_array_equal(r, seen[0][1])
+    red = seen[0][0][1::2]
+    np.testing.assert_array_equal(red, np.tile(red[0], (len(red), 1)))
