@@ -532,6 +532,12 @@ int mgwr_server_release(mgwr_server_t s, double* buf);
 int mgwr_poll(mgwr_server_t s, uint64_t ticket, int timeout_us, double* u_out, mgwr_result* res);
 int mgwr_server_stats(mgwr_server_t s, mgwr_server_info* info);
 
+/* Failure injection for tests of error handling: marks the handle as if a
+ * bounded wait of one of its kernels had given up (no kernel runs).  The next
+ * solve or component call of this handle that runs such kernels returns
+ * MGWR_E_CUDA and clears the mark; other handles are not affected. */
+int mgwr_inject_give_up(mgwr_t h);
+
 /* Number of CUDA kernel launches issued through the library so far
  * (process-wide; h may be NULL). */
 int mgwr_launch_count(mgwr_t h, long long* count);

@@ -121,8 +121,8 @@ struct mgwr_handle {
   // shared by every precision (one launch at a time on the handle's stream)
   Cx<double>* scratch = nullptr;
   size_t scratch_count = 0;
-  unsigned long long* norm_bits = nullptr;  // device, one per instance
-  unsigned long long* norm_host = nullptr;  // pinned, one per instance
+  unsigned long long* norm_bits = nullptr;  // device, one per instance, then the give-up word
+  unsigned long long* norm_host = nullptr;  // pinned, the same
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   std::vector<double> r0, relres;  // per instance
   bool r0_valid = false;
@@ -248,19 +248,25 @@ constexpr int defect_class() {
          : std::is_same<R, mgwr::dd>::value ? MGWR_K_DEFECT_DD : MGWR_K_DEFECT64;
 }
 
-// A staged sweep that gave up waiting for its copies (never expected: a copy of
-// a valid line always lands) turns into an error of the call that ran it.
-int check_staging(mgwr_t h) {
-  bool hit = false;
-  if (h->toep_band != nullptr) {
-    MGWR_CK(h, mgwr::take_toep_timeout(&hit));
-    if (hit) return fail(h, MGWR_E_CUDA, "sliced product: wait for its copies or MMAs gave up");
-  }
-  MGWR_CK(h, mgwr::take_stage_timeout(&hit));
-  if (hit) return fail(h, MGWR_E_CUDA, "staged sweep: wait for bulk copies gave up");
-  MGWR_CK(h, mgwr::take_tc_timeout(&hit));
-  if (hit) return fail(h, MGWR_E_CUDA, "tensor-core sweep: wait for its MMAs gave up");
-  return MGWR_OK;
+// The handle's give-up word (device): set by its own launches alone.
+unsigned* gave_up(const mgwr_handle* h) {
+  return reinterpret_cast<unsigned*>(h->norm_bits + h->B);
+}
+
+// A kernel of this handle that gave up a bounded wait (never expected: a copy of a
+// valid line always lands) turns into an error of the call that ran it.
+// Synchronises the handle's stream.
+int check_waits(mgwr_t h) {
+  MGWR_CK(h, cudaMemcpyAsync(h->norm_host + h->B, h->norm_bits + h->B, sizeof(unsigned long long),
+                             cudaMemcpyDeviceToHost, h->stream));
+  MGWR_CK(h, cudaStreamSynchronize(h->stream));
+  const unsigned long long bits = h->norm_host[h->B];
+  if (bits == 0) return MGWR_OK;
+  MGWR_CK(h, cudaMemsetAsync(gave_up(h), 0, sizeof(unsigned long long), h->stream));
+  return fail(h, MGWR_E_CUDA,
+              (bits & mgwr::kGaveUpToep) ? "sliced product: wait for its copies or MMAs gave up"
+              : (bits & mgwr::kGaveUpTc) ? "tensor-core sweep: wait for its MMAs gave up"
+                                         : "staged sweep: wait for bulk copies gave up");
 }
 
 int split_of(const mgwr_handle* h, int cls, int l) {
@@ -501,7 +507,7 @@ cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
       return mgwr::launch_sweep_toep(f, u, delta, h->kcol + (size_t)l * h->M,
                                      (size_t)h->nlev * h->M, h->toep_band + (size_t)l * bb,
                                      (size_t)h->nlev * bb, h->toep_scratch, ls, par, h->hinv2[l],
-                                     h->stream, zero_u);
+                                     gave_up(h), h->stream, zero_u);
     }
   }
   if constexpr (std::is_same<R, float>::value) {
@@ -510,7 +516,7 @@ cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
     if ((eff & mgwr::kTensor) && h->tc_band != nullptr) {
       const size_t bb = mgwr::tc_band_bytes(h->M);
       return mgwr::launch_sweep_tc(f, u, delta, h->tc_band + (size_t)l * bb, (size_t)h->nlev * bb,
-                                   ls, par, (float)h->hinv2[l], h->stream, zero_u);
+                                   ls, par, (float)h->hinv2[l], gave_up(h), h->stream, zero_u);
     }
     if ((eff & mgwr::kRadix) && H.spec_rp != nullptr)
       return mgwr::launch_sweep_rp(f, u, delta, H.spec_rp + (size_t)l * h->L,
@@ -519,7 +525,7 @@ cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
   }
   return mgwr::launch_sweep<R>(f, u, delta, H.spec + (size_t)l * h->L, (size_t)h->nlev * h->L,
                                H.tw, H.zero, scratch_for<R>(h), ls, par, false, R(h->hinv2[l]),
-                               E & ~(mgwr::kTensor | mgwr::kRadix), h->stream, zero_u);
+                               E & ~(mgwr::kTensor | mgwr::kRadix), gave_up(h), h->stream, zero_u);
 }
 
 template <class R>
@@ -538,7 +544,7 @@ int coarsest(mgwr_t h, Hier<R>& H) {
   if (std::is_same<R, float>::value && E == 0) E = default_sweep32(shape(h, 0));
   MGWR_CK(h, mgwr::launch_sweep<R>(H.f[0], H.u[0], (R*)nullptr, H.spec, (size_t)h->nlev * h->L,
                                     H.tw, H.zero, scratch_for<R>(h), shape(h, 0), 0, true, R(0),
-                                    E & ~(mgwr::kTensor | mgwr::kRadix), h->stream));
+                                    E & ~(mgwr::kTensor | mgwr::kRadix), gave_up(h), h->stream));
   prof_end(h, pm);
   H.rs[0] = R_STALE;
   H.uz[0] = 0;
@@ -597,7 +603,7 @@ int defect64(mgwr_t h, int l, unsigned long long* norm_bits) {
   Hier<double>& H = h->h64;
   if (h->toep_band != nullptr && mgwr::toep_defect(shape(h, l)))
     MGWR_CK(h, mgwr::launch_defect_toep(H.u[l], H.f[l], H.r[l], h->toep_tband, h->toep_scratch,
-                                        shape(h, l), h->hinv2[l], norm_bits, h->stream));
+                                        shape(h, l), h->hinv2[l], norm_bits, gave_up(h), h->stream));
   else
     MGWR_CK(h, (mgwr::launch_defect<double, double>(
                    H.u[l], H.f[l], H.r[l], H.tspec, (size_t)h->L, H.tw, H.zero,
@@ -1175,7 +1181,7 @@ int tune_hierarchy(mgwr_t h, Hier<R>& H, int cls_sweep, int cls_defect) {
         if (l == 0)
           return mgwr::launch_sweep<R>(H.f[0], out, (R*)nullptr, spec, sstride, H.tw, H.zero,
                                        scratch_for<R>(h), ls, 0, true, R(0),
-                                       E & ~(mgwr::kTensor | mgwr::kRadix), h->stream);
+                                       E & ~(mgwr::kTensor | mgwr::kRadix), gave_up(h), h->stream);
         const cudaError_t e =
             level_sweep(h, H, l, H.f[l], out, (R*)nullptr, ls, parity(h, MGWR_RED), E);
         if (e != cudaSuccess) return e;
@@ -1380,13 +1386,18 @@ int create_impl(int d, int n, int M, const double* T, const double* alpha, int b
   }
   h->stream = h->own_stream;
   if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess ||
-      cudaMallocHost(&h->norm_host, sizeof(unsigned long long) * batch) != cudaSuccess) {
+      cudaMallocHost(&h->norm_host, sizeof(unsigned long long) * (batch + (size_t)1)) != cudaSuccess) {
     cudaGetLastError();
     return bail(MGWR_E_CUDA);
   }
   const size_t B = batch;
   int s;
-  if ((s = dev_alloc(h, &h->norm_bits, sizeof(unsigned long long) * B)) != MGWR_OK) return bail(s);
+  if ((s = dev_alloc(h, &h->norm_bits, sizeof(unsigned long long) * (B + 1))) != MGWR_OK)
+    return bail(s);
+  if (cudaMemsetAsync(gave_up(h), 0, sizeof(unsigned long long), h->stream) != cudaSuccess) {
+    cudaGetLastError();
+    return bail(MGWR_E_CUDA);
+  }
   if ((s = dev_alloc(h, &h->r, sizeof(double) * B * M)) != MGWR_OK) return bail(s);
   if ((s = dev_alloc(h, &h->dk, sizeof(double) * B * (M + 1))) != MGWR_OK) return bail(s);
   if ((s = dev_alloc(h, &h->kcol, sizeof(double) * B * h->nlev * M)) != MGWR_OK) return bail(s);
@@ -1647,7 +1658,7 @@ int mgwr_autotune(mgwr_t h) {
   }
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
   drop_graph(h);
-  return check_staging(h);
+  return check_waits(h);
 }
 
 int mgwr_set_outer_switch(mgwr_t h, double rel) {
@@ -2040,8 +2051,7 @@ int solve_end(mgwr_t h, SolveState& S, mgwr_stats* st) {
   int status = S.status;
   if (!std::isfinite(S.rel)) status = MGWR_E_NUMERIC;
   MGWR_CK(h, cudaEventRecord(h->ev1, h->stream));
-  MGWR_CK(h, cudaEventSynchronize(h->ev1));
-  MGWR_TRY(check_staging(h));
+  MGWR_TRY(check_waits(h));
   prof_collect(h);
   float ms = 0.f;
   MGWR_CK(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
@@ -2542,7 +2552,7 @@ int mgwr_smooth(mgwr_t h, int hierarchy, int level, int colour) {
   if (colour != MGWR_RED && colour != MGWR_BLACK) return fail(h, MGWR_E_INVAL, "bad colour");
   MGWR_TRY(with_hier(h, hierarchy, [&](auto& H) { return smooth_colour(h, H, level, colour); }));
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
-  return check_staging(h);
+  return check_waits(h);
 }
 
 // largest per-instance norm of the last reduction
@@ -2579,7 +2589,7 @@ int mgwr_smooth_restrict(mgwr_t h, int hierarchy, int level) {
     return restrict_delta_into(h, H, level, true);
   }));
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
-  return check_staging(h);
+  return check_waits(h);
 }
 
 int mgwr_defect(mgwr_t h, int hierarchy, int level, double* norm_inf) {
@@ -2630,7 +2640,7 @@ int mgwr_cycle(mgwr_t h, int hierarchy, int cyc, int nu1, int nu2) {
   MGWR_TRY(with_hier(h, hierarchy,
                      [&](auto& H) { return cycle(h, H, h->nlev - 1, cyc, nu1, nu2); }));
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
-  return check_staging(h);
+  return check_waits(h);
 }
 
 int mgwr_toeplitz_column(mgwr_t h, double* r_host) {
@@ -2692,7 +2702,7 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
   }
   const size_t nlev = pts.size();
   size_t total = 2u << 20;
-  total += r512(8 * B) + r512(8 * B * M) + r512(8 * B * (M + 1)) + r512(8 * B * nlev * M);
+  total += r512(8 * (B + 1)) + r512(8 * B * M) + r512(8 * B * (M + 1)) + r512(8 * B * nlev * M);
   total += 2 * r512(8 * B) + r512(8 * nlev);
   total += r512(16 * B * nlev * 3 * M);  // divide-and-conquer work (freed after setup)
   total += r512(16 * B * nlev * L) + r512(16 * B * L) + r512(16 * Lt);
@@ -2723,6 +2733,13 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
       total += r512(8 * B * pts[0] * M) + r512(16 * B * L) + r512(16 * Lt);
   }
   *bytes = total;
+  return MGWR_OK;
+}
+
+int mgwr_inject_give_up(mgwr_t h) {
+  if (h == nullptr) return MGWR_E_INVAL;
+  MGWR_CK(h, cudaMemsetAsync(gave_up(h), mgwr::kGaveUpToep, 1, h->stream));
+  MGWR_CK(h, cudaStreamSynchronize(h->stream));
   return MGWR_OK;
 }
 

@@ -84,6 +84,11 @@ inline size_t long_scratch_count(const LevelShape& ls) {
   return (size_t)ls.batch * ((pts + 1) / 2) * 2 * (size_t)ls.M;
 }
 
+// Bits of a handle's give-up word: a bounded wait that ran out in a kernel of the
+// sliced products, the staged sweep or the tensor-core sweep; a pair of the staged
+// sweep with more lines than slots.
+constexpr unsigned kGaveUpToep = 1, kGaveUpStage = 2, kGaveUpTc = 4, kGaveUpSlots = 8;
+
 // ---- launchers (kernels in mgwr_kernels.cu); all return the launch status ----
 // Every launcher covers all `batch` instances (blockIdx.y = instance).
 
@@ -98,38 +103,36 @@ inline size_t long_scratch_count(const LevelShape& ls) {
 // otherwise, may be null).
 // E: butterflies per thread of the FFT engine (engine_split; the launch shape
 // only, results are identical for every E).
+// gave_up (here and in the other forms with bounded waits): the handle's device
+// word, in which a wait that gives up sets its kernel's bit.
 // zero_u (here and in the other forms below): u is zero; its memory is not read
 // (delta null).
 template <class R>
 cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t spec_stride,
                          const Cx<R>* tw, const R* zero, Cx<R>* scratch, const LevelShape& ls,
-                         int par, bool all_points, R hinv2, int E, cudaStream_t s,
-                         bool zero_u = false);
+                         int par, bool all_points, R hinv2, int E, unsigned* gave_up,
+                         cudaStream_t s, bool zero_u = false);
 
 // launch_sweep<float> for 64 <= M <= kShortMaxM without all_points, E carrying
 // kStaged: a persistent grid (as many CTAs as fit on the GPU) walks the line
 // pairs; while a group transforms one pair, the f and neighbour lines of its
 // next pair are copied into shared memory by cp.async.bulk, completing on an
 // mbarrier.  Same arithmetic in the same order as the direct-load kernel, so
-// the results are bitwise identical.  A wait that gives up (half a second) sets
-// a device flag read by take_stage_timeout.
+// the results are bitwise identical.  Waits give up after half a second.
 cudaError_t launch_sweep_staged(const float* f, float* u, float* delta, const Cx<float>* spec,
                                 size_t spec_stride, const Cx<float>* tw, const float* zero,
                                 const LevelShape& ls, int par, float hinv2, int E,
-                                cudaStream_t s);
-// Reads and clears the flag of the staged sweep's bounded waits (synchronous).
-cudaError_t take_stage_timeout(bool* hit);
+                                unsigned* gave_up, cudaStream_t s);
 
 // One colour half-sweep of FP32 lines of M = 64, 128 or 256 steps on the
 // tensor cores (tcgen05.mma, bf16 x 3 pieces, FP32 accumulation): as
 // launch_sweep without all_points, with the inverse column of instance b given
 // as its Toeplitz band (band + b * bstride, tc_band_bytes(M) bytes, written by
 // launch_band_bf16x3).  Results agree with the FFT engine's to FP32 rounding
-// (not bitwise).  A wait that gives up (half a second) sets a flag read by
-// take_tc_timeout.
+// (not bitwise).  Waits give up after half a second.
 cudaError_t launch_sweep_tc(const float* f, float* u, float* delta, const unsigned char* band,
                             size_t bstride, const LevelShape& ls, int par, float hinv2,
-                            cudaStream_t s, bool zero_u = false);
+                            unsigned* gave_up, cudaStream_t s, bool zero_u = false);
 // Bytes of one Toeplitz band: three bf16 pieces of M rows x 32 columns.
 size_t tc_band_bytes(int M);
 // band + line * tc_band_bytes(M): the band of the inverse column kcol[line]
@@ -137,7 +140,6 @@ size_t tc_band_bytes(int M);
 // (x = x0 + x1 + x2), in the tensor-core kernel's shared-memory layout.
 cudaError_t launch_band_bf16x3(const double* kcol, unsigned char* band, int M, size_t lines,
                                cudaStream_t s);
-cudaError_t take_tc_timeout(bool* hit);
 
 // One colour half-sweep of FP64 lines of M = 64 .. 1024 steps as sliced integer
 // products on the tensor cores, or where the lines are few as FP64 sums
@@ -145,14 +147,13 @@ cudaError_t take_tc_timeout(bool* hit);
 // coarsest grid is colour 0 of n = 1), the inverse column of instance b given
 // in FP64 (cols + b * cstride) and as its sliced band (band + b * bstride,
 // toep_band_bytes(M) bytes, written by launch_toep_band).  scratch holds
-// toep_scratch_bytes.  A wait that gives up (half a second) sets a flag read by
-// take_toep_timeout.  A line with an infinity or NaN in its gathered values
-// becomes NaN.
+// toep_scratch_bytes.  Waits give up after half a second.  A line with an
+// infinity or NaN in its gathered values becomes NaN.
 inline bool toep_length(int M) { return M >= 64 && M <= 1024; }
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
                               size_t cstride, const unsigned char* band, size_t bstride,
                               unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
-                              cudaStream_t s, bool zero_u = false);
+                              unsigned* gave_up, cudaStream_t s, bool zero_u = false);
 // The FP64 defect r = f - (T_M (x) I + A_h) u with the time term as sliced products
 // (bands of the instances' Toeplitz columns, toep_band_bytes(M) apart), for the
 // shapes toep_defect names (the transform's single launch is cheaper below);
@@ -161,7 +162,7 @@ bool toep_defect(const LevelShape& ls);
 cudaError_t launch_defect_toep(const double* u, const double* f, double* r,
                                const unsigned char* band, unsigned char* scratch,
                                const LevelShape& ls, double hinv2, unsigned long long* norm_bits,
-                               cudaStream_t s);
+                               unsigned* gave_up, cudaStream_t s);
 size_t toep_band_bytes(int M);
 // Bytes of scratch the launches on a level of this shape need (bounded: larger
 // fields go through it in slabs).
@@ -169,7 +170,6 @@ size_t toep_scratch_bytes(const LevelShape& ls);
 // blob + line * toep_band_bytes(M): the sliced band of column cols[line].
 cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, size_t lines,
                              cudaStream_t s);
-cudaError_t take_toep_timeout(bool* hit);
 
 // One colour half-sweep of FP32 lines of 64 .. 4096 steps on the register-pass
 // FFT engine (mgwr_fft_rp.cuh): as launch_sweep without all_points, with the

@@ -107,8 +107,8 @@ cudaError_t sweep_launch(dim3 grid, size_t smem, cudaStream_t s, const R* f, R* 
 template <class R>
 cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t spec_stride,
                          const Cx<R>* tw, const R* zero, Cx<R>* scratch, const LevelShape& ls,
-                         int par, bool all_points, R hinv2, int E, cudaStream_t s,
-                         bool zero_u) {
+                         int par, bool all_points, R hinv2, int E, unsigned* gave_up,
+                         cudaStream_t s, bool zero_u) {
   if (ls.M > kShortMaxM)
     return launch_sweep_long(f, u, delta, spec, spec_stride, tw, scratch, ls, par, all_points,
                              hinv2, E, s, zero_u);
@@ -117,7 +117,7 @@ cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t s
   E = effective_split(M, (int)sizeof(R) == 4 ? 4 : 8, E);
   if constexpr (sizeof(R) == 4) {
     if ((E & kStaged) && !all_points && !zero_u)
-      return launch_sweep_staged(f, u, delta, spec, spec_stride, tw, zero, ls, par, hinv2, E, s);
+      return launch_sweep_staged(f, u, delta, spec, spec_stride, tw, zero, ls, par, hinv2, E, gave_up, s);
   }
   E &= ~(kStaged | kTensor | kRadix);
   const int npts = all_points ? (d == 1 ? n : n * n) : colour_count(d, n, par);
@@ -172,13 +172,15 @@ cudaError_t launch_sweep(const R* f, R* u, R* delta, const Cx<R>* spec, size_t s
 
 template cudaError_t launch_sweep<double>(const double*, double*, double*, const Cx<double>*,
                                           size_t, const Cx<double>*, const double*, Cx<double>*,
-                                          const LevelShape&, int, bool, double, int, cudaStream_t, bool);
+                                          const LevelShape&, int, bool, double, int, unsigned*,
+                                          cudaStream_t, bool);
 template cudaError_t launch_sweep<float>(const float*, float*, float*, const Cx<float>*, size_t,
                                          const Cx<float>*, const float*, Cx<float>*,
-                                         const LevelShape&, int, bool, float, int, cudaStream_t, bool);
+                                         const LevelShape&, int, bool, float, int, unsigned*,
+                                         cudaStream_t, bool);
 
 template cudaError_t launch_sweep<dd>(const dd*, dd*, dd*, const Cx<dd>*, size_t, const Cx<dd>*,
                                       const dd*, Cx<dd>*, const LevelShape&, int, bool, dd, int,
-                                      cudaStream_t, bool);
+                                      unsigned*, cudaStream_t, bool);
 
 }  // namespace mgwr

@@ -13,10 +13,6 @@
 
 namespace mgwr {
 
-// Bit 0: a group gave up waiting for its copies; bit 1: a pair needed more
-// staging slots than it has (read by take_stage_timeout).
-__device__ unsigned g_stage_timeout;
-
 namespace {
 
 // Staged lines per group: fA, fB and at most seven distinct neighbour lines.
@@ -39,7 +35,8 @@ struct PairLines {
 };
 
 __device__ __forceinline__ void pair_lines(PairLines& P, int item, int g, int groups, int nblk,
-                                           int npairs, int npts, int d, int n, int par, int M) {
+                                           int npairs, int npts, int d, int n, int par, int M,
+                                           unsigned* gave_up) {
   P.inst = item / nblk;
   const int pair = (item - P.inst * nblk) * groups + g;
   P.valid = pair < npairs;
@@ -63,7 +60,7 @@ __device__ __forceinline__ void pair_lines(PairLines& P, int item, int g, int gr
   P.copies = shared_lr ? (present & ~64u) : present;
   if (__popc(P.copies) > kSlots) {  // cannot happen (see kSlots); flagged, never overruns
     P.present = P.copies = 0;
-    atomicOr(&g_stage_timeout, 2u);
+    atomicOr(gave_up, kGaveUpSlots);
   }
   int next = 0;
 #pragma unroll
@@ -100,9 +97,9 @@ __device__ __forceinline__ void issue_copies(const PairLines& P, const float* f,
 __device__ __noinline__ void stage_item(int item, int g, int groups, int nblk, int npairs, int npts,
                                         int d, int n, int par, int M, const float* f,
                                         const float* u, size_t fstride, float* stage,
-                                        uint64_t* bar) {
+                                        uint64_t* bar, unsigned* gave_up) {
   PairLines Q;
-  pair_lines(Q, item, g, groups, nblk, npairs, npts, d, n, par, M);
+  pair_lines(Q, item, g, groups, nblk, npairs, npts, d, n, par, M, gave_up);
   const size_t off = (size_t)Q.inst * fstride;
   fence_proxy_async_smem();
   issue_copies(Q, f + off, u + off, stage, bar, n, M);
@@ -115,7 +112,7 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<float>(BLOCK, E))
     k_sweep_staged(const float* __restrict__ f, float* __restrict__ u, float* __restrict__ delta,
                    const Cx<float>* __restrict__ spec, const Cx<float>* __restrict__ tw, int d,
                    int n, int par, float hinv2, int npts, int npairs, int nblk, int nitems,
-                   size_t fstride, size_t sstride) {
+                   size_t fstride, size_t sstride, unsigned* __restrict__ gave_up) {
   constexpr int TL = SH::L8 / E;  // threads per line pair
   constexpr int groups = BLOCK / TL;
   constexpr int M = SH::L / 2;
@@ -136,7 +133,8 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<float>(BLOCK, E))
 
   int item = blockIdx.x;
   if (t == 0 && item < nitems)
-    stage_item(item, g, groups, nblk, npairs, npts, d, n, par, M, f, u, fstride, stage, bar);
+    stage_item(item, g, groups, nblk, npairs, npts, d, n, par, M, f, u, fstride, stage, bar,
+               gave_up);
   for (unsigned j = 0; item < nitems; ++j, item += gridDim.x) {
     // one thread per group waits; the CTA barrier also ends every read of buf by
     // the previous item, and a group that gave up ends the whole CTA (every group
@@ -145,14 +143,14 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<float>(BLOCK, E))
     if (t == 0) failed = mbar_wait_bounded(bar, j & 1u) ? 0 : 1;
     if (__syncthreads_or(failed)) {
       if (failed) {
-        atomicOr(&g_stage_timeout, 1u);
+        atomicOr(gave_up, kGaveUpStage);
         (void)mbar_wait_bounded(bar, j & 1u);  // the copies in flight land before the CTA ends
       }
       return;
     }
     (void)mbar_try_wait(bar, j & 1u);  // completed phase: acquire the staged lines here too
     PairLines P;
-    pair_lines(P, item, g, groups, nblk, npairs, npts, d, n, par, M);
+    pair_lines(P, item, g, groups, nblk, npairs, npts, d, n, par, M, gave_up);
     // line k at time m: the staged value, or the zero Dirichlet value outside the grid
     auto rd = [&](int k, int m) -> float {
       return ((P.present >> k) & 1u) ? stage[P.off[k] + m] : 0.f;
@@ -168,7 +166,8 @@ __global__ void __launch_bounds__(BLOCK, min_blocks<float>(BLOCK, E))
     const int next = item + (int)gridDim.x;
     auto refill = [&]() {
       if (t == 0 && next < nitems)
-        stage_item(next, g, groups, nblk, npairs, npts, d, n, par, M, f, u, fstride, stage, bar);
+        stage_item(next, g, groups, nblk, npairs, npts, d, n, par, M, f, u, fstride, stage, bar,
+               gave_up);
     };
     Cx<float> v[E][8];
     fft_forward<E>(buf, t, sh, tw, load, v, sync, refill);
@@ -204,7 +203,7 @@ namespace {
 template <int BLOCK, class SH, int E>
 cudaError_t staged_launch(const float* f, float* u, float* delta, const Cx<float>* spec,
                           size_t sstride, const Cx<float>* tw, const LevelShape& ls, int par, float hinv2, int npts, int npairs,
-                          cudaStream_t s) {
+                          unsigned* gave_up, cudaStream_t s) {
   constexpr int TL = SH::L8 / E;
   constexpr int groups = BLOCK / TL;
   constexpr int M = SH::L / 2;
@@ -227,7 +226,7 @@ cudaError_t staged_launch(const float* f, float* u, float* delta, const Cx<float
   const long long cap = (long long)per_sm * sms;
   const unsigned grid = (unsigned)(nitems < cap ? nitems : cap);
   kern<<<grid, BLOCK, smem, s>>>(f, u, delta, spec, tw, ls.d, ls.n, par, hinv2, npts, npairs,
-                                 nblk, (int)nitems, ls.field_stride(), sstride);
+                                 nblk, (int)nitems, ls.field_stride(), sstride, gave_up);
   return cudaSuccess;
 }
 
@@ -236,7 +235,7 @@ cudaError_t staged_launch(const float* f, float* u, float* delta, const Cx<float
 cudaError_t launch_sweep_staged(const float* f, float* u, float* delta, const Cx<float>* spec,
                                 size_t spec_stride, const Cx<float>* tw, const float* zero,
                                 const LevelShape& ls, int par, float hinv2, int E,
-                                cudaStream_t s) {
+                                unsigned* gave_up, cudaStream_t s) {
   (void)zero;  // lines outside the grid are not read: the kernel adds zeros
   const int M = ls.M;
   if (M < 64 || M > kShortMaxM) return cudaErrorInvalidValue;
@@ -246,7 +245,7 @@ cudaError_t launch_sweep_staged(const float* f, float* u, float* delta, const Cx
   E = engine_split(2 * M, E);
   const int logL = ilog2(2 * M);
   cudaError_t e = cudaErrorInvalidValue;
-#define MGWR_STAGED_ARGS f, u, delta, spec, spec_stride, tw, ls, par, hinv2, npts, npairs, s
+#define MGWR_STAGED_ARGS f, u, delta, spec, spec_stride, tw, ls, par, hinv2, npts, npairs, gave_up, s
   switch (logL * 8 + E) {
 #define MGWR_CASE_E(LG, EE)                                                                    \
   case LG * 8 + EE:                                                                            \
@@ -263,18 +262,6 @@ cudaError_t launch_sweep_staged(const float* f, float* u, float* delta, const Cx
 #undef MGWR_STAGED_ARGS
   if (e != cudaSuccess) return e;
   return counted(cudaGetLastError());
-}
-
-cudaError_t take_stage_timeout(bool* hit) {
-  unsigned v = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(&v, g_stage_timeout, sizeof(v));
-  if (e != cudaSuccess) return e;
-  *hit = v != 0;
-  if (v != 0) {
-    const unsigned z = 0;
-    e = cudaMemcpyToSymbol(g_stage_timeout, &z, sizeof(z));
-  }
-  return e;
 }
 
 }  // namespace mgwr

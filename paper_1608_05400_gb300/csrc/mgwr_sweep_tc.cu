@@ -34,9 +34,6 @@
 
 namespace mgwr {
 
-// Set when a CTA gave up waiting for its MMAs (read by take_tc_timeout).
-__device__ unsigned g_tc_timeout;
-
 namespace {
 
 constexpr int kTileRows = 128;  // lines per CTA: the MMA's M
@@ -116,7 +113,8 @@ template <int M>
 __global__ void __launch_bounds__(kThreads, 2)
     k_sweep_tc(const float* __restrict__ f, float* __restrict__ u, float* __restrict__ delta,
                const unsigned char* __restrict__ band, int d, int n, int par, bool zero_u, float hinv2,
-               int npts, int tiles_per_inst, size_t fstride, size_t bstride) {
+               int npts, int tiles_per_inst, size_t fstride, size_t bstride,
+               unsigned* __restrict__ gave_up) {
   constexpr int kA = kTileRows * kChunk * 2;  // bytes per piece of a b-values chunk
   constexpr int kB = M * kChunk * 2;          // bytes per piece of the Kt band
   constexpr int kNumChunks = M / kChunk;
@@ -216,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       if (ok) {
         mma_commit(done);
       } else {
-        atomicOr(&g_tc_timeout, 1u);
+        atomicOr(gave_up, kGaveUpTc);
         // the band's bulk copy may still be writing shared memory: give it one more
         // bounded wait before the CTA can end
         if (!band_ok) (void)mbar_wait_bounded(band_bar, 0u);
@@ -291,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     // the accumulator is complete once every MMA has
     if (ok && !mbar_wait_bounded(done, 0u)) ok = false;
-    if (!ok && gt == 0) atomicOr(&g_tc_timeout, 1u);
+    if (!ok && gt == 0) atomicOr(gave_up, kGaveUpTc);
   }
   // every thread agrees on the outcome before the accumulator is read
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
@@ -343,8 +341,8 @@ namespace {
 
 template <int M>
 cudaError_t tc_launch(const float* f, float* u, float* delta, const unsigned char* band,
-                      size_t bstride, const LevelShape& ls, int par, float hinv2, cudaStream_t s,
-                      bool zero_u) {
+                      size_t bstride, const LevelShape& ls, int par, float hinv2,
+                      unsigned* gave_up, cudaStream_t s, bool zero_u) {
   const int npts = colour_count(ls.d, ls.n, par);
   if (npts == 0 || ls.batch == 0) return cudaSuccess;
   const int tiles = (npts + kTileRows - 1) / kTileRows;
@@ -361,7 +359,7 @@ cudaError_t tc_launch(const float* f, float* u, float* delta, const unsigned cha
   cudaError_t e = prepare_smem(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)grid, kThreads, smem, s>>>(f, u, delta, band, ls.d, ls.n, par, zero_u, hinv2, npts,
-                                              tiles, ls.field_stride(), bstride);
+                                              tiles, ls.field_stride(), bstride, gave_up);
   return cudaSuccess;
 }
 
@@ -393,12 +391,12 @@ __global__ void k_band_bf16x3(const double* __restrict__ kcol, unsigned char* __
 
 cudaError_t launch_sweep_tc(const float* f, float* u, float* delta, const unsigned char* band,
                             size_t bstride, const LevelShape& ls, int par, float hinv2,
-                            cudaStream_t s, bool zero_u) {
+                            unsigned* gave_up, cudaStream_t s, bool zero_u) {
   cudaError_t e = cudaErrorInvalidValue;
   switch (ls.M) {
-    case 64: e = tc_launch<64>(f, u, delta, band, bstride, ls, par, hinv2, s, zero_u); break;
-    case 128: e = tc_launch<128>(f, u, delta, band, bstride, ls, par, hinv2, s, zero_u); break;
-    case 256: e = tc_launch<256>(f, u, delta, band, bstride, ls, par, hinv2, s, zero_u); break;
+    case 64: e = tc_launch<64>(f, u, delta, band, bstride, ls, par, hinv2, gave_up, s, zero_u); break;
+    case 128: e = tc_launch<128>(f, u, delta, band, bstride, ls, par, hinv2, gave_up, s, zero_u); break;
+    case 256: e = tc_launch<256>(f, u, delta, band, bstride, ls, par, hinv2, gave_up, s, zero_u); break;
     default: break;
   }
   if (e != cudaSuccess) return e;
@@ -411,18 +409,6 @@ cudaError_t launch_band_bf16x3(const double* kcol, unsigned char* band, int M, s
                                cudaStream_t s) {
   k_band_bf16x3<<<elementwise_grid(lines * (size_t)M * kChunk), 256, 0, s>>>(kcol, band, M, lines);
   return counted(cudaGetLastError());
-}
-
-cudaError_t take_tc_timeout(bool* hit) {
-  unsigned v = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(&v, g_tc_timeout, sizeof(v));
-  if (e != cudaSuccess) return e;
-  *hit = v != 0;
-  if (v != 0) {
-    const unsigned z = 0;
-    e = cudaMemcpyToSymbol(g_tc_timeout, &z, sizeof(z));
-  }
-  return e;
 }
 
 }  // namespace mgwr

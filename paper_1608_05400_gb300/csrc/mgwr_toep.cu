@@ -68,9 +68,6 @@
 
 namespace mgwr {
 
-// Set when a CTA gave up waiting (read by take_toep_timeout).
-__device__ unsigned g_toep_timeout;
-
 namespace {
 
 constexpr int kSlices = 8;
@@ -588,7 +585,8 @@ template <int NL>
 __global__ void __launch_bounds__(kThreads, 1)
     k_toep_mma(double* __restrict__ u, double* __restrict__ delta,
                const unsigned char* __restrict__ band, const unsigned char* __restrict__ dig,
-               const int* __restrict__ lexp, Geometry G, Items items, int stages) {
+               const int* __restrict__ lexp, Geometry G, Items items, int stages,
+               unsigned* __restrict__ gave_up) {
   constexpr int kCols = kSlices * NL;               // columns of the accumulators of a segment
   constexpr unsigned kTmem = 2 * kCols;             // 512 or 256
   constexpr int kStage = kCols * kChunk * 2;        // bytes of a chunk's digits
@@ -838,7 +836,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   }
-  if (!ok) atomicOr(&g_toep_timeout, 1u);
+  if (!ok) atomicOr(gave_up, kGaveUpToep);
   tc_fence_before();
   __syncthreads();
   if (warp == kIssuer / 32)
@@ -898,7 +896,8 @@ cudaError_t gather_launch(const double* f, const double* u, const unsigned char*
 
 template <int NL>
 cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigned char* band,
-                        unsigned char* scratch, const Geometry& G, double hinv2, cudaStream_t s) {
+                        unsigned char* scratch, const Geometry& G, double hinv2, unsigned* gave_up,
+                        cudaStream_t s) {
   const int M = G.M;
   unsigned char* dig = scratch;
   int* lexp = reinterpret_cast<int*>(scratch + (size_t)G.groups * NL * M * kLineValue);
@@ -921,7 +920,8 @@ cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigne
   if (smem < 116 * 1024) smem = 116 * 1024;
   e = prepare_smem(k_toep_mma<NL>, smem);
   if (e != cudaSuccess) return e;
-  k_toep_mma<NL><<<grid, kThreads, smem, s>>>(u, delta, band, dig, lexp, G, items, stages);
+  k_toep_mma<NL><<<grid, kThreads, smem, s>>>(u, delta, band, dig, lexp, G, items, stages,
+                                             gave_up);
   return counted(cudaGetLastError());
 }
 
@@ -955,7 +955,8 @@ int direct_tile(long long lines, int M) {
 
 // Every line of a launch, in slabs of groups.
 cudaError_t product(const double* f, double* u, double* delta, const unsigned char* band,
-                    unsigned char* scratch, Geometry G, int batch, double hinv2, cudaStream_t s) {
+                    unsigned char* scratch, Geometry G, int batch, double hinv2, unsigned* gave_up,
+                    cudaStream_t s) {
   const int NL = lines_per_group(G.M, G.npts, batch);
   G.per_inst = (G.npts + NL - 1) / NL;
   const int total = G.per_inst * batch;
@@ -963,8 +964,9 @@ cudaError_t product(const double* f, double* u, double* delta, const unsigned ch
   for (int g0 = 0; g0 < total; g0 += step) {
     G.group0 = g0;
     G.groups = total - g0 < step ? total - g0 : step;
-    const cudaError_t e = NL == 32 ? slab_launch<32>(f, u, delta, band, scratch, G, hinv2, s)
-                                   : slab_launch<16>(f, u, delta, band, scratch, G, hinv2, s);
+    const cudaError_t e =
+        NL == 32 ? slab_launch<32>(f, u, delta, band, scratch, G, hinv2, gave_up, s)
+                 : slab_launch<16>(f, u, delta, band, scratch, G, hinv2, gave_up, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1033,7 +1035,7 @@ size_t toep_scratch_bytes(const LevelShape& ls) {
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
                               size_t cstride, const unsigned char* band, size_t bstride,
                               unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
-                              cudaStream_t s, bool zero_u) {
+                              unsigned* gave_up, cudaStream_t s, bool zero_u) {
   if (!toep_length(ls.M)) return cudaErrorInvalidValue;
   const int npts = colour_count(ls.d, ls.n, par);
   if (npts == 0 || ls.batch == 0) return cudaSuccess;
@@ -1063,7 +1065,7 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
 #undef MGWR_DIRECT
     return counted(cudaGetLastError());
   }
-  return product(f, u, delta, band, scratch, G, ls.batch, hinv2, s);
+  return product(f, u, delta, band, scratch, G, ls.batch, hinv2, gave_up, s);
 }
 
 // Few lines keep the transform's defect (one launch).
@@ -1075,7 +1077,7 @@ bool toep_defect(const LevelShape& ls) {
 cudaError_t launch_defect_toep(const double* u, const double* f, double* r,
                                const unsigned char* band, unsigned char* scratch,
                                const LevelShape& ls, double hinv2, unsigned long long* norm_bits,
-                               cudaStream_t s) {
+                               unsigned* gave_up, cudaStream_t s) {
   if (!toep_length(ls.M)) return cudaErrorInvalidValue;
   if (ls.batch == 0) return cudaSuccess;
   Geometry G;
@@ -1087,25 +1089,13 @@ cudaError_t launch_defect_toep(const double* u, const double* f, double* r,
   G.fstride = ls.field_stride();
   G.bstride = blob_bytes(ls.M);
   G.zero_u = false;
-  const cudaError_t e = product(u, r, nullptr, band, scratch, G, ls.batch, 0.0, s);
+  const cudaError_t e = product(u, r, nullptr, band, scratch, G, ls.batch, 0.0, gave_up, s);
   if (e != cudaSuccess) return e;
   const int per = ls.M / 2, tpl = per < 64 ? per : 64;
   const unsigned blocks = (unsigned)((G.npts + 256 / tpl - 1) / (256 / tpl));
   k_defect_finish<<<dim3(blocks, (unsigned)ls.batch), 256, 0, s>>>(
       u, f, r, ls.d, ls.n, ls.M, ilog2(tpl), G.npts, hinv2, norm_bits, G.fstride);
   return counted(cudaGetLastError());
-}
-
-cudaError_t take_toep_timeout(bool* hit) {
-  unsigned v = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(&v, g_toep_timeout, sizeof(v));
-  if (e != cudaSuccess) return e;
-  *hit = v != 0;
-  if (v != 0) {
-    const unsigned z = 0;
-    e = cudaMemcpyToSymbol(g_toep_timeout, &z, sizeof(z));
-  }
-  return e;
 }
 
 }  // namespace mgwr

@@ -124,6 +124,7 @@ _SIGS = {
     "mgwr_cycle": (C.c_int, [_h, C.c_int, C.c_int, C.c_int, C.c_int]),
     "mgwr_toeplitz_column": (C.c_int, [_h, _dp]),
     "mgwr_inverse_column": (C.c_int, [_h, C.c_int, _dp]),
+    "mgwr_inject_give_up": (C.c_int, [_h]),
     "mgwr_launch_count": (C.c_int, [_h, C.POINTER(C.c_longlong)]),
     "mgwr_peak_probe": (C.c_int, [_dp, _dp]),
     "mgwr_inverse_column_noalloc": (C.c_int, [C.c_void_p, C.c_int, C.c_double, C.c_void_p, C.c_void_p]),
@@ -297,6 +298,10 @@ class Solver:
 
     def set_outer_switch(self, rel: float):
         self._check(self.lib.mgwr_set_outer_switch(self.h, float(rel)), "mgwr_set_outer_switch")
+
+    def inject_give_up(self):
+        """Mark the handle as if a bounded wait of one of its kernels had given up (for tests)."""
+        self._check(self.lib.mgwr_inject_give_up(self.h), "mgwr_inject_give_up")
 
     def set_engine_split(self, kernel_class: int, split: int, level: int = -1):
         """E for one level, or every level (level -1)."""
