@@ -2362,6 +2362,7 @@ int mgwr_residual(mgwr_t h, double* relres, double* r_host) {
   if (h == nullptr) return MGWR_E_INVAL;
   std::vector<double> norms;
   MGWR_TRY(finest_defect_norms(h, norms, false));
+  MGWR_TRY(check_waits(h));
   if (!h->r0_valid) {
     h->r0 = norms;
     h->r0_valid = true;
@@ -2575,6 +2576,7 @@ int mgwr_smooth_defect(mgwr_t h, int hierarchy, int level, double* norm_inf) {
   }));
   std::vector<double> norms;
   MGWR_TRY(read_norms(h, norms));
+  MGWR_TRY(check_waits(h));
   if (norm_inf != nullptr) *norm_inf = max_norm(h, norms);
   return MGWR_OK;
 }
@@ -2599,6 +2601,7 @@ int mgwr_defect(mgwr_t h, int hierarchy, int level, double* norm_inf) {
   MGWR_TRY(with_hier(h, hierarchy, [&](auto& H) { return defect(h, H, level, h->norm_bits); }));
   std::vector<double> norms;
   MGWR_TRY(read_norms(h, norms));
+  MGWR_TRY(check_waits(h));
   if (norm_inf != nullptr) *norm_inf = max_norm(h, norms);
   return MGWR_OK;
 }
@@ -2629,7 +2632,7 @@ int mgwr_coarsest(mgwr_t h, int hierarchy) {
   MGWR_TRY(check_level(h, hierarchy, 0));
   MGWR_TRY(with_hier(h, hierarchy, [&](auto& H) { return coarsest(h, H); }));
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
-  return MGWR_OK;
+  return check_waits(h);
 }
 
 int mgwr_cycle(mgwr_t h, int hierarchy, int cyc, int nu1, int nu2) {

@@ -61,3 +61,21 @@ def test_marks_of_handles_on_several_threads():
     for s in handles:
         s.close()
     assert status == [G.MGWR_OK, G.MGWR_OK, G.MGWR_E_CUDA, G.MGWR_OK]
+
+
+# every call that runs a half-sweep, a one-point solve or a defect reports it
+@pytest.mark.parametrize("call", [
+    lambda s, l: s.residual(), lambda s, l: s.defect(G.MGWR_H64, l),
+    lambda s, l: s.coarsest(G.MGWR_H64), lambda s, l: s.smooth_defect(G.MGWR_H64, l),
+    lambda s, l: s.smooth(G.MGWR_H64, l, G.MGWR_RED), lambda s, l: s.smooth_restrict(G.MGWR_H64, l),
+    lambda s, l: s.cycle(G.MGWR_H64, 1, 1, 1)],
+    ids=["residual", "defect", "coarsest", "smooth_defect", "smooth", "smooth_restrict", "cycle"])
+def test_component_calls_report_a_mark(call):
+    with _solver(G.MGWR_FP64) as s:
+        l = s.num_levels() - 1
+        call(s, l)
+        s.inject_give_up()
+        with pytest.raises(G.MGWRError) as e:
+            call(s, l)
+        assert e.value.status == G.MGWR_E_CUDA
+        call(s, l)
