@@ -67,8 +67,9 @@ extern "C" {
 /* MGWR_FP64 computes in IEEE double, but for the half-sweeps of lines of 64 ..
  * 1024 steps: the line products run as exact integer products of eight-bit
  * slices on the tensor cores, rounded to double once (error about 1e-16 of a
- * line's scale, below that of an FP64 transform); a line whose right-hand side
- * holds an infinity or NaN becomes NaN.
+ * line's scale, below that of an FP64 transform).  A line whose right-hand side
+ * holds an infinity or NaN becomes NaN there; on levels of few lines, summed in
+ * IEEE double, it is not finite from that step on.
  * MGWR_MIXED keeps the finest iterate, the update and the stencil part of
  * every outer defect in IEEE double.  Its full outer defects take the time
  * convolution T_M u in double-float (FP32 instructions, error about 2^-44

@@ -148,7 +148,8 @@ cudaError_t launch_band_bf16x3(const double* kcol, unsigned char* band, int M, s
 // in FP64 (cols + b * cstride) and as its sliced band (band + b * bstride,
 // toep_band_bytes(M) bytes, written by launch_toep_band).  scratch holds
 // toep_scratch_bytes.  Waits give up after half a second.  A line with an
-// infinity or NaN in its gathered values becomes NaN.
+// infinity or NaN in its gathered values becomes NaN (FP64 sums: is not finite
+// from that step on).
 inline bool toep_length(int M) { return M >= 64 && M <= 1024; }
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
                               size_t cstride, const unsigned char* band, size_t bstride,

@@ -541,9 +541,11 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ double join(long long hi, long long lo, int shift, int e) {
   const long long v =
       (hi << (32 - shift)) + (shift > 8 ? ((lo >> (shift - 9)) + 1) >> 1 : lo << (8 - shift));
-  if (v == 0) return 0.0;
-  if (e <= -1000 || e >= 900)
+  if (e <= -1000 || e >= 900) {
+    // INT_MIN: an infinity or NaN in the line, whose finite values have no digits left
     return e == INT_MIN ? __longlong_as_double(0x7FF8000000000000ll) : scalbn((double)v, e);
+  }
+  if (v == 0) return 0.0;
   const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ull;
   const unsigned long long mag = (unsigned long long)(v < 0 ? -v : v);
   const int z = __clzll((long long)mag);

@@ -196,3 +196,28 @@ def test_sliced_products_repeat_their_bits(n, M):
         np.testing.assert_array_equal(r, seen[0][1])
     red = seen[0][0][1::2]
     np.testing.assert_array_equal(red, np.tile(red[0], (len(red), 1)))
+
+
+# a line with an infinity or NaN in it: NaN throughout where it is sliced, unchanged values before
+# that step and none finite from it on where it is summed
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("n,M", [(4095, 64), (511, 256), (127, 1024), (31, 64), (15, 1024)])
+def test_a_line_with_a_non_finite_value(n, M, bad):
+    f = inputs.random_field(n, M, 8)
+    hit, step = n // 2 | 1, M // 3
+    out = []
+    for g in (f, f.copy()):
+        if g is not f:
+            g[hit, step] = bad
+        with G.Solver(1, n, M, 1.0, 0.5) as s:
+            l = s.num_levels() - 1
+            s.field_set(G.MGWR_H64, l, G.MGWR_F, g)
+            s.field_set(G.MGWR_H64, l, G.MGWR_U, np.zeros_like(f))
+            s.smooth(G.MGWR_H64, l, G.MGWR_RED)
+            out.append(s.field_get(G.MGWR_H64, l, G.MGWR_U))
+    if _sums(n // 2, M):
+        np.testing.assert_array_equal(out[1][hit, :step], out[0][hit, :step])
+        assert not np.isfinite(out[1][hit, step:]).any()
+    else:
+        assert np.isnan(out[1][hit]).all()
+    np.testing.assert_array_equal(np.delete(out[1], hit, axis=0), np.delete(out[0], hit, axis=0))
