@@ -210,7 +210,9 @@ int mgwr_set_outer_switch(mgwr_t h, double rel);
  * M > 4096, where E is 1 or 2), synchronising with warp barriers when the
  * group fits in one warp.  A request a length cannot take falls back to the
  * nearest smaller E; mgwr_get_engine_split reports the E launches use.  The
- * FP64 half-sweeps of 64 .. 1024 steps have one form, whatever E is set.
+ * FP64 half-sweeps of 64 .. 1024 steps run the transform with the E that was
+ * set; where none was, they run as sliced products (MGWR_FP64), which have one
+ * launch shape and which mgwr_autotune goes back to.
  * MGWR_K_SWEEP32 that was neither set nor tuned takes E = 1 or 2, by the line
  * length and the lines of the launch.
  * For MGWR_K_SWEEP32 (not the one-point solve) with 64 <= M <= 4096, `split`
@@ -538,6 +540,9 @@ int mgwr_server_stats(mgwr_server_t s, mgwr_server_info* info);
  * solve or component call of this handle that runs such kernels returns
  * MGWR_E_CUDA and clears the mark; other handles are not affected. */
 int mgwr_inject_give_up(mgwr_t h);
+/* The same for device memory: the next `allocations` of the handle fail as if
+ * the device had none left. */
+int mgwr_inject_nomem(mgwr_t h, int allocations);
 
 /* Number of CUDA kernel launches issued through the library so far
  * (process-wide; h may be NULL). */

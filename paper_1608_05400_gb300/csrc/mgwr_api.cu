@@ -104,7 +104,7 @@ struct mgwr_handle {
   unsigned char* toep_band = nullptr;
   unsigned char* toep_tband = nullptr;  // the same of the Toeplitz columns (FP64 defects)
   unsigned char* toep_scratch = nullptr;
-  bool toep_off = false;  // no memory for them
+  int refuse_allocs = 0;  // the next allocations to fail (mgwr_inject_nomem)
   double* c_dev = nullptr;      // batch
   Hier<double> h64;
   Hier<float> h32;
@@ -214,6 +214,10 @@ int fail(mgwr_t h, int code, const std::string& msg) {
 template <class P>
 int dev_alloc(mgwr_t h, P** p, size_t bytes) {
   void* q = nullptr;
+  if (h->refuse_allocs > 0) {
+    --h->refuse_allocs;
+    return fail(h, MGWR_E_NOMEM, "allocation refused (mgwr_inject_nomem)");
+  }
   cudaError_t e = cudaMallocAsync(&q, bytes < 16 ? 16 : bytes, h->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -373,9 +377,14 @@ int ensure_h32(mgwr_t h) {
 }
 
 // The sliced bands of the FP64 half-sweeps on the tensor cores and their
-// scratch (before any capture that runs them).
+// scratch (before any capture that runs them).  A handle without room for them runs
+// the transforms and tries again at its next call; one whose half-sweeps are all set
+// to a split of the transform (mgwr_set_engine_split) has no use for them.
 int ensure_toep(mgwr_t h) {
-  if (h->toep_band != nullptr || h->toep_off || !mgwr::toep_length(h->M)) return MGWR_OK;
+  if (h->toep_band != nullptr || !mgwr::toep_length(h->M)) return MGWR_OK;
+  bool any = false;
+  for (int l = 0; l < h->nlev; ++l) any = any || split_of(h, MGWR_K_SWEEP64, l) == 0;
+  if (!any) return MGWR_OK;
   const size_t lines = (size_t)h->B * h->nlev;
   unsigned char* part[3] = {};
   const size_t bytes[3] = {mgwr::toep_scratch_bytes(shape(h, h->nlev - 1)),
@@ -383,16 +392,15 @@ int ensure_toep(mgwr_t h) {
                            mgwr::toep_band_bytes(h->M) * lines};
   for (int k = 0; k < 3; ++k) {
     if (dev_alloc(h, &part[k], bytes[k]) == MGWR_OK) continue;
-    // no room: this handle keeps the transforms
     for (unsigned char* p : part) {
       if (p == nullptr) continue;
       cudaFreeAsync(p, h->stream);
       h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)p));
     }
     h->err.clear();
-    h->toep_off = true;
     return MGWR_OK;
   }
+  drop_graph(h);  // captured with the transforms
   MGWR_CK(h, mgwr::launch_toep_band(h->kcol, part[2], h->M, lines, h->stream));
   MGWR_CK(h, mgwr::launch_toep_band(h->r, part[1], h->M, (size_t)h->B, h->stream));
   h->toep_scratch = part[0];
@@ -496,13 +504,14 @@ int default_sweep32(const LevelShape& ls) {
 }
 
 // One colour half-sweep of level l >= 1 (parity par) of the fields f -> u with
-// launch shape E: the tensor-core form for FP32 lines of 64 .. 256 steps when E
-// carries kTensor, else the FFT engine.
+// launch shape E (0: neither set nor tuned): for FP64 lines of 64 .. 1024 steps and
+// E = 0 the sliced products, for FP32 lines of 64 .. 256 steps the tensor-core form
+// when E carries kTensor, else the FFT engine.
 template <class R>
 cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
                         const LevelShape& ls, int par, int E, bool zero_u = false) {
   if constexpr (std::is_same<R, double>::value) {
-    if (h->toep_band != nullptr) {
+    if (h->toep_band != nullptr && E == 0) {
       const size_t bb = mgwr::toep_band_bytes(h->M);
       return mgwr::launch_sweep_toep(f, u, delta, h->kcol + (size_t)l * h->M,
                                      (size_t)h->nlev * h->M, h->toep_band + (size_t)l * bb,
@@ -532,8 +541,8 @@ template <class R>
 int coarsest(mgwr_t h, Hier<R>& H) {
   const int pm = prof_begin(h, MGWR_K_COARSEST, (double)h->B);
   if constexpr (std::is_same<R, double>::value) {
-    if (h->toep_band != nullptr) {
-      MGWR_CK(h, level_sweep(h, H, 0, H.f[0], H.u[0], (R*)nullptr, shape(h, 0), 0, 1));
+    if (h->toep_band != nullptr && split_of(h, MGWR_K_SWEEP64, 0) == 0) {
+      MGWR_CK(h, level_sweep(h, H, 0, H.f[0], H.u[0], (R*)nullptr, shape(h, 0), 0, 0));
       prof_end(h, pm);
       H.rs[0] = R_STALE;
       H.uz[0] = 0;
@@ -1171,8 +1180,9 @@ int tune_hierarchy(mgwr_t h, Hier<R>& H, int cls_sweep, int cls_defect) {
     const LevelShape ls = tune_sample(h, l);
     st = ensure_field(h, &H.u[l], level_count(h, l));
     if (st == MGWR_OK) st = ensure_field(h, &H.f[l], level_count(h, l));
-    // FP64 sweeps on the tensor cores have one launch shape (so have their defects)
-    const bool fixed = std::is_same<R, double>::value && h->toep_band != nullptr;
+    // the sliced products have one launch shape; a recorded split would take later
+    // handles of this shape away from them
+    const bool fixed = std::is_same<R, double>::value && mgwr::toep_length(h->M);
     if (st == MGWR_OK && !fixed)
       st = tune_class(h, cls_sweep, l, sizeof(R) == 4 ? 4 : 8, [&](int E) {
         // one smoothing step as the cycle runs it: red, then black recording its changes
@@ -1187,7 +1197,7 @@ int tune_hierarchy(mgwr_t h, Hier<R>& H, int cls_sweep, int cls_defect) {
         if (e != cudaSuccess) return e;
         return level_sweep(h, H, l, H.f[l], out, dlt, ls, parity(h, MGWR_BLACK), E);
       });
-    if (st == MGWR_OK && !(fixed && mgwr::toep_defect(shape(h, l))))
+    if (st == MGWR_OK && !(fixed && h->toep_band != nullptr && mgwr::toep_defect(shape(h, l))))
       st = tune_class(h, cls_defect, l, sizeof(R) == 4 ? 4 : 8, [&](int E) {
         return mgwr::launch_defect<R, R>(H.u[l], H.f[l], out, H.tspec, (size_t)h->L, H.tw,
                                          H.zero, scratch_for<R>(h), ls, R(h->hinv2[l]), nullptr,
@@ -1648,6 +1658,7 @@ int mgwr_autotune(mgwr_t h) {
   if (h == nullptr) return MGWR_E_INVAL;
   MGWR_CK(h, cudaStreamSynchronize(h->stream));
   if (h->precision == MGWR_FP64) {
+    if (mgwr::toep_length(h->M)) h->split[MGWR_K_SWEEP64].clear();
     MGWR_TRY(ensure_toep(h));
     MGWR_TRY(tune_hierarchy(h, h->h64, MGWR_K_SWEEP64, MGWR_K_DEFECT64));
   } else if (h->precision == MGWR_DD) {
@@ -2736,6 +2747,12 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
       total += r512(8 * B * pts[0] * M) + r512(16 * B * L) + r512(16 * Lt);
   }
   *bytes = total;
+  return MGWR_OK;
+}
+
+int mgwr_inject_nomem(mgwr_t h, int allocations) {
+  if (h == nullptr || allocations < 0) return MGWR_E_INVAL;
+  h->refuse_allocs = allocations;
   return MGWR_OK;
 }
 

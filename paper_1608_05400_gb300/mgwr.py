@@ -125,6 +125,7 @@ _SIGS = {
     "mgwr_toeplitz_column": (C.c_int, [_h, _dp]),
     "mgwr_inverse_column": (C.c_int, [_h, C.c_int, _dp]),
     "mgwr_inject_give_up": (C.c_int, [_h]),
+    "mgwr_inject_nomem": (C.c_int, [_h, C.c_int]),
     "mgwr_launch_count": (C.c_int, [_h, C.POINTER(C.c_longlong)]),
     "mgwr_peak_probe": (C.c_int, [_dp, _dp]),
     "mgwr_inverse_column_noalloc": (C.c_int, [C.c_void_p, C.c_int, C.c_double, C.c_void_p, C.c_void_p]),
@@ -302,6 +303,10 @@ class Solver:
     def inject_give_up(self):
         """Mark the handle as if a bounded wait of one of its kernels had given up (for tests)."""
         self._check(self.lib.mgwr_inject_give_up(self.h), "mgwr_inject_give_up")
+
+    def inject_nomem(self, allocations: int):
+        """Let the handle's next `allocations` of device memory fail (for tests)."""
+        self._check(self.lib.mgwr_inject_nomem(self.h, allocations), "mgwr_inject_nomem")
 
     def set_engine_split(self, kernel_class: int, split: int, level: int = -1):
         """E for one level, or every level (level -1)."""

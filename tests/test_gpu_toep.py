@@ -221,3 +221,54 @@ def test_a_line_with_a_non_finite_value(n, M, bad):
     else:
         assert np.isnan(out[1][hit]).all()
     np.testing.assert_array_equal(np.delete(out[1], hit, axis=0), np.delete(out[0], hit, axis=0))
+
+
+SWEEP64 = G.KERNEL_CLASSES.index("sweep64")
+
+
+def _solved(s, f):
+    s.set_rhs(f)
+    st = s.solve(1, 1, 1, tol=1e-10, max_cycles=40)
+    return s.solution(), st.cycles
+
+
+# a split that was set runs the transform it names (half-sweeps, one-point solve, whole solves with
+# their zero starts, graphs and device loops), on one level or on all
+@pytest.mark.parametrize("d,n,M,batch", [(1, 63, 64, 1), (2, 15, 256, 3), (2, 31, 1024, 1)])
+def test_a_set_split_runs_the_transform(d, n, M, batch):
+    alphas = 0.45 if batch == 1 else list(np.linspace(0.15, 0.95, batch))
+    shape = (n ** d, M) if batch == 1 else (batch, n ** d, M)
+    f = np.random.default_rng(9).uniform(-1, 1, shape)
+    out = []
+    for split, level in ((None, 0), (1, -1), (2, -1), (1, 1)):
+        with G.Solver(d, n, M, 1.0, alphas) as s:
+            if split is not None:
+                s.set_engine_split(SWEEP64, split, level=level)
+            out.append(_solved(s, f)[0])
+    sliced, one, two, mixed = out
+    np.testing.assert_array_equal(one, two)  # E moves butterflies between threads only
+    scale = np.abs(sliced).max()
+    # each form solves to 1e-10 of the defect, which bounds the difference of the solutions
+    for u in (one, mixed):
+        assert not np.array_equal(u, sliced)
+        assert np.abs(u - sliced).max() <= 1e-9 * scale
+
+
+# without memory for the bands and digits a handle runs the transforms, and the sliced products as
+# soon as there is some
+def test_sliced_products_come_back_with_the_memory():
+    d, n, M = 2, 31, 256
+    f = inputs.random_field(n ** d, M, 10)
+    with G.Solver(d, n, M, 1.0, 0.5) as s:
+        sliced = _solved(s, f)
+    with G.Solver(d, n, M, 1.0, 0.5) as s:
+        s.set_engine_split(SWEEP64, 1)
+        transform = _solved(s, f)
+        s.inject_nomem(1)
+        s.autotune()  # no split is set any more
+        s.inject_nomem(1)
+        short = _solved(s, f)
+        again = _solved(s, f)
+    np.testing.assert_array_equal(short[0], transform[0])
+    np.testing.assert_array_equal(again[0], sliced[0])
+    assert not np.array_equal(sliced[0], transform[0])
