@@ -2699,6 +2699,20 @@ int mgwr_profile_read(mgwr_t h, int kernel_class, long long* launches, double* m
   return MGWR_OK;
 }
 
+}  // extern "C"
+
+size_t mgwr::toep_footprint(int d, int n, int M, int batch) {
+  if (!toep_length(M)) return 0;
+  auto r512 = [](size_t b) { return (b + 511) / 512 * 512; };
+  const size_t B = batch;
+  size_t nlev = 1;
+  for (int m = n; m > 1; m = (m - 1) / 2) ++nlev;
+  return r512(toep_band_bytes(M) * B * nlev) + r512(toep_band_bytes(M) * B) +
+         B * r512(toep_scratch_bytes(LevelShape{d, n, M, 1}));
+}
+
+extern "C" {
+
 int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes) {
   if (bytes == nullptr) return MGWR_E_INVAL;
   if ((d != 1 && d != 2) || n < 1 || !is_pow2((long long)n + 1) || !is_pow2(M) || M < 4 ||
@@ -2723,11 +2737,7 @@ int mgwr_footprint(int d, int n, int M, int batch, int precision, size_t* bytes)
   if (M > mgwr::kShortMaxM)  // partitioned-convolution scratch: all block spectra of the finest level
     total += r512(16 * B * ((pts[0] + 1) / 2) * L);
   if (precision == MGWR_FP64) {
-    // sliced bands and digits of the tensor-core sweeps; a batch's digits (at most one
-    // slab) counted as its instances', so that the footprint is linear in the batch
-    if (mgwr::toep_length(M))
-      total += r512(mgwr::toep_band_bytes(M) * B * nlev) + r512(mgwr::toep_band_bytes(M) * B) +
-               B * r512(mgwr::toep_scratch_bytes(LevelShape{d, n, M, 1}));
+    total += mgwr::toep_footprint(d, n, M, batch);
     for (size_t l = 0; l < nlev; ++l) total += (l + 1 < nlev ? 4 : 3) * r512(8 * B * pts[l] * M);
   } else if (precision == MGWR_DD) {
     total += 2 * r512(8 * B * pts[0] * M);  // FP64 finest iterate and right-hand side

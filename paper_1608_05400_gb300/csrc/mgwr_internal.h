@@ -168,6 +168,10 @@ size_t toep_band_bytes(int M);
 // Bytes of scratch the launches on a level of this shape need (bounded: larger
 // fields go through it in slabs).
 size_t toep_scratch_bytes(const LevelShape& ls);
+// The part of mgwr_footprint that the sliced bands and digits of an MGWR_FP64 handle
+// take; it runs the transforms without them.  A batch's digits (at most one slab) are
+// counted as its instances', so that the footprint is linear in the batch.
+size_t toep_footprint(int d, int n, int M, int batch);
 // blob + line * toep_band_bytes(M): the sliced band of column cols[line].
 cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, size_t lines,
                              cudaStream_t s);

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "../../include/mgwr.h"
+#include "mgwr_internal.h"
 
 namespace {
 
@@ -157,6 +158,7 @@ struct Ticket {
   HostBuf f, u;
   std::vector<double> g;
   size_t footprint = 0;
+  bool transforms = false;  // FP64 without the memory of the sliced products
   size_t N = 0;
   int state = 0;  // 0 queued, 1 running, 2 done
   mgwr_t h = nullptr;   // its handle while it runs
@@ -324,6 +326,7 @@ int prepare(mgwr_server* s, Ticket* t) {
     st = mgwr_create(q.d, q.n, q.M, q.T, q.alpha, &h);
     if (st == MGWR_OK && q.precision != MGWR_FP64) st = mgwr_set_precision(h, q.precision);
   }
+  if (st == MGWR_OK && t->transforms) st = mgwr_set_engine_split(h, MGWR_K_SWEEP64, -1, 1);
   if (st == MGWR_OK) st = mgwr_set_order(h, q.order);
   if (st == MGWR_OK) st = mgwr_set_rhs(h, t->f.data(), t->g.empty() ? nullptr : t->g.data());
   if (st != MGWR_OK && h != nullptr) {
@@ -517,6 +520,12 @@ int check_request(const mgwr_request* q) {
 int submit_ticket(mgwr_server* s, const mgwr_request* rq, double* lent, uint64_t* ticket) {
   size_t fp = 0;
   if (mgwr_footprint(rq->d, rq->n, rq->M, 1, rq->precision, &fp) != MGWR_OK) return MGWR_E_INVAL;
+  // a plain FP64 request that fits only without the sliced products runs the transforms
+  // (a server's budget is fixed, so every request of its shape does)
+  const size_t sliced =
+      rq->precision == MGWR_FP64 ? mgwr::toep_footprint(rq->d, rq->n, rq->M, 1) : 0;
+  const bool transforms = sliced > 0 && fp > s->budget && fp - sliced <= s->budget;
+  if (transforms) fp -= sliced;
   if (fp > s->budget) return MGWR_E_TOOBIG;
   auto t = std::unique_ptr<Ticket>(new (std::nothrow) Ticket);
   if (!t) return MGWR_E_NOMEM;
@@ -539,6 +548,7 @@ int submit_ticket(mgwr_server* s, const mgwr_request* rq, double* lent, uint64_t
   t->rq.f = nullptr;
   t->rq.g = nullptr;
   t->footprint = fp;
+  t->transforms = transforms;
   t->t_submit = Clock::now();
   {
     std::lock_guard<std::mutex> lk(s->mu);

@@ -180,3 +180,29 @@ def test_requests_in_flight_share_graph_launches_and_reuse_handles():
         u, st = _alone(d, n, M, a, f, p, 1e-10)
         np.testing.assert_array_equal(res.u, u)
         assert res.stats.cycles == st.cycles and res.stats.relres == st.relres
+
+
+# a plain FP64 request whose memory fits the budget only without the bands and digits of the sliced
+# products is served with the transforms; below that it is refused
+def test_fp64_requests_at_the_edge_of_the_budget_run_the_transforms():
+    d, n, M = 2, 63, 256
+    fp = G.footprint(d, n, M, 1, G.MGWR_FP64)
+    f = inputs.Problem(d, n, M, 1.0, 0.5, "t2").rhs()
+    with G.Solver(d, n, M, 1.0, 0.5) as s:
+        s.set_engine_split(G.KERNEL_CLASSES.index("sweep64"), 1)
+        s.set_rhs(f)
+        s.solve(1, 1, 1, tol=1e-10, max_cycles=100)
+        want = s.solution()
+    with G.Server(hbm_budget=fp - 1, slots=2) as srv:
+        for _ in range(2):
+            res = srv.poll(srv.submit(d, n, M, 1.0, 0.5, f, precision=G.MGWR_FP64, tol=1e-10),
+                           timeout_us=60_000_000)
+            assert res.status == G.MGWR_OK
+            np.testing.assert_array_equal(res.u, want)
+        assert srv.info()["peak_bytes"] <= fp - 1
+    # 16 bytes of digits a value of one colour and the bands
+    digits = 16 * ((n ** d + 1) // 2) * M
+    with G.Server(hbm_budget=fp - 2 * digits, slots=2) as srv:
+        with pytest.raises(G.MGWRError) as e:
+            srv.submit(d, n, M, 1.0, 0.5, f, precision=G.MGWR_FP64)
+        assert e.value.status == G.MGWR_E_TOOBIG
