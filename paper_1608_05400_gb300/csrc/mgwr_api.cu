@@ -2707,8 +2707,9 @@ size_t mgwr::toep_footprint(int d, int n, int M, int batch) {
   const size_t B = batch;
   size_t nlev = 1;
   for (int m = n; m > 1; m = (m - 1) / 2) ++nlev;
-  return r512(toep_band_bytes(M) * B * nlev) + r512(toep_band_bytes(M) * B) +
-         B * r512(toep_scratch_bytes(LevelShape{d, n, M, 1}));
+  const size_t bands = r512(toep_band_bytes(M) * B * nlev) + r512(toep_band_bytes(M) * B);
+  const size_t one = r512(toep_scratch_bytes(LevelShape{d, n, M, 1}));
+  return bands + std::min(B * one, r512(2 * toep_slab_bytes(M)));
 }
 
 extern "C" {

@@ -168,9 +168,12 @@ size_t toep_band_bytes(int M);
 // Bytes of scratch the launches on a level of this shape need (bounded: larger
 // fields go through it in slabs).
 size_t toep_scratch_bytes(const LevelShape& ls);
+// The most that is: one slab of lines of M steps.
+size_t toep_slab_bytes(int M);
 // The part of mgwr_footprint that the sliced bands and digits of an MGWR_FP64 handle
-// take; it runs the transforms without them.  A batch's digits (at most one slab) are
-// counted as its instances', so that the footprint is linear in the batch.
+// take; it runs the transforms without them.  A handle holds one slab of digits at
+// most; a batch's are counted as its instances' up to two slabs, so that the footprint
+// is linear in the batch while they are small beside its fields.
 size_t toep_footprint(int d, int n, int M, int batch);
 // blob + line * toep_band_bytes(M): the sliced band of column cols[line].
 cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, size_t lines,

@@ -1030,6 +1030,10 @@ cudaError_t launch_toep_band(const double* cols, unsigned char* blob, int M, siz
   return counted(cudaGetLastError());
 }
 
+size_t toep_slab_bytes(int M) {
+  return kSlabBytes / ((size_t)M * kLineValue) * ((size_t)M * kLineValue + sizeof(int));
+}
+
 size_t toep_scratch_bytes(const LevelShape& ls) {
   return slab_lines(ls.M, ls.d, ls.n, ls.batch) * ((size_t)ls.M * kLineValue + sizeof(int));
 }

@@ -207,3 +207,14 @@ def test_pipelined_transfer_calls_reject_a_null_handle(lib):
     assert lib.mgwr_take_rhs(None) == mgwr.MGWR_E_INVAL
     assert lib.mgwr_stage_solution(None, None) == mgwr.MGWR_E_INVAL
     assert lib.mgwr_wait_staged(None) == mgwr.MGWR_E_INVAL
+
+
+def test_footprint_of_a_batch_counts_two_slabs_of_digits_at_most(lib):
+    # sliced FP64 products hold one slab (256 MB) of digits whatever the batch: a large instance's
+    # own, a batch's not once per instance; the other precisions have none
+    from paper_1608_05400_gb300.mgwr import MGWR_FP64, MGWR_MIXED, footprint
+    slab = 256 << 20
+    one, many = footprint(2, 255, 1024, 1, MGWR_FP64), footprint(2, 255, 1024, 64, MGWR_FP64)
+    assert 64 * one - 63 * slab - 64 * (4 << 20) <= many <= 64 * one - 61 * slab
+    mixed = footprint(2, 255, 1024, 1, MGWR_MIXED), footprint(2, 255, 1024, 64, MGWR_MIXED)
+    assert abs(64 * mixed[0] - mixed[1]) < 64 * (3 << 20)
