@@ -99,8 +99,9 @@ struct mgwr_handle {
   double* dk = nullptr;         // batch * (M+1): d_0..d_M
   double* kcol = nullptr;       // batch * nlev * M inverse columns
   unsigned char* tc_band = nullptr;  // their Toeplitz bands in bf16 pieces (tensor-core sweeps)
-  // sliced bands of the inverse columns (FP64 half-sweeps on the tensor cores,
-  // lines of 64 .. 1024 steps) and the scratch of their digits
+  // FP64 half-sweeps of 64 .. 1024 steps as FP64 sums and sliced products: the bands
+  // of the inverse columns and the scratch of the digits, where a level has products
+  bool toep_on = false;
   unsigned char* toep_band = nullptr;
   unsigned char* toep_tband = nullptr;  // the same of the Toeplitz columns (FP64 defects)
   unsigned char* toep_scratch = nullptr;
@@ -376,15 +377,30 @@ int ensure_h32(mgwr_t h) {
   return MGWR_OK;
 }
 
+// Whether a level runs sliced products (its defect, or a colour's half-sweep).
+bool has_products(const std::vector<LevelShape>& levels) {
+  for (const LevelShape& ls : levels)
+    if (mgwr::toep_defect(ls) || mgwr::toep_form(ls, 0) == mgwr::kToepProduct ||
+        (ls.n > 1 && mgwr::toep_form(ls, 1) == mgwr::kToepProduct))
+      return true;
+  return false;
+}
+
 // The sliced bands of the FP64 half-sweeps on the tensor cores and their
 // scratch (before any capture that runs them).  A handle without room for them runs
 // the transforms and tries again at its next call; one whose half-sweeps are all set
 // to a split of the transform (mgwr_set_engine_split) has no use for them.
 int ensure_toep(mgwr_t h) {
-  if (h->toep_band != nullptr || !mgwr::toep_length(h->M)) return MGWR_OK;
+  if (h->toep_on || !mgwr::toep_length(h->M)) return MGWR_OK;
   bool any = false;
   for (int l = 0; l < h->nlev; ++l) any = any || split_of(h, MGWR_K_SWEEP64, l) == 0;
   if (!any) return MGWR_OK;
+  std::vector<LevelShape> levels;
+  for (int l = 0; l < h->nlev; ++l) levels.push_back(shape(h, l));
+  if (!has_products(levels)) {
+    h->toep_on = true;
+    return MGWR_OK;
+  }
   const size_t lines = (size_t)h->B * h->nlev;
   unsigned char* part[3] = {};
   const size_t bytes[3] = {mgwr::toep_scratch_bytes(shape(h, h->nlev - 1)),
@@ -406,6 +422,7 @@ int ensure_toep(mgwr_t h) {
   h->toep_scratch = part[0];
   h->toep_tband = part[1];
   h->toep_band = part[2];
+  h->toep_on = true;
   return MGWR_OK;
 }
 
@@ -511,10 +528,11 @@ template <class R>
 cudaError_t level_sweep(mgwr_t h, Hier<R>& H, int l, const R* f, R* u, R* delta,
                         const LevelShape& ls, int par, int E, bool zero_u = false) {
   if constexpr (std::is_same<R, double>::value) {
-    if (h->toep_band != nullptr && E == 0) {
+    if (h->toep_on && E == 0 && mgwr::toep_form(ls, par) != mgwr::kToepTransform) {
       const size_t bb = mgwr::toep_band_bytes(h->M);
+      const unsigned char* band = h->toep_band == nullptr ? nullptr : h->toep_band + (size_t)l * bb;
       return mgwr::launch_sweep_toep(f, u, delta, h->kcol + (size_t)l * h->M,
-                                     (size_t)h->nlev * h->M, h->toep_band + (size_t)l * bb,
+                                     (size_t)h->nlev * h->M, band,
                                      (size_t)h->nlev * bb, h->toep_scratch, ls, par, h->hinv2[l],
                                      gave_up(h), h->stream, zero_u);
     }
@@ -541,7 +559,7 @@ template <class R>
 int coarsest(mgwr_t h, Hier<R>& H) {
   const int pm = prof_begin(h, MGWR_K_COARSEST, (double)h->B);
   if constexpr (std::is_same<R, double>::value) {
-    if (h->toep_band != nullptr && split_of(h, MGWR_K_SWEEP64, 0) == 0) {
+    if (h->toep_on && split_of(h, MGWR_K_SWEEP64, 0) == 0) {
       MGWR_CK(h, level_sweep(h, H, 0, H.f[0], H.u[0], (R*)nullptr, shape(h, 0), 0, 0));
       prof_end(h, pm);
       H.rs[0] = R_STALE;
@@ -2703,10 +2721,11 @@ int mgwr_profile_read(mgwr_t h, int kernel_class, long long* launches, double* m
 
 size_t mgwr::toep_footprint(int d, int n, int M, int batch) {
   if (!toep_length(M)) return 0;
+  std::vector<LevelShape> levels;
+  for (int m = n; m >= 1; m = (m - 1) / 2) levels.push_back(LevelShape{d, m, M, batch});
+  if (!has_products(levels)) return 0;
   auto r512 = [](size_t b) { return (b + 511) / 512 * 512; };
-  const size_t B = batch;
-  size_t nlev = 1;
-  for (int m = n; m > 1; m = (m - 1) / 2) ++nlev;
+  const size_t B = batch, nlev = levels.size();
   const size_t bands = r512(toep_band_bytes(M) * B * nlev) + r512(toep_band_bytes(M) * B);
   const size_t one = r512(toep_scratch_bytes(LevelShape{d, n, M, 1}));
   return bands + std::min(B * one, r512(2 * toep_slab_bytes(M)));

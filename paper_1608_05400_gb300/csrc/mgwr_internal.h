@@ -151,6 +151,11 @@ cudaError_t launch_band_bf16x3(const double* kcol, unsigned char* band, int M, s
 // infinity or NaN in its gathered values becomes NaN (FP64 sums: is not finite
 // from that step on).
 inline bool toep_length(int M) { return M >= 64 && M <= 1024; }
+// The form of a half-sweep of colour par: sums and products by launch_sweep_toep
+// (sums need neither bands nor scratch); the transform (launch_sweep) is the
+// caller's.
+enum ToepForm { kToepSums, kToepProduct, kToepTransform };
+ToepForm toep_form(const LevelShape& ls, int par);
 cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const double* cols,
                               size_t cstride, const unsigned char* band, size_t bstride,
                               unsigned char* scratch, const LevelShape& ls, int par, double hinv2,
@@ -171,7 +176,7 @@ size_t toep_scratch_bytes(const LevelShape& ls);
 // The most that is: one slab of lines of M steps.
 size_t toep_slab_bytes(int M);
 // The part of mgwr_footprint that the sliced bands and digits of an MGWR_FP64 handle
-// take; it runs the transforms without them.  A handle holds one slab of digits at
+// take (0 where none of its levels has use for them); it runs the transforms without.  A handle holds one slab of digits at
 // most; a batch's are counted as its instances' up to two slabs, so that the footprint
 // is linear in the batch while they are small beside its fields.
 size_t toep_footprint(int d, int n, int M, int batch);

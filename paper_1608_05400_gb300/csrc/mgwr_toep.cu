@@ -937,6 +937,30 @@ bool few_lines(long long lines, int M) {
   return lines * M * M / 2 <= (1ll << 21) + (1ll << 13) * M;
 }
 
+// Groups of lines of a launch over all instances (an instance's last group is padded).
+long long line_groups(int npts, int batch, int M) {
+  const int NL = lines_per_group(M, npts, batch);
+  return (long long)((npts + NL - 1) / NL) * batch;
+}
+
+// Batches of few lines an instance and 512 or 1024 steps: the pair's groups are mostly
+// padding (every instance has a column of its own), the transform takes one block per
+// 1024 / M line pairs.  Measured, us, pair / transform: M = 1024, one line each of 64,
+// 512, 4096 instances 99 / 48, 559 / 167, 4460 / 1078; three lines 94 / 49, 536 / 296,
+// 4271 / 2224; five of 512 552 / 470; seven of 512 and 4096 535 / 586, 4276 / 4456;
+// M = 512, one to three lines of 64, 512, 4096 46 / 28, 195 / 160, 1325 / 1049; seven
+// of 512 195 / 280; M = 256 and below the pair throughout (one line of 512 84 / 131).
+bool transform_pays(int npts, int batch, int M) {
+  if (M < 512) return false;
+  const long long pairs = (npts + 1) / 2, per_block = 1024 / M;
+  const long long blocks = (pairs + per_block - 1) / per_block * batch;
+  // hundredths of us
+  const long long pair = 2000 + line_groups(npts, batch, M) * (M == 1024 ? 104 : 32);
+  const long long least = M == 1024 ? 4800 : 2700;
+  const long long transform = (M == 1024 ? 2000 : 1200) + 28 * blocks;
+  return pair > (transform > least ? transform : least);
+}
+
 // Steps per tile of the FP64 sums: the one whose rounds of blocks (one per SM) take
 // least, a block costing its tile's sums and about five steps' worth for the rest
 // (M = 512, tiles of 8, 16, 32: 4 lines 4.7, 5.6, 7.6 us; 8 lines 6.3, 5.7, 7.6;
@@ -1055,7 +1079,7 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
   G.bstride = bstride;
   G.zero_u = zero_u;
   const long long lines = (long long)npts * ls.batch;
-  if (few_lines(lines, ls.M)) {
+  if (toep_form(ls, par) == kToepSums) {
     G.per_inst = G.group0 = G.groups = 0;
 #define MGWR_DIRECT(OB)                                                                     \
   k_toep_direct<OB><<<dim3((unsigned)lines, ls.M / (2 * OB)), 256, 0, s>>>(f, u, delta, cols, \
@@ -1074,10 +1098,17 @@ cudaError_t launch_sweep_toep(const double* f, double* u, double* delta, const d
   return product(f, u, delta, band, scratch, G, ls.batch, hinv2, gave_up, s);
 }
 
+ToepForm toep_form(const LevelShape& ls, int par) {
+  const int npts = colour_count(ls.d, ls.n, par);
+  if (few_lines((long long)npts * ls.batch, ls.M)) return kToepSums;
+  return transform_pays(npts, ls.batch, ls.M) ? kToepTransform : kToepProduct;
+}
+
 // Few lines keep the transform's defect (one launch).
 bool toep_defect(const LevelShape& ls) {
-  const long long lines = (long long)(ls.d == 1 ? ls.n : ls.n * ls.n) * ls.batch;
-  return toep_length(ls.M) && lines * ls.M * ls.M / 2 > (1ll << 22);
+  const int npts = ls.d == 1 ? ls.n : ls.n * ls.n;
+  return toep_length(ls.M) && (long long)npts * ls.batch * ls.M * ls.M / 2 > (1ll << 22) &&
+         !transform_pays(npts, ls.batch, ls.M);
 }
 
 cudaError_t launch_defect_toep(const double* u, const double* f, double* r,

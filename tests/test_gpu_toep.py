@@ -272,3 +272,24 @@ def test_sliced_products_come_back_with_the_memory():
     np.testing.assert_array_equal(short[0], transform[0])
     np.testing.assert_array_equal(again[0], sliced[0])
     assert not np.array_equal(sliced[0], transform[0])
+
+
+# batches of few lines an instance, on both sides of the line to the transform (its rounding:
+# log2(2M) stages of a few half-ulps of the norms of k and b, 1e-12 of the largest S as for every
+# transform), every instance with a column of its own; and the one-point solve
+@pytest.mark.parametrize("d,n,M,batch", [(1, 3, 1024, 64), (1, 7, 1024, 64), (2, 3, 1024, 48),
+                                         (1, 7, 512, 64), (1, 15, 512, 64), (1, 3, 256, 96)])
+def test_batches_of_few_lines_an_instance(d, n, M, batch):
+    rng = np.random.default_rng(11)
+    N = n ** d
+    u, f = rng.uniform(-1, 1, (batch, N, M)), rng.uniform(-1, 1, (batch, N, M)) * (n + 1) ** 2
+    with G.Solver(d, n, M, 1.0, list(np.linspace(0.15, 0.95, batch))) as s:
+        _check(s, d, n, M, G.MGWR_RED, u, f, batch, (0.0, 1.0), 1e-12)
+        s.field_set(G.MGWR_H64, 0, G.MGWR_F, f[:, :1])
+        s.coarsest(G.MGWR_H64)
+        got, k = s.field_get(G.MGWR_H64, 0, G.MGWR_U), s.inverse_column(0)
+        for b in (0, batch - 1):
+            line, kq = f[b, 0].astype(Q), k[b].astype(Q)
+            want = np.array([np.dot(kq[:m + 1][::-1], line[:m + 1]) for m in range(M)])
+            scale = float(np.abs(kq).sum() * np.abs(line).max())
+            assert float(np.abs(got[b].reshape(M) - want).max()) <= 1e-12 * scale
