@@ -687,15 +687,17 @@ int mgwr_poll(mgwr_server_t s, uint64_t ticket, int timeout_us, double* u_out, m
   std::unique_lock<std::mutex> lk(s->mu);
   auto it = s->tickets.find(ticket);
   if (it == s->tickets.end()) return MGWR_E_INVAL;
-  Ticket* t = it->second.get();
-  if (t->state != 2) {
+  if (it->second->state != 2) {
     if (timeout_us <= 0) return MGWR_E_AGAIN;
-    const bool done = s->cv_done.wait_for(lk, std::chrono::microseconds(timeout_us),
-                                          [&] { return t->state == 2; });
-    if (!done) return MGWR_E_TIMEOUT;
-    it = s->tickets.find(ticket);  // others may have been added or taken meanwhile
+    // looked up at every wake: another call may take the ticket while this one waits
+    const bool over = s->cv_done.wait_for(lk, std::chrono::microseconds(timeout_us), [&] {
+      it = s->tickets.find(ticket);
+      return it == s->tickets.end() || it->second->state == 2;
+    });
+    if (!over) return MGWR_E_TIMEOUT;
     if (it == s->tickets.end()) return MGWR_E_INVAL;
   }
+  Ticket* t = it->second.get();
   if (res != nullptr) *res = t->res;
   // the ticket is this call's now: its solution is copied without holding up the server
   const std::unique_ptr<Ticket> own = std::move(it->second);

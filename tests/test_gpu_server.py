@@ -206,3 +206,21 @@ def test_fp64_requests_at_the_edge_of_the_budget_run_the_transforms():
         with pytest.raises(G.MGWRError) as e:
             srv.submit(d, n, M, 1.0, 0.5, f, precision=G.MGWR_FP64)
         assert e.value.status == G.MGWR_E_TOOBIG
+
+
+# several calls wait for one ticket: one takes the result, the others learn that it is gone
+def test_several_polls_of_one_ticket():
+    import threading
+    d, n, M = 2, 127, 512
+    f = inputs.Problem(d, n, M, 1.0, 0.5, "t2").rhs()
+    with G.Server(hbm_budget=8 << 30, slots=1) as srv:
+        for _ in range(3):
+            t = srv.submit(d, n, M, 1.0, 0.5, f, precision=G.MGWR_FP64, tol=1e-10)
+            status = []
+            waits = [threading.Thread(target=lambda: status.append(
+                srv.lib.mgwr_poll(srv.h, t, 60_000_000, None, None))) for _ in range(6)]
+            for w in waits:
+                w.start()
+            for w in waits:
+                w.join(timeout=90)
+            assert sorted(status) == sorted([G.MGWR_OK] + [G.MGWR_E_INVAL] * 5)
