@@ -730,7 +730,7 @@ void drop_graph(mgwr_fas* h) {
 }
 
 // enqueue_cycle as a graph replay, captured on first use; the launches themselves
-// where the stream cannot be captured.
+// where the stream cannot be captured or the graph not be made.
 cudaError_t replay_cycle(mgwr_fas* h, int nu1, int nu2, int gamma) {
   const long long key =
       (((long long)h->order * 4 + h->smoother) * 4 + gamma) * 1024 + nu1 * 32 + nu2;
@@ -751,7 +751,8 @@ cudaError_t replay_cycle(mgwr_fas* h, int nu1, int nu2, int gamma) {
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) {
       h->graph = nullptr;
-      return e;
+      cudaGetLastError();
+      return enqueue_cycle(h, nu1, nu2, gamma);
     }
     h->graph_key = key;
     h->graph_kernels = kernels;

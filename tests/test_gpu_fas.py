@@ -322,3 +322,19 @@ def test_whole_line_smoother_repeats_its_bits_beside_other_work(n, M):
     torch.cuda.synchronize()
     for o in out[1:]:
         np.testing.assert_array_equal(o, out[0])
+
+
+def test_solve_on_a_stream_that_cannot_be_captured():
+    # the device's legacy default stream refuses capture: the cycles run as launches
+    n, M = 63, 128
+    out = []
+    for stream in (None, 1):
+        with G.FAS(n, M, 1.0, 0.4, 1.0) as g:
+            g.set_order(G.MGWR_ORDER_TABLE)
+            g.set_stream(stream)
+            g.set_rhs(np.ones((n, M)))
+            st = g.solve(1, 0, 1, tol=1e-10, max_cycles=30)
+            out.append((g.solution(), st.cycles))
+            g.set_stream(None)
+    assert out[0][1] == out[1][1] and out[0][1] >= 3
+    np.testing.assert_array_equal(out[0][0], out[1][0])
