@@ -274,7 +274,7 @@ template <int C>
 __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(1024)
     k_fas_fixed_sums(double* __restrict__ u, const double* __restrict__ f,
                      const double* __restrict__ kcol, int n, int M, double hinv, double hinv2,
-                     double c, double sigma, int coef, int parity, int all_points, int max_it,
+                     double c, int coef, int parity, int all_points, int max_it,
                      int* __restrict__ status, unsigned long long* __restrict__ iterations) {
   namespace cg = cooperative_groups;
   extern __shared__ double sums_sm[];
@@ -590,7 +590,7 @@ cudaError_t launch_line(mgwr_fas* h, int l, int parity, int all_points) {
 #define MGWR_SUMS_LAUNCH(CC)                                                                      \
   mgwr::k_fas_fixed_sums<CC><<<(unsigned)(count * CC), (unsigned)M, smem, h->stream>>>(           \
       h->u[l], h->f[l], h->kcol + (size_t)l * M, n, (int)M, 1.0 / hl, 1.0 / (hl * hl), h->c,      \
-      h->sigma[l], h->coef, parity, all_points, kFixedMaxIt, st, h->flags + 2)
+      h->coef, parity, all_points, kFixedMaxIt, st, h->flags + 2)
       switch (C) {
         case 8: MGWR_SUMS_LAUNCH(8); break;
         case 4: MGWR_SUMS_LAUNCH(4); break;

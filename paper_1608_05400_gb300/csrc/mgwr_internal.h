@@ -242,7 +242,7 @@ cudaError_t launch_restrict(const R* r, R* fc, R* uc, const LevelShape& fine, cu
 // fc = full weighting of the defect after a red-black step, formed from the
 // black half-sweep's changes delta (as launch_defect_from_delta would write
 // it, red points of parity red_par) without storing it; uc = 0 when given.  Bitwise the
-// same fc as launch_defect_from_delta followed by launch_restrict.
+// same fc as launch_defect_from_delta followed by launch_restrict.  FP32 only.
 template <class R>
 cudaError_t launch_restrict_delta(const R* delta, R* fc, R* uc, const R* zero, const LevelShape& fine,
                                   int red_par, R hinv2, cudaStream_t s);

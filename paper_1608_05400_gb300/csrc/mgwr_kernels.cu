@@ -251,8 +251,6 @@ __global__ void __launch_bounds__(kLineBlock)
 // a * b rounded on its own (never fused into a following addition), as when
 // the product is stored and read back.
 __device__ __forceinline__ float mul_rounded(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rounded(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ dd mul_rounded(dd a, dd b) { return a * b; }
 
 // Full weighting of the defect that a complete red-black step leaves (the
 // defect from the black half-sweep's changes, see k_defect_from_delta) without
@@ -1250,13 +1248,13 @@ cudaError_t launch_round_cx(Cx<float>* dst, const Cx<double>* src, size_t count,
                                                    int, R, unsigned long long*, cudaStream_t); \
   template cudaError_t launch_restrict<R>(const R*, R*, R*, const LevelShape&, cudaStream_t);  \
   template cudaError_t launch_prolong<R>(R*, const R*, const LevelShape&, int, bool,         \
-                                         cudaStream_t);                                      \
-  template cudaError_t launch_restrict_delta<R>(const R*, R*, R*, const R*, const LevelShape&, \
-                                                int, R, cudaStream_t);
+                                         cudaStream_t);
 MGWR_INST_R(double)
 MGWR_INST_R(float)
 MGWR_INST_R(dd)
 #undef MGWR_INST_R
+template cudaError_t launch_restrict_delta<float>(const float*, float*, float*, const float*,
+                                                  const LevelShape&, int, float, cudaStream_t);
 template cudaError_t launch_restrict_changes<double>(const double*, double*, const double*,
                                                      const LevelShape&, int, double, cudaStream_t);
 template cudaError_t launch_restrict_changes<dd>(const dd*, dd*, const dd*, const LevelShape&, int,
