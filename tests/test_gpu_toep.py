@@ -293,3 +293,44 @@ def test_batches_of_few_lines_an_instance(d, n, M, batch):
             want = np.array([np.dot(kq[:m + 1][::-1], line[:m + 1]) for m in range(M)])
             scale = float(np.abs(kq).sum() * np.abs(line).max())
             assert float(np.abs(got[b].reshape(M) - want).max()) <= 1e-12 * scale
+
+
+# the defect with a sliced time term against extended sums.  Bound of a value, with S the largest
+# sum |T| |u| of its line and A = h^-2 sum over the neighbours (|u_p| + |u_q|): the product 4e-16 S;
+# the differences, at most three sums and the two subtractions from f one rounding each.
+@pytest.mark.parametrize("d,n,M,batch", [(2, 63, 64, 1), (1, 1023, 128, 1), (2, 15, 256, 3),
+                                         (1, 63, 512, 2), (1, 127, 1024, 1)])
+@pytest.mark.parametrize("data", ["random", "wide"])
+def test_sliced_defect_against_extended_sums(d, n, M, batch, data):
+    rng = np.random.default_rng(12)
+    N = n ** d
+    assert N * batch * M * M // 2 > 1 << 22
+    u, f = rng.uniform(-1, 1, (batch, N, M)), rng.uniform(-1, 1, (batch, N, M)) * (n + 1) ** 2
+    if data == "wide":
+        u, f = (x * 10.0 ** rng.uniform(-12, 0, (batch, N, M)) for x in (u, f))
+    shape = (N, M) if batch == 1 else (batch, N, M)
+    hinv2, eps = float((n + 1) ** 2), 2.0 ** -53
+    alphas = 0.45 if batch == 1 else list(np.linspace(0.15, 0.95, batch))
+    with G.Solver(d, n, M, 1.0, alphas) as s:
+        l = s.num_levels() - 1
+        s.field_set(G.MGWR_H64, l, G.MGWR_U, u.reshape(shape))
+        s.field_set(G.MGWR_H64, l, G.MGWR_F, f.reshape(shape))
+        norm = s.defect(G.MGWR_H64, l)
+        got = s.field_get(G.MGWR_H64, l, G.MGWR_R).reshape(batch, N, M)
+        r = s.toeplitz_column().reshape(batch, M)
+    assert norm == np.abs(got).max()
+    for b in range(batch):
+        rq = r[b].astype(Q)
+        for p in sorted({int(x * (N - 1)) for x in (0.0, 0.37, 0.5, 1.0)}):
+            i, j = (p, 0) if d == 1 else (p % n, p // n)
+            v = u[b, p].astype(Q)
+            lap, A = np.zeros(M, dtype=Q), np.zeros(M)
+            for ok, q in ((i > 0, p - 1), (i < n - 1, p + 1), (j > 0, p - n), (j < n - 1, p + n))[:2 * d]:
+                w = u[b, q].astype(Q) if ok else 0 * v
+                lap, A = lap + (v - w), A + hinv2 * np.abs(u[b, p]) + hinv2 * np.abs(w).astype(float)
+            y = np.array([np.dot(rq[:m + 1][::-1], v[:m + 1]) for m in range(M)])
+            S = max(np.dot(np.abs(r[b][:m + 1][::-1]), np.abs(u[b, p][:m + 1])) for m in range(M))
+            want = f[b, p].astype(Q) - y - Q(hinv2) * lap
+            bound = 4e-16 * S + eps * (2 * np.abs(f[b, p]) + 2 * S + 6 * A)
+            err = np.abs(got[b, p].astype(Q) - want).astype(float)
+            assert (err <= bound).all(), (b, p, float((err / bound).max()))
