@@ -97,17 +97,14 @@ SMS = 152
 FP32_LANES_PER_SM = 128
 # DRAM bytes (read + write) per smoothed line of the FP64 half-sweep as sliced products,
 # from an ncu capture of k_toep_gather (132.2 + 89.8 MB) and k_toep_mma (199.4 + 36.6 MB) on
-# 8064 lines of 1024 steps (profiles/k_toep_fp64_2d_127x127_M1024.md).
+# 8064 lines of 1024 steps.
 SWEEP64_DRAM_BYTES_PER_LINE_M1024 = 56800.0
-# DRAM bytes per line of further kernels from single-kernel ncu captures (see
-# profiles/), by kernel class and M
-# (k_defect<double, float>: 1059.1 MB read + 254.9 MB written for 16,129 lines of 4096,
-# profiles/k_defect_fp64_outer_2d_127x127_M4096.md; k_sweep_rp_res, the resident paired
-# sweep: 264.5 + 102.2 MB for 8065 red lines, 396.6 + 218.7 MB for 8064 black lines that
-# record their changes, weighted as a V(1,1) cycle runs them per level (two red, one
-# recording black, one plain black), profiles/k_sweep_rp_res_fp32_2d_127x127_M4096.md;
-# k_defect_update_rp: 793.7 + 737.1 MB for 16,129 lines of 4096,
-# profiles/k_defect_outer_forms_2d_127x127_M4096.md)
+# DRAM bytes per line of further kernels from single-kernel ncu captures, by kernel class
+# and M (k_defect<double, float>: 1059.1 MB read + 254.9 MB written for 16,129 lines of
+# 4096; k_sweep_rp_res, the resident paired sweep: 264.5 + 102.2 MB for 8065 red lines,
+# 396.6 + 218.7 MB for 8064 black lines that record their changes, weighted as a V(1,1)
+# cycle runs them per level (two red, one recording black, one plain black);
+# k_defect_update_rp: 793.7 + 737.1 MB for 16,129 lines of 4096)
 NCU_DRAM_BYTES_PER_LINE: dict = {"defect64": {4096: 81468.0}, "sweep32": {4096: 53174.0},
                                  "defect32": {4096: 94908.0}}
 
@@ -346,13 +343,16 @@ CLASS_KERNELS = {
 }
 
 
-def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
-    """Roofline of one kernel class from its summed event-timed launches: the
-    FP64 kernels against the FP64 ALU peak (GB300 runs FP64 at 1/64 of FP32) or,
-    where lines of 64 .. 1024 steps run as sliced products, against the tensor
-    peak; the FP32 and line kernels against HBM with the FP32-issue view beside."""
+def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict, precision: str) -> dict:
+    """Roofline of one kernel class of a solve in `precision` from its summed
+    event-timed launches: the FP64 transforms against the FP64 ALU peak (GB300 runs
+    FP64 at 1/64 of FP32); the FP32 and line kernels against HBM with the FP32-issue
+    view beside; the lines of 64 .. 1024 steps of an MGWR_FP64 solve, whose sliced
+    products skip slices that vanish and whose small levels are FP64 sums, against HBM
+    with the rate of the multiply-adds they stand for beside."""
     secs = p["ms"] * 1e-3
-    name, word, kind = CLASS_KERNELS.get(cls, (cls, 8, "line"))
+    # line kernels work on the fields of the cycles
+    name, word, kind = CLASS_KERNELS.get(cls, (cls, 8 if precision in ("fp64", "dd") else 4, "line"))
     long = M > 4096
     if long and kind != "line":
         name = f"k_long_forward+k_long_inverse ({name})"
@@ -363,11 +363,14 @@ def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
     # its line; a defect reads u and f and writes r (the FP64 outer defect of the
     # mixed form writes FP32); the carried outer defect reads the FP32 correction and
     # the double-float defect and writes it back and rounded (24 bytes per value);
-    # line kernels: three words per line value
+    # the interpolation reads a coarse value and corrects half of the fine ones (a
+    # smoothing step rewrites the others); other line kernels: three words per line value
     if cls == "defect32":
         bytes_per_line = 24 * M
     elif kind == "defect":
-        bytes_per_line = (2 * word + (4 if cls == "defect64" else word)) * M
+        bytes_per_line = (2 * word + (4 if cls == "defect64" and precision != "fp64" else word)) * M
+    elif cls == "prolong":
+        bytes_per_line = (1.0 + 0.5 ** d) * word * M
     else:
         bytes_per_line = 3 * word * M
     bytes_alg = p["lines"] * bytes_per_line
@@ -377,16 +380,14 @@ def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
            "avg_launch_ms": p["ms"] / max(p["launches"], 1),
            "lines_per_launch": p["lines"] / max(p["launches"], 1),
            "bytes_per_line": bytes_per_line, "flops_per_line": per_line}
-    if cls in ("sweep64", "defect64") and 64 <= M <= 1024:
-        # 36 products of 8-bit slices per multiply-add of the triangle, in blocks of 128
-        # steps, those of zero slices at far lags included
-        per_line = 36.0 * M * (M + 128)
-        achieved, peak = p["lines"] * per_line / secs / 1e12, float(pk.get("bf16_tflops", 1900.0))
-        out.update({"kernel": "k_toep_gather + k_toep_mma (k_toep_direct on levels of few lines)",
-                    "flops_per_line": per_line, "bound": "tensor", "achieved": achieved,
-                    "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                    "peak_source": "measured (MEASURED_PEAKS.json bf16_tflops)",
-                    "hbm_view": {"achieved_gbs": hbm, "peak_gbs": hbm_peak, "frac": hbm / hbm_peak}})
+    if cls in ("sweep64", "defect64") and 64 <= M <= 1024 and precision == "fp64":
+        per_line = float(M * (M + 1))  # multiply-adds of the triangle, two operations each
+        names = ("k_toep_gather + k_toep_mma, k_toep_direct on levels of few lines" if cls == "sweep64"
+                 else "k_toep_gather + k_toep_mma + k_defect_finish, k_defect<double> on small levels")
+        out.update({"kernel": names, "flops_per_line": per_line, "bound": "hbm", "achieved": hbm,
+                    "peak": hbm_peak, "unit": "GB/s", "frac": hbm / hbm_peak,
+                    "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)",
+                    "multiply_add_view": {"achieved_tflops": p["lines"] * per_line / secs / 1e12}})
     elif cls in ("sweep64", "defect64"):
         peak = fp64_peak_tflops(pk)
         achieved = flops / secs / 1e12
@@ -405,7 +406,7 @@ def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
                                       "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop "
                                                      "x max SM clock"}
     out["traffic"] = None
-    if cls == "sweep64" and M == 1024:
+    if cls == "sweep64" and M == 1024 and precision == "fp64":
         out["traffic"] = SWEEP64_DRAM_BYTES_PER_LINE_M1024 * out["lines_per_launch"]
         out["traffic_note"] = "ncu dram bytes per line x lines per launch"
     elif cls in NCU_DRAM_BYTES_PER_LINE and M in NCU_DRAM_BYTES_PER_LINE[cls]:
@@ -414,9 +415,9 @@ def kernel_roofline(cls: str, p: dict, d: int, M: int, pk: dict) -> dict:
     return out
 
 
-def roofline_from_profile(prof: dict, d: int, M: int, pk: dict) -> dict:
+def roofline_from_profile(prof: dict, d: int, M: int, pk: dict, precision: str) -> dict:
     dom = max(prof, key=lambda k: prof[k]["ms"])
-    return kernel_roofline(dom, prof[dom], d, M, pk)
+    return kernel_roofline(dom, prof[dom], d, M, pk, precision)
 
 
 def oracle_threads() -> int:
@@ -1079,13 +1080,13 @@ def main():
                        inner_cycles=main_arm["inner_cycles"]),
         "solve": main_arm["solve"],
         "gpu_launches": main_arm["gpu_launches"],
-        "roofline": roofline_from_profile(prof, d, Mw, pk),
+        "roofline": roofline_from_profile(prof, d, Mw, pk, main_arm["precision"]),
         "kernel_classes": prof,
         "clocks": main_arm["clocks"],
         "e2e": main_arm.get("e2e"),
     }
     if "sweep32" in prof and out["roofline"]["class"] != "sweep32":
-        out["roofline_sweep32"] = kernel_roofline("sweep32", prof["sweep32"], d, Mw, pk)
+        out["roofline_sweep32"] = kernel_roofline("sweep32", prof["sweep32"], d, Mw, pk, main_arm["precision"])
     # name the FP32 sweep by the engine the tuner chose for the finest level
     sp = (main_arm["engine_splits"] or {}).get("sweep32")
     if sp:
