@@ -190,7 +190,11 @@ __global__ void __launch_bounds__(kThreads, 2)
       const bool band_ok = ok;
       for (int ch = 0; ok && ch < kNumChunks; ++ch) {
         const int b = ch & 1;
-        if (!mbar_wait_bounded(&full[b], (unsigned)((ch >> 1) & 1))) {
+        // The chunks' products have different widths and overlap in the accumulator.  The
+        // PTX ISA orders two tcgen05.mma only where accumulator and shape are the same, so
+        // a chunk's are issued when the last chunk's have completed.
+        if (!mbar_wait_bounded(&full[b], (unsigned)((ch >> 1) & 1)) ||
+            (ch > 0 && !mbar_wait_bounded(&empty[b ^ 1], (unsigned)(((ch - 1) >> 1) & 1)))) {
           ok = false;
           break;
         }

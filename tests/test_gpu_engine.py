@@ -388,3 +388,24 @@ def test_peak_probe_measures_both_pipes():
     assert 0.05 < p["fp64_tflops"] <= 152 * 2 * 2 * 2.2e9 / 1e12
     assert 1.0 < p["fp32_tflops"] <= 152 * 128 * 2 * 2.2e9 / 1e12
     assert p["fp32_tflops"] > 8 * p["fp64_tflops"]
+
+
+@pytest.mark.parametrize("d,n,M", [(1, 1023, 64), (2, 63, 128), (2, 63, 256)])
+def test_tensor_sweep_repeats_its_bits(d, n, M):
+    # the chunks' products overlap in the accumulator: no sum is lost in any launch
+    N = n ** d
+    u = inputs.random_field(N, M, seed=5)
+    f = inputs.random_field(N, M, seed=6, scale=2.0 * d * (n + 1) ** 2)
+    with G.Solver(d, n, M, 1.0, 0.45) as s:
+        s.set_precision(G.MGWR_MIXED)
+        s.set_engine_split(K["sweep32"], 1 | G.MGWR_SPLIT_TENSOR)
+        l = s.num_levels() - 1
+        s.field_set(G.MGWR_H32, l, G.MGWR_F, f)
+        out = []
+        for _ in range(20):
+            s.field_set(G.MGWR_H32, l, G.MGWR_U, u)
+            s.smooth(G.MGWR_H32, l, G.MGWR_RED)
+            s.smooth(G.MGWR_H32, l, G.MGWR_BLACK)
+            out.append(s.field_get(G.MGWR_H32, l, G.MGWR_U))
+    for o in out[1:]:
+        np.testing.assert_array_equal(o, out[0])
