@@ -96,9 +96,9 @@ SMS = 152
 # FP32 lanes of a GB300 SM (4 partitions x 32)
 FP32_LANES_PER_SM = 128
 # DRAM bytes (read + write) per smoothed line of the FP64 half-sweep as sliced products,
-# from an ncu capture of k_toep_gather (132.2 + 89.8 MB) and k_toep_mma (199.4 + 36.6 MB) on
+# from an ncu capture of k_toep_gather (132.2 + 89.3 MB) and k_toep_mma (202.1 + 37.3 MB) on
 # 8064 lines of 1024 steps.
-SWEEP64_DRAM_BYTES_PER_LINE_M1024 = 56800.0
+SWEEP64_DRAM_BYTES_PER_LINE_M1024 = 57200.0
 # DRAM bytes per line of further kernels from single-kernel ncu captures, by kernel class
 # and M (k_defect<double, float>: 1059.1 MB read + 254.9 MB written for 16,129 lines of
 # 4096; k_sweep_rp_res, the resident paired sweep: 264.5 + 102.2 MB for 8065 red lines,

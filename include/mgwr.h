@@ -64,10 +64,12 @@ extern "C" {
 #define MGWR_MIXED_DD 2 /* FP32 V-cycles; defect + update in double-float    */
 #define MGWR_DD 3       /* refinement with double-float inner cycles         */
 #define MGWR_AUTO 4     /* MGWR_MIXED_DD or MGWR_DD by the grid (below)      */
-/* MGWR_FP64 computes in IEEE double, but for the half-sweeps of lines of 64 ..
- * 1024 steps: the line products run as exact integer products of eight-bit
- * slices on the tensor cores, rounded to double once (error about 1e-16 of a
- * line's scale, below that of an FP64 transform).  A line whose right-hand side
+/* MGWR_FP64 computes in IEEE double, but for the half-sweeps and the time term
+ * of the defects of lines of 64 .. 1024 steps: their line products run as exact
+ * integer products of eight-bit slices on the tensor cores, rounded to double
+ * once (error about 1e-16 of a line's scale, below that of an FP64 transform).
+ * Levels of few lines are summed in IEEE double; batches of few lines an
+ * instance keep the FP64 transform.  A line whose right-hand side
  * holds an infinity or NaN becomes NaN there; on levels of few lines, summed in
  * IEEE double, it is not finite from that step on.
  * MGWR_MIXED keeps the finest iterate, the update and the stencil part of

@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(kLineBlock)
 // walking a coarse row, five loads and nine operations per coarse value, where
 // the fine defects and their stencil take about 30 operations in two passes over
 // the field.  2-D 255 x 255, M = 1024, FP64 solve: defects and restrictions 20.4 ->
-// 12.0 ms, 6.5 of them the norms of the twelve convergence checks.  In 1-D: half the sum of the two changes beside a red coarse
-// point, or a quarter of [1 2 1] at a black one (both colour orders occur).
+// 12.0 ms.  In 1-D: half the sum of the two changes beside a red coarse point, or a
+// quarter of [1 2 1] at a black one (both colour orders occur).
 template <class R>
 __global__ void __launch_bounds__(kLineBlock)
     k_restrict_changes(const R* __restrict__ delta, R* __restrict__ fc, const R* __restrict__ zero,

@@ -51,14 +51,17 @@
 // accumulator is double-buffered (2 x 8 NL columns).  Every wait is bounded.
 //
 // Measured (2-D, finest half-sweep, alpha = 0.5; 255 x 255, M = 1024): FFT form
-// 4.8 ms; k_toep_gather 0.34 ms (0.22 ms of it FP64 sums at the pipe's rate) and
-// k_toep_mma 0.58 ms.  What k_toep_mma takes is folding (seven conversions a value and
-// segment at a quarter of the rate, tcgen05.ld latency) and the hand-overs of about
-// 18 chunks an item: without its MMAs it is a fifth faster.
+// 4.8 ms; k_toep_gather 0.27 ms (0.22 ms of it FP64 sums at the pipe's rate) and
+// k_toep_mma 0.74 ms, bound by its MMAs (tensor pipe 69 % of the active clocks, each
+// reading as many clocks of shared memory as it multiplies) and by folding (seven
+// conversions a value and segment at a quarter of the rate, tcgen05.ld latency).  With
+// MMAs of eight widths, which nothing keeps in order, it took 0.58 ms (63 %).  The ring's
+// depth does not bound it: 2, 3, 4 and 8 stages 284, 270, 270 and 271 us for gather and
+// products of 127 x 127 x 1024, 391, 378, 378, 381 us of 255 x 255 x 512.
 //
 // Where there are too few lines to fill the chip the product is a sum of FP64
 // products (k_toep_direct): one launch, 4.5 us for one line of 512 steps (FFT form
-// 26 us, the tensor-core pair 17 us).
+// 26 us, the tensor-core pair 21 us).
 #include <cuda_fp16.h>
 
 #include <climits>
@@ -849,7 +852,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Bytes of a slab's digits.  Both kernels are bound by arithmetic, so writing the digits
 // to HBM and reading them back costs nothing, while every slab leaves SMs idle at the
 // end of two launches: 255 x 255 x 1024 solves with slabs of 32, 64, 128, 256 and 600 MB
-// (the last: one slab) take 101, 87, 82.3, 79.2 and 78.8 ms.
+// (the last: one slab) took 101, 87, 82.3, 79.2 and 78.8 ms (products at 0.58 of the 0.74
+// ms a half-sweep they take now).
 constexpr size_t kSlabBytes = size_t(256) << 20;
 constexpr size_t kLineValue = 2 * kSlices;  // bytes of digits per value
 
@@ -928,11 +932,12 @@ cudaError_t slab_launch(const double* f, double* u, double* delta, const unsigne
 }
 
 // Few lines: the FP64 sums (about 4 us + 2 us a million multiply-adds) instead of
-// the tensor-core pair (11.6, 12.5, 14.3, 17.8 and 23.3 us at M = 64 .. 1024 for any
+// the tensor-core pair (14.0, 15.5, 17.3, 21.5 and 29.5 us at M = 64 .. 1024 for any
 // grid up to one item per SM, and a second launch).  Measured, sums against pair
-// without that launch: M = 64, 481 lines (1.0 M) 7.5 / 11.5 us; M = 256, 128 lines
-// (4.2 M) 14.0 / 14.3; M = 512, 32 lines (4.2 M) 12.5 / 17.8, 64 lines (8.4 M) 22.7 /
-// 17.8; M = 1024, 16 lines (8.4 M) 21.3 / 23.3, 32 lines 40 / 23.3.
+// without that launch: M = 64, 1023 lines (2.1 M) 11.8 / 14.0 us; M = 128, 255 lines
+// (2.1 M) 11.5 / 15.5; M = 256, 127 lines (4.2 M) 16.4 / 17.3; M = 512, 31 lines
+// (4.1 M) 13.2 / 21.4, 64 lines (8.4 M) 22.7 / 21.7; M = 1024, 15 lines (7.9 M) 22.1 /
+// 30.2, 32 lines 40 / 30.2.
 bool few_lines(long long lines, int M) {
   return lines * M * M / 2 <= (1ll << 21) + (1ll << 13) * M;
 }
